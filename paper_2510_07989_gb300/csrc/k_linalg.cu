@@ -9,6 +9,8 @@
 // column = one right-hand side component (u-part columns 0..B-1, v-part B..2B-1).
 #include <math.h>
 
+#include <algorithm>
+
 #include "mot_internal.h"
 
 namespace {
@@ -245,47 +247,67 @@ __global__ void __launch_bounds__(1024) k_cg(int N, int C, CsrV A, CsrV A2, cons
 }
 
 // ----------------------------------------------------------------- dense GEMM
-// Y[n][C] = A[n][n] X[n][C] (n = npad, multiple of 32), FP64.
-constexpr int GB_M = 64, GB_K = 32, GB_N = 32;
-__global__ void __launch_bounds__(256) k_gemm(int n, int K, int C, const double* __restrict__ A,
+// Y[n][C] = A[n][K] X[K][C] (K a multiple of 32), FP64, for C > 8. Bound by the
+// FP64 units (two multiply-adds per clock and SM), so what matters is that all
+// of them work: 64-row x TX-column tiles alone are a few dozen CTAs at the
+// sizes of the march (576 x 576 x 10: nine), so K is split over gridDim.z as
+// well and the splits are summed in a fixed order. TX = 16 for C <= 16 (a
+// masked lane of a warp costs what a live one does), else 32.
+constexpr int GB_M = 64, GB_K = 32;
+template <int TX>
+__global__ void __launch_bounds__(256) k_gemm(int n, int K, int C, int kchunk, const double* __restrict__ A,
                                               const double* __restrict__ X, double* __restrict__ Y) {
-    // rows n, contraction K (multiple of GB_K), A row-major with lda = K
+    constexpr int TY = 256 / TX, RPT = GB_M / TY;
     __shared__ double sa[GB_M][GB_K + 1];
-    __shared__ double sx[GB_K][GB_N];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-    const int row0 = blockIdx.x * GB_M, col0 = blockIdx.y * GB_N;
-    double acc[8];
+    __shared__ double sx[GB_K][TX];
+    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+    const int row0 = blockIdx.x * GB_M, col0 = blockIdx.y * TX;
+    const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
+    double acc[RPT];
 #pragma unroll
-    for (int i = 0; i < 8; i++) acc[i] = 0.0;
-    for (int k0 = 0; k0 < K; k0 += GB_K) {
+    for (int i = 0; i < RPT; i++) acc[i] = 0.0;
+    for (int k0 = kbeg; k0 < kend; k0 += GB_K) {
+#pragma unroll
         for (int e = threadIdx.x; e < GB_M * GB_K; e += 256) {
             const int r = e / GB_K, k = e - r * GB_K;
             sa[r][k] = (row0 + r < n) ? A[(size_t)(row0 + r) * K + k0 + k] : 0.0;
         }
-        for (int e = threadIdx.x; e < GB_K * GB_N; e += 256) {
-            const int k = e / GB_N, cc = e - k * GB_N;
+#pragma unroll
+        for (int e = threadIdx.x; e < GB_K * TX; e += 256) {
+            const int k = e / TX, cc = e - k * TX;
             sx[k][cc] = (col0 + cc < C) ? X[(size_t)(k0 + k) * C + col0 + cc] : 0.0;
         }
         __syncthreads();
-#pragma unroll 4
+#pragma unroll 8
         for (int k = 0; k < GB_K; k++) {
             const double xv = sx[k][tx];
 #pragma unroll
-            for (int i = 0; i < 8; i++) acc[i] = fma(sa[ty + 8 * i][k], xv, acc[i]);
+            for (int i = 0; i < RPT; i++) acc[i] = fma(sa[ty + TY * i][k], xv, acc[i]);
         }
         __syncthreads();
     }
     if (col0 + tx < C) {
+        double* out = Y + (size_t)blockIdx.z * n * C;
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            const int r = row0 + ty + 8 * i;
-            if (r < n) Y[(size_t)r * C + col0 + tx] = acc[i];
+        for (int i = 0; i < RPT; i++) {
+            const int r = row0 + ty + TY * i;
+            if (r < n) out[(size_t)r * C + col0 + tx] = acc[i];
         }
     }
 }
 
-// Y[n][C] = A[n][n] X[n][C] for C <= 8: one warp per row, lanes over the
-// contraction index (coalesced rows of A), warp-shuffle reduction.
+// Y = sum over the S splits of W, in order
+__global__ void k_split_sum(long long n, int S, const double* __restrict__ W, double* __restrict__ Y) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        double v = 0.0;
+        for (int z = 0; z < S; z++) v += W[(size_t)z * n + i];
+        Y[i] = v;
+    }
+}
+
+// Y[n][C] = A[n][K] X[K][C] for C <= 8: one warp per row, lanes over the
+// contraction index (coalesced rows of A), warp-shuffle reduction. Bound by
+// reading A (C <= 2) or the FP64 units.
 template <int CC>
 __global__ void __launch_bounds__(256) k_gemv_small(int n, int K, const double* __restrict__ A,
                                                     const double* __restrict__ X, double* __restrict__ Y) {
@@ -295,6 +317,7 @@ __global__ void __launch_bounds__(256) k_gemv_small(int n, int K, const double* 
 #pragma unroll
         for (int c = 0; c < CC; c++) acc[c] = 0.0;
         const double* a = A + (size_t)row * K;
+#pragma unroll 8
         for (int k = lane; k < K; k += 32) {
             const double av = a[k];
 #pragma unroll
@@ -779,18 +802,37 @@ void launch_gemm_rect(mot_handle* h, int M, int K, const double* A, const double
         switch (C) {
             case 1: k_gemv_small<1><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
             case 2: k_gemv_small<2><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
+            case 3: k_gemv_small<3><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
             case 4: k_gemv_small<4><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
+            case 5: k_gemv_small<5><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
             case 6: k_gemv_small<6><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
-            case 8: k_gemv_small<8><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
-            default: goto general;
+            case 7: k_gemv_small<7><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
+            default: k_gemv_small<8><<<g, 256, 0, s>>>(M, K, A, X, Y); break;
         }
         h->launches++;
         return;
     }
-general:
-    dim3 grid((M + GB_M - 1) / GB_M, (C + GB_N - 1) / GB_N);
-    k_gemm<<<grid, 256, 0, s>>>(M, K, C, A, X, Y);
+    const int tx = C <= 16 ? 16 : 32;
+    const int tiles = ((M + GB_M - 1) / GB_M) * ((C + tx - 1) / tx);
+    // about four CTAs per SM, each split at least two K blocks long
+    int nsm = 148;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    int S = std::max(1, std::min(4 * nsm / tiles, K / (2 * GB_K)));
+    const int kchunk = ((K + S - 1) / S + GB_K - 1) / GB_K * GB_K;
+    S = (K + kchunk - 1) / kchunk;
+    double* ws = S > 1 ? split_workspace(h, sizeof(double) * (size_t)S * M * C) : nullptr;
+    const bool split = ws != nullptr;
+    const dim3 grid((M + GB_M - 1) / GB_M, (C + tx - 1) / tx, split ? S : 1);
+    if (tx == 16)
+        k_gemm<16><<<grid, 256, 0, s>>>(M, K, C, split ? kchunk : K, A, X, split ? ws : Y);
+    else
+        k_gemm<32><<<grid, 256, 0, s>>>(M, K, C, split ? kchunk : K, A, X, split ? ws : Y);
     h->launches++;
+    if (split) {
+        const long long n = (long long)M * C;
+        k_split_sum<<<grid_for(n), 256, 0, s>>>(n, S, ws, Y);
+        h->launches++;
+    }
 }
 
 void launch_gemm(mot_handle* h, const double* A, const double* X, int C, double* Y, cudaStream_t s) {

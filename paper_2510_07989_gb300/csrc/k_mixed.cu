@@ -441,31 +441,35 @@ void launch_history_reduce(mot_handle* h, const TaskList& tl, int C2, double* ou
     h->launches++;
 }
 
+double* split_workspace(mot_handle* h, size_t bytes) {
+    if (bytes > h->sgws_bytes) {
+        if (h->d_sgws) {
+            cudaFree(h->d_sgws);
+            h->device_bytes -= (int64_t)h->sgws_bytes;
+        }
+        h->sgws_bytes = 0;
+        h->d_sgws = (double*)dalloc(h, bytes);
+        if (h->d_sgws) h->sgws_bytes = bytes;
+    }
+    return h->d_sgws;
+}
+
 void launch_sgemm_d(mot_handle* h, int M, int N, int K, const float* A, const float* X, double* Y, cudaStream_t s) {
     int nsm = 148;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
     const int tiles = ((M + SG_M - 1) / SG_M) * ((N + SG_N - 1) / SG_N);
     // K splits: about four CTAs per SM, each split a multiple of the FP64 flush length
     int S = std::max(1, std::min((4 * nsm + tiles - 1) / tiles, std::min(16, (K + SG_FLUSH - 1) / SG_FLUSH)));
-    const size_t need = (size_t)S * M * N * sizeof(double);
-    if (S > 1 && need > h->sgws_bytes) {
-        if (h->d_sgws) {
-            cudaFree(h->d_sgws);
-            h->device_bytes -= (int64_t)h->sgws_bytes;
-        }
-        h->sgws_bytes = 0;
-        h->d_sgws = (double*)dalloc(h, need);
-        if (h->d_sgws) h->sgws_bytes = need;
-    }
-    if (S > 1 && !h->d_sgws) S = 1;  // no workspace: one split
+    double* ws = S > 1 ? split_workspace(h, (size_t)S * M * N * sizeof(double)) : nullptr;
+    if (!ws) S = 1;  // no workspace: one split
     const int kchunk = ((K + S - 1) / S + SG_FLUSH - 1) / SG_FLUSH * SG_FLUSH;
     S = (K + kchunk - 1) / kchunk;
     dim3 grid((M + SG_M - 1) / SG_M, (N + SG_N - 1) / SG_N, S);
-    k_sgemm_d<<<grid, 256, 0, s>>>(M, N, K, kchunk, A, X, S > 1 ? h->d_sgws : Y);
+    k_sgemm_d<<<grid, 256, 0, s>>>(M, N, K, kchunk, A, X, S > 1 ? ws : Y);
     h->launches++;
     if (S > 1) {
         const size_t n = (size_t)M * N;
-        k_sgemm_reduce<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256, 0, s>>>(n, S, h->d_sgws, Y);
+        k_sgemm_reduce<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256, 0, s>>>(n, S, ws, Y);
         h->launches++;
     }
 }

@@ -311,7 +311,8 @@ void apply_q0_dense64(mot_handle* h, const double* v, double* out, cudaStream_t 
         launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Q0, v, h->B, out, s);
 }
 
-// out = Q_0 v: dense Q_0 (mixed path, FP32 or FP64 copy) or the FP64 product form
+// out = Q_0 v: dense Q_0 (mixed path: emulated, FP32 or FP64; FP64 path: the FP64
+// matrix formed at load), or the FP64 product form
 void apply_q0(mot_handle* h, const Work& W, const double* v, double* out, cudaStream_t s) {
     const int n = h->npad * 2 * h->B;
     const size_t bv = (size_t)n;
@@ -341,6 +342,10 @@ void apply_q0(mot_handle* h, const Work& W, const double* v, double* out, cudaSt
     if (h->prec_active && h->d_Minv64) {  // FP64 right preconditioning: Q_0 (M v), M = Q_0^{-1} in FP64
         launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Minv64, v, h->B, W.q1, s);
         v = W.q1;  // consumed before left_factor reuses W.q1
+    }
+    if (h->d_Q0 && !h->precomputing) {  // FP64 dense Q_0 formed at load
+        launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Q0, v, h->B, out, s);
+        return;
     }
     project_sigma(h, W, v, W.sig, s);
     launch_axpby(h, n, 1.0, v, -1.0, W.sig, W.ell, s);
@@ -1455,42 +1460,74 @@ int precompute_mixed(mot_handle* h) {
     return MOT_OK;
 }
 
-// FP64 path with fp64_precond: Q_0^{-1} in FP64 as the right preconditioner of
-// GMRES. Q_0 is assembled column by column from the FP64 product form (64 unit
-// columns per batch), factorised by LU with partial pivoting and inverted; the
-// padded rows carry the identity.
-int precompute_fp64_precond(mot_handle* h) {
+// FP64 path set-up: dense Q_0, assembled column by column from the FP64
+// product form (64 unit columns per batch) and applied by every GMRES iteration
+// of the march; with fp64_precond also Q_0^{-1} (LU with partial pivoting, the
+// padded rows carry the identity), the right preconditioner.
+// The product form costs a step of the march, per GMRES iteration, a lag-0
+// contraction, two products with T_0 and five CG solves; its two T_0 products
+// alone are as many multiplications as one product with the dense Q_0
+// (4 npad^2 B each), so the dense form is taken whenever it can be formed. It
+// cannot when the memory is not there or a CG solve runs into its limit while
+// assembling: the march then applies the product form (with fp64_precond the
+// load fails as it needs Q_0 itself).
+int precompute_fp64(mot_handle* h) {
     const int Bp = 64;
-    h->precomputing = true;
-    int st = ensure_state(h, Bp);
-    if (st != MOT_OK) return st;
-    Work W = work_of(h);
+    const bool need = h->opt.fp64_precond != 0;
     cudaStream_t s = 0;
     const long long n2 = 2LL * h->npad;
-    double* q0 = (double*)dalloc(h, sizeof(double) * (size_t)n2 * n2);
-    int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(n2 + 1));
-    h->d_Minv64 = (double*)dalloc(h, sizeof(double) * (size_t)n2 * n2);
-    if (!q0 || !piv || !h->d_Minv64) return fail(h, MOT_EOOM, "device allocation (FP64 Q_0 factorisation)");
+    const size_t qbytes = sizeof(double) * (size_t)n2 * n2;
+    const int64_t held = h->device_bytes;  // without the assembly's temporary march state
+    h->precomputing = true;
+    int st = ensure_state(h, Bp);
+    double* q0 = st == MOT_OK ? (double*)dalloc(h, qbytes) : nullptr;
+    if (!q0) {
+        free_state(h);
+        h->precomputing = false;
+        h->device_bytes = held;
+        if (need) return st != MOT_OK ? st : fail(h, MOT_EOOM, "device allocation (FP64 Q_0)");
+        h->err.clear();
+        return MOT_OK;
+    }
+    Work W = work_of(h);
     CK(cudaMemsetAsync(h->d_cg_iters, 0, 2 * sizeof(int), s));
     for (long long J0 = 0; J0 < n2; J0 += Bp) {
         launch_unit_cols(h, J0, n2, W.x, s);
         apply_q0(h, W, W.x, W.w, s);
         launch_scatter_cols(h, J0, n2, W.w, q0, n2, s);
     }
-    dense_pad_identity(h, (int)n2, h->ne, q0, s);
-    const int bad = dense_lu(h, (int)n2, q0, piv, piv + n2, s);
-    if (bad == 0) dense_inverse_from_lu(h, (int)n2, q0, piv, h->d_Minv64, s);
     CK(cudaGetLastError());
     CK(cudaDeviceSynchronize());
     int it[2];
     CK(cudaMemcpy(it, h->d_cg_iters, 2 * sizeof(int), cudaMemcpyDeviceToHost));
-    cudaFree(q0);
-    cudaFree(piv);
-    h->device_bytes -= (int64_t)(sizeof(double) * (size_t)n2 * n2 + sizeof(int) * (size_t)(n2 + 1));
     free_state(h);
     h->precomputing = false;
+    h->device_bytes = held;
+    if (it[1] > 0) {
+        cudaFree(q0);
+        return need ? fail(h, MOT_ENOCONV, "a CG solve did not converge while assembling Q_0") : MOT_OK;
+    }
+    h->d_Q0 = q0;
+    h->device_bytes += (int64_t)qbytes;
+    if (!need) return MOT_OK;
+    double* lu = (double*)dalloc(h, qbytes);
+    int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(n2 + 1));
+    h->d_Minv64 = (double*)dalloc(h, qbytes);
+    if (!lu || !piv || !h->d_Minv64) {
+        if (lu) cudaFree(lu);
+        if (piv) cudaFree(piv);
+        return fail(h, MOT_EOOM, "device allocation (FP64 Q_0 factorisation)");
+    }
+    CK(cudaMemcpyAsync(lu, q0, qbytes, cudaMemcpyDeviceToDevice, s));
+    dense_pad_identity(h, (int)n2, h->ne, lu, s);
+    const int bad = dense_lu(h, (int)n2, lu, piv, piv + n2, s);
+    if (bad == 0) dense_inverse_from_lu(h, (int)n2, lu, piv, h->d_Minv64, s);
+    CK(cudaGetLastError());
+    CK(cudaDeviceSynchronize());
+    cudaFree(lu);
+    cudaFree(piv);
+    h->device_bytes -= (int64_t)(qbytes + sizeof(int) * (size_t)(n2 + 1));
     if (bad > 0) return fail(h, MOT_EINVAL, "Q_0 is singular to working precision (LU pivot breakdown)");
-    if (it[1] > 0) return fail(h, MOT_ENOCONV, "a CG solve did not converge while assembling Q_0");
     return MOT_OK;
 }
 
@@ -1617,8 +1654,7 @@ MOT_API int mot_load_operators(mot_handle* h, const mot_operators* ops) {
     h->tc_bulk = h->opt.precision == MOT_PREC_MIXED && mflag(h, MOT_MIX_TC) && mflag(h, MOT_MIX_TCBULK);
     if ((st = build_tiles(h, ops)) != MOT_OK) return st;
     if (h->opt.precision == MOT_PREC_MIXED && (st = precompute_mixed(h)) != MOT_OK) return st;
-    if (h->opt.precision == MOT_PREC_FP64 && h->opt.fp64_precond && (st = precompute_fp64_precond(h)) != MOT_OK)
-        return st;
+    if (h->opt.precision == MOT_PREC_FP64 && (st = precompute_fp64(h)) != MOT_OK) return st;
     h->loaded = true;
     return MOT_OK;
 }

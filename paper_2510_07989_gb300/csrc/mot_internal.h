@@ -194,7 +194,7 @@ struct mot_handle {
     double* d_LF = nullptr;        // dense [M1 | M2], npad x 2 npad, FP64
     float* d_LFf = nullptr;        // FP32 copy
     float* d_xf = nullptr;         // FP32 staging: [2 bv]
-    double* d_sgws = nullptr;      // split-K partial results of the FP32 dense products
+    double* d_sgws = nullptr;      // split-K partial results of the dense products
     size_t sgws_bytes = 0;
     EmuMat emu_Q0, emu_LF;         // Q_0 and [M1 | M2] for the emulated FP64 products (MOT_MIX_EMU64)
     EmuMat emu_Q0s, emu_Minv;      // Q_0 and Q_0^{-1} with 4 slices: the products of the FP32 solves
@@ -243,6 +243,9 @@ inline void once_per_device(std::atomic<unsigned long long>& done, int dev, F&& 
 }
 int cuda_fail(mot_handle* h, cudaError_t e, const char* where);
 void* dalloc(mot_handle* h, size_t bytes);
+
+// workspace of the split-K products (grown on demand; null: no memory, take one split)
+double* split_workspace(mot_handle* h, size_t bytes);
 
 // history
 void launch_history(mot_handle* h, const TaskList& tl, const double* tiles, const double* ring, const double* win,

@@ -1,0 +1,46 @@
+"""FP64 march over the batch sizes at which its dense products and its history
+contraction change form: skinny products (B columns of Q_0, 2B and 4B columns
+of the left factor) by rows, in 16- and in 32-column tiles, whole and split,
+ragged last tiles; the history with whole tiles (B < 4) and by nonzero masks
+(warps inside one row, and across two). Against the product-form FP64 oracle
+within the 1e-10 of the FP64 path's other parity tests (the dense oracle's
+pseudo-inverse of Lambda^T Lambda keeps a rounding-sized singular value of this
+45-vertex mesh: its projector misses P^2 = P by 1e-4)."""
+import numpy as np
+import pytest
+
+from oracle import product as P
+from paper_2510_07989_gb300.inputs import meshes as MS
+from paper_2510_07989_gb300.inputs.assemble import assemble
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    from paper_2510_07989_gb300.build import build
+    build()
+    from paper_2510_07989_gb300 import mot
+    return mot
+
+
+@pytest.fixture(scope="module")
+def torus():
+    ops = assemble(MS.torus(1.0, 0.3, 9, 5), 4.0, 1.0, 0.3)  # 135 edges: ragged last row block
+    return ops, P.ProductSystem(ops)
+
+
+@pytest.mark.parametrize("kw", [{}, {"fp64_precond": 1}, {"fp64_direct": 1}], ids=["plain", "precond", "direct"])
+@pytest.mark.parametrize("B", [1, 2, 3, 5, 7, 8, 9, 15, 16, 17, 24, 33, 64])
+def test_fp64_march_over_batches(M, torus, B, kw):
+    if kw and B not in (3, 9, 33):
+        pytest.skip("the products' forms are those of the plain path")
+    ops, S = torus
+    exc = MS.fibonacci_batch(B, ops.dt, w_steps=20, t0_steps=20, r_obj=1.3)
+    n = 35
+    s = M.Solver(ops, **kw)
+    W = s.run(exc, n)
+    assert s.noconv == 0
+    for b in sorted({0, B - 1}):
+        ref = S.march(exc, n, b=b)
+        assert np.abs(W[:, b].reshape(n, -1) - ref).max() < 1e-10 * np.abs(ref).max()
