@@ -202,22 +202,6 @@ __global__ void __launch_bounds__(128) k_hist_f32_b128(const HistTask* __restric
     for (int e = tid; e < 2 * T * V2_C; e += 128) dst[e] = acc64[e];
 }
 
-__global__ void k_hist_reduce2(const int* __restrict__ chunk_ptr, const double* __restrict__ partial, int C2,
-                               double* __restrict__ s1, double* __restrict__ s2) {
-    const int rb = blockIdx.x;
-    const int nout = T * C2;
-    const int c0 = chunk_ptr[rb], c1 = chunk_ptr[rb + 1];
-    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-        double a = 0.0, b = 0.0;
-        for (int c = c0; c < c1; c++) {
-            a += partial[(size_t)c * 2 * nout + o];
-            b += partial[(size_t)c * 2 * nout + nout + o];
-        }
-        s1[(size_t)rb * nout + o] = a;
-        s2[(size_t)rb * nout + o] = b;
-    }
-}
-
 // Y[M][N] (double) = A[M][K] (float, row-major, lda = K) * X[K][N] (float).
 // 128 x 64 output tile per CTA, 8 x 4 outputs per thread; FP32 products summed
 // in FP32 over 128 consecutive k, then added into FP64 accumulators. K is split
@@ -433,12 +417,6 @@ void launch_history32(mot_handle* h, const TaskList& tl, const float* tiles, con
         h->launches++;
     }
     launch_history_reduce(h, tl, C2, out_s1, out_s2, s);
-}
-
-void launch_history_reduce(mot_handle* h, const TaskList& tl, int C2, double* out_s1, double* out_s2,
-                           cudaStream_t s) {
-    k_hist_reduce2<<<h->nrb, 256, 0, s>>>(tl.chunk_ptr, h->d_partial, C2, out_s1, out_s2);
-    h->launches++;
 }
 
 double* split_workspace(mot_handle* h, size_t bytes) {

@@ -1251,6 +1251,10 @@ int build_tiles(mot_handle* h, const mot_operators* ops) {
     }
     std::vector<double>().swap(buf);
     std::vector<float>().swap(buf32);
+    h->d_tmask = (uint32_t*)dalloc(h, sizeof(uint32_t) * T * (size_t)std::max<int64_t>(1, h->ntiles_fp64));
+    if (!h->d_tmask) return fail(h, MOT_EOOM, "device allocation (history tile masks)");
+    launch_tile_masks(h, h->ntiles_fp64, h->d_tiles, h->d_tmask, 0);
+    CK(cudaGetLastError());
     int64_t nz = 0;
     for (int64_t t = 0; t < nt; t++) nz += tnnz[t];
     h->tile_fill = nt ? (double)nz / ((double)nt * T * T) : 0.0;
@@ -1294,6 +1298,7 @@ int build_tiles(mot_handle* h, const mot_operators* ops) {
                 }
     int nsm = 148;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    auto tnnz_of = [&](const HistTask& t) { return (int64_t)tnnz[t.tile]; };  // FP64 path: tiles numbered as stored
     auto make_list = [&](std::vector<HistTask>& tasks, std::vector<int>& rbs, TaskList& tl) -> int {
         std::vector<int> order(tasks.size());
         std::iota(order.begin(), order.end(), 0);
@@ -1310,8 +1315,13 @@ int build_tiles(mot_handle* h, const mot_operators* ops) {
             sorted[i] = tasks[order[i]];
             srb[i] = rbs[order[i]];
         }
-        const size_t target_chunks = (size_t)4 * nsm;
-        const int ch = (int)std::max<size_t>(1, (sorted.size() + target_chunks - 1) / target_chunks);
+        // about 4 nsm chunks of equal weight: the nonzeros of a task's tile are
+        // what it multiplies (FP64; the FP32 kernels take whole tiles), plus a
+        // constant for its loads and barriers
+        auto weight = [&](const HistTask& t) { return mixed_tiles ? 1 : 64 + tnnz_of(t); };
+        int64_t total = 0;
+        for (const HistTask& t : sorted) total += weight(t);
+        const int64_t per_chunk = std::max<int64_t>(1, (total + 4 * nsm - 1) / (4 * nsm));
         std::vector<HistChunk> chunks;
         std::vector<int> cptr(nrb + 1, 0);
         size_t i = 0;
@@ -1319,7 +1329,7 @@ int build_tiles(mot_handle* h, const mot_operators* ops) {
             cptr[rb] = (int)chunks.size();
             while (i < sorted.size() && srb[i] == rb) {
                 size_t j = i;
-                while (j < sorted.size() && srb[j] == rb && (int)(j - i) < ch) j++;
+                for (int64_t w = 0; j < sorted.size() && srb[j] == rb && w < per_chunk; j++) w += weight(sorted[j]);
                 chunks.push_back(HistChunk{rb, (int)i, (int)(j - i)});
                 i = j;
             }
@@ -1453,9 +1463,11 @@ int precompute_mixed(mot_handle* h) {
     }
     if (h32) {  // the FP64 lag-0 tiles (the dense Q_0 assembly's input) are no longer read
         cudaFree(h->d_tiles);
-        h->device_bytes -=
-            (int64_t)(sizeof(double) * (size_t)std::max<int64_t>(1, h->ntiles_fp64) * MOT_TILE * MOT_TILE);
+        cudaFree(h->d_tmask);
+        h->device_bytes -= (int64_t)((sizeof(double) * MOT_TILE * MOT_TILE + sizeof(uint32_t) * MOT_TILE) *
+                                     (size_t)std::max<int64_t>(1, h->ntiles_fp64));
         h->d_tiles = nullptr;
+        h->d_tmask = nullptr;
     }
     return MOT_OK;
 }
@@ -2253,7 +2265,7 @@ MOT_API void mot_destroy(mot_handle* h) {
     void* ptrs[] = {h->d_edge_faces, h->d_edge_verts, h->d_face_edges, h->d_face_sgn, h->d_iperm, h->d_cg_iters,
                     h->vtx_edges.rowptr, h->vtx_edges.col, h->vtx_edges.val, h->Lf.rowptr, h->Lf.col, h->Lf.val,
                     h->Lv.rowptr, h->Lv.col, h->Lv.val, h->G.rowptr, h->G.col, h->G.val, h->Gt.rowptr,
-                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_x, h->d_rhs_wf, h->d_tiles,
+                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_x, h->d_rhs_wf, h->d_tiles, h->d_tmask,
                     h->hist.tasks, h->hist.chunks, h->hist.chunk_ptr, h->lag0.tasks, h->lag0.chunks,
                     h->lag0.chunk_ptr, h->d_omega, h->d_colidx, h->d_tiles32, h->d_Q0, h->d_Q0f, h->d_LF,
                     h->d_LFf, h->d_Minvf, h->d_Minv64, h->d_Lfinvf, h->hist_tc_list.packed, h->hist_tc_list.chunks,

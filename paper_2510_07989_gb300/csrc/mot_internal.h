@@ -105,6 +105,7 @@ struct mot_handle {
     // block-sparse history
     double* d_tiles = nullptr;     // FP64 tiles (mixed path: lag 0 only, compact numbering, until set-up ends)
     int64_t ntiles = 0;
+    uint32_t* d_tmask = nullptr;   // nonzero masks of the rows of d_tiles, [tile][32]
     int64_t ntiles_fp64 = 0;       // tiles held in FP64 (all; on the mixed path only those of lag 0)
     double tile_fill = 0;
     TaskList hist, lag0;
@@ -250,6 +251,9 @@ double* split_workspace(mot_handle* h, size_t bytes);
 // history
 void launch_history(mot_handle* h, const TaskList& tl, const double* tiles, const double* ring, const double* win,
                     const double* kry, int mode, long long step_i, double* out_s1, double* out_s2, cudaStream_t s);
+
+// nonzero masks of ntiles FP64 tiles (k_hist_f64)
+void launch_tile_masks(mot_handle* h, int64_t ntiles, const double* tiles, uint32_t* masks, cudaStream_t s);
 
 // tensor-core history (mixed path, B a multiple of 8): tiles from d_tiles16, panels from d_ring16/d_win16
 void launch_history_tc(mot_handle* h, const TaskList& tl, long long step_i, double* out_s1, double* out_s2,
