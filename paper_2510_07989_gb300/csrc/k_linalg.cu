@@ -2,8 +2,7 @@
 // products and FP64 CG solves behind the quasi-Helmholtz projectors
 // (paper Section IV-B), the Gram solve and the static preconditioner products
 // (Section III, Eq. (CP)), the right-hand side (Section V-C), current recovery
-// and running Fourier sums (Eq. (dis_jm)), and the batched GMRES pieces of the
-// Q_0 solve (Eq. (MOT)).
+// and running Fourier sums (Eq. (dis_jm)).
 //
 // Block vectors are row-major [rows][C]: row = edge (or face / vertex),
 // column = one right-hand side component (u-part columns 0..B-1, v-part B..2B-1).
@@ -446,66 +445,6 @@ __global__ void k_pack_w(int ne, int B, const int* __restrict__ iperm, const dou
     }
 }
 
-// ----------------------------------------------------------------- GMRES
-// System b of the batch uses columns b and B+b of a block vector.
-// partial[chunk][v][b] = sum over the chunk's rows of <V_v, w>_b
-constexpr int GM_ROWS = 256;
-__global__ void k_gm_dots(int npad, int B, const double* __restrict__ V, size_t vstride, int nvec,
-                          const double* __restrict__ w, double* __restrict__ partial) {
-    const int C2 = 2 * B;
-    const int v = blockIdx.y;
-    const int r0 = blockIdx.x * GM_ROWS;
-    const double* Vv = V + (size_t)v * vstride;
-    __shared__ double sred[256];
-    // thread layout: column b = tid % B, row sub = tid / B
-    const int b = threadIdx.x % B, rs = threadIdx.x / B, RS = blockDim.x / B;
-    double s = 0.0;
-    if (threadIdx.x < RS * B)
-        for (int r = r0 + rs; r < min(r0 + GM_ROWS, npad); r += RS) {
-            const size_t ix = (size_t)r * C2 + b;
-            s = fma(Vv[ix], w[ix], s);
-            s = fma(Vv[ix + B], w[ix + B], s);
-        }
-    sred[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x < B) {
-        double t = 0.0;
-        for (int k = 0; k < RS; k++) t += sred[k * B + threadIdx.x];
-        partial[((size_t)blockIdx.x * nvec + v) * B + threadIdx.x] = t;
-    }
-}
-
-__global__ void k_gm_dots_reduce(int nchunk, int nvec, int B, const double* __restrict__ partial,
-                                 double* __restrict__ out, int do_sqrt) {
-    for (int i = threadIdx.x; i < nvec * B; i += blockDim.x) {
-        double s = 0.0;
-        for (int c = 0; c < nchunk; c++) s += partial[(size_t)c * nvec * B + i];
-        out[i] = do_sqrt ? sqrt(s) : s;
-    }
-}
-
-// w[r][c] -= sum_v V_v[r][c] coef[v][b(c)]  (sign = -1) or x += V y (sign = +1)
-__global__ void k_gm_update(int npad, int B, const double* __restrict__ V, size_t vstride, int nvec,
-                            const double* __restrict__ coef, double sign, double* __restrict__ w) {
-    const int C2 = 2 * B;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npad * C2; i += gridDim.x * blockDim.x) {
-        const int c = i % C2, b = c % B;
-        double s = 0.0;
-        for (int v = 0; v < nvec; v++) s = fma(V[(size_t)v * vstride + i], coef[v * B + b], s);
-        w[i] += sign * s;
-    }
-}
-
-__global__ void k_gm_scale(int npad, int B, const double* __restrict__ w, const double* __restrict__ nrm,
-                           const int* __restrict__ active, double* __restrict__ v) {
-    const int C2 = 2 * B;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npad * C2; i += gridDim.x * blockDim.x) {
-        const int b = (i % C2) % B;
-        const double d = nrm[b];
-        v[i] = (active[b] && d > 0.0) ? w[i] / d : 0.0;
-    }
-}
-
 // Per wave b (the u and v columns b and B + b of a block vector): sc[b] =
 // 2^-e, 2^e the power of two at or below max |x| over both columns (1 when
 // x is zero). One CTA per wave.
@@ -534,75 +473,6 @@ __global__ void k_wave_apply(int npad, int B, const double* __restrict__ sc, int
         x[i] = inverse ? x[i] / f : x[i] * f;
     }
 }
-
-// gstate layout per system b: H[(m+1) x m], g[m+1], cs[m], sn[m]
-__global__ void k_gm_init(int B, int m, const double* __restrict__ beta, double* __restrict__ H,
-                          double* __restrict__ g, int* __restrict__ active, int* __restrict__ jend,
-                          double* __restrict__ bnorm, int first_cycle, double* __restrict__ resid) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    for (int i = 0; i <= m; i++) g[(size_t)b * (m + 1) + i] = 0.0;
-    g[(size_t)b * (m + 1)] = beta[b];
-    if (first_cycle) bnorm[b] = beta[b];
-    const double bn = bnorm[b];
-    active[b] = (beta[b] > 0.0 && bn > 0.0) ? 1 : 0;
-    jend[b] = 0;
-    if (resid) resid[b] = bn > 0.0 ? beta[b] / bn : 0.0;
-}
-
-__global__ void k_gm_arnoldi(int B, int m, int j, const double* __restrict__ hcol, const double* __restrict__ nrm,
-                             double* __restrict__ H, double* __restrict__ g, double* __restrict__ cs,
-                             double* __restrict__ sn, int* __restrict__ active, int* __restrict__ jend,
-                             const double* __restrict__ bnorm, double tol, double* __restrict__ resid) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    double* Hb = H + (size_t)b * (m + 1) * m;
-    double* gb = g + (size_t)b * (m + 1);
-    double* cb = cs + (size_t)b * m;
-    double* sb = sn + (size_t)b * m;
-    if (!active[b]) return;
-    for (int i = 0; i <= j; i++) Hb[i * m + j] = hcol[i * B + b];
-    Hb[(j + 1) * m + j] = nrm[b];
-    for (int i = 0; i < j; i++) {
-        const double a = Hb[i * m + j], c2 = Hb[(i + 1) * m + j];
-        Hb[i * m + j] = cb[i] * a + sb[i] * c2;
-        Hb[(i + 1) * m + j] = -sb[i] * a + cb[i] * c2;
-    }
-    const double a = Hb[j * m + j], c2 = Hb[(j + 1) * m + j];
-    const double d = hypot(a, c2);
-    double cc = 1.0, ss = 0.0;
-    if (d > 0.0) {
-        cc = a / d;
-        ss = c2 / d;
-    }
-    cb[j] = cc;
-    sb[j] = ss;
-    Hb[j * m + j] = d;
-    Hb[(j + 1) * m + j] = 0.0;
-    gb[j + 1] = -ss * gb[j];
-    gb[j] = cc * gb[j];
-    const double rr = fabs(gb[j + 1]) / bnorm[b];
-    resid[b] = rr;
-    jend[b] = j + 1;
-    if (rr <= tol || !(nrm[b] > 0.0)) active[b] = 0;
-}
-
-// y = H^{-1} g (upper triangular, size jend[b]) into y[i][b]
-__global__ void k_gm_backsolve(int B, int m, const double* __restrict__ H, const double* __restrict__ g,
-                               const int* __restrict__ jend, double* __restrict__ y) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const double* Hb = H + (size_t)b * (m + 1) * m;
-    const double* gb = g + (size_t)b * (m + 1);
-    const int n = jend[b];
-    for (int i = 0; i < m; i++) y[i * B + b] = 0.0;
-    for (int i = n - 1; i >= 0; i--) {
-        double s = gb[i];
-        for (int k = i + 1; k < n; k++) s -= Hb[i * m + k] * y[k * B + b];
-        y[i * B + b] = Hb[i * m + i] != 0.0 ? s / Hb[i * m + i] : 0.0;
-    }
-}
-
 
 // out[r][0..C) = a[r], out[r][C..2C) = b[r]
 __global__ void k_pack2(int n, int C, const double* __restrict__ a, const double* __restrict__ b,
@@ -866,34 +736,6 @@ void launch_pack_w(mot_handle* h, const double* x, double* out, cudaStream_t s) 
     h->launches++;
 }
 
-void launch_gm_dots(mot_handle* h, const double* V, int nvec, const double* w, double* out, cudaStream_t s) {
-    const int nchunk = (h->npad + GM_ROWS - 1) / GM_ROWS;
-    dim3 grid(nchunk, nvec);
-    k_gm_dots<<<grid, 256, 0, s>>>(h->npad, h->B, V, (size_t)h->npad * 2 * h->B, nvec, w, h->d_red);
-    k_gm_dots_reduce<<<1, 256, 0, s>>>(nchunk, nvec, h->B, h->d_red, out, 0);
-    h->launches += 2;
-}
-
-void launch_gm_norm(mot_handle* h, const double* w, double* out, cudaStream_t s) {
-    const int nchunk = (h->npad + GM_ROWS - 1) / GM_ROWS;
-    dim3 grid(nchunk, 1);
-    k_gm_dots<<<grid, 256, 0, s>>>(h->npad, h->B, w, 0, 1, w, h->d_red);
-    k_gm_dots_reduce<<<1, 256, 0, s>>>(nchunk, 1, h->B, h->d_red, out, 1);
-    h->launches += 2;
-}
-
-void launch_gm_update(mot_handle* h, const double* V, int nvec, const double* coef, double* w, cudaStream_t s) {
-    const long long n = (long long)h->npad * 2 * h->B;
-    k_gm_update<<<grid_for(n), 256, 0, s>>>(h->npad, h->B, V, (size_t)n, nvec, coef, -1.0, w);
-    h->launches++;
-}
-
-void launch_gm_scale(mot_handle* h, const double* w, const double* nrm, double* v, cudaStream_t s) {
-    const long long n = (long long)h->npad * 2 * h->B;
-    k_gm_scale<<<grid_for(n), 256, 0, s>>>(h->npad, h->B, w, nrm, h->d_gm_active, v);
-    h->launches++;
-}
-
 void launch_wave_scale(mot_handle* h, const double* x, double* sc, cudaStream_t s) {
     k_wave_scale<<<h->B, 256, 0, s>>>(h->npad, h->B, x, sc);
     h->launches++;
@@ -904,26 +746,6 @@ void launch_wave_apply(mot_handle* h, const double* sc, bool inverse, double* x,
     k_wave_apply<<<grid_for(n), 256, 0, s>>>(h->npad, h->B, sc, inverse ? 1 : 0, x);
     h->launches++;
 }
-
-void launch_gm_init(mot_handle* h, const double* beta, int first_cycle, cudaStream_t s) {
-    k_gm_init<<<1, 64, 0, s>>>(h->B, h->gm_m, beta, h->d_H, h->d_g, h->d_gm_active, h->d_gm_jend, h->d_gm_bnorm,
-                               first_cycle, h->d_resid);
-    h->launches++;
-}
-
-void launch_gm_arnoldi_finish(mot_handle* h, int j, const double* hcol, const double* nrm, cudaStream_t s) {
-    k_gm_arnoldi<<<1, 64, 0, s>>>(h->B, h->gm_m, j, hcol, nrm, h->d_H, h->d_g, h->d_cs, h->d_sn, h->d_gm_active,
-                                  h->d_gm_jend, h->d_gm_bnorm, h->gm_tol, h->d_resid);
-    h->launches++;
-}
-
-void launch_gm_solve_update(mot_handle* h, double* y, double* x, cudaStream_t s) {
-    k_gm_backsolve<<<1, 64, 0, s>>>(h->B, h->gm_m, h->d_H, h->d_g, h->d_gm_jend, y);
-    const long long n = (long long)h->npad * 2 * h->B;
-    k_gm_update<<<grid_for(n), 256, 0, s>>>(h->npad, h->B, h->d_V, (size_t)n, h->gm_m, y, 1.0, x);
-    h->launches += 2;
-}
-
 
 void launch_pack2(mot_handle* h, const double* a, const double* b, int C, double* out, cudaStream_t s) {
     k_pack2<<<grid_for((long long)h->npad * 2 * C), 256, 0, s>>>(h->npad, C, a, b, out);

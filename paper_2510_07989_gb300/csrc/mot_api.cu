@@ -168,7 +168,7 @@ struct Work {
     double *q1, *q2, *t1, *t2, *dd, *pd;
     double *fvec, *zvec;      // faces / vertices x 4B
     double *cgw;              // CG scratch 4 x maxN x 4B
-    double *hc1, *hc2, *hsum, *nrm, *beta, *ygm;
+    double *ygm;
 };
 
 Work work_of(mot_handle* h) {
@@ -211,11 +211,6 @@ Work work_of(mot_handle* h) {
     W.zvec = take((size_t)std::max(h->nf, h->nv) * 4 * h->B);
     W.cgw = take((size_t)4 * maxN * 4 * h->B);
     const size_t gm = (size_t)(h->gm_m + 1) * h->B;
-    W.hc1 = take(gm);
-    W.hc2 = take(gm);
-    W.hsum = take(gm);
-    W.nrm = take(h->B);
-    W.beta = take(h->B);
     W.ygm = take(gm);
     return W;
 }
@@ -233,11 +228,6 @@ size_t work_doubles(mot_handle* h) {
     add((size_t)std::max(h->nf, h->nv) * 4 * h->B);
     add((size_t)std::max(h->nf, h->nv) * 4 * h->B);
     add((size_t)4 * maxN * 4 * h->B);
-    add(gm);
-    add(gm);
-    add(gm);
-    add(h->B);
-    add(h->B);
     add(gm);
     return n;
 }
@@ -311,37 +301,40 @@ void apply_q0_dense64(mot_handle* h, const double* v, double* out, cudaStream_t 
         launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Q0, v, h->B, out, s);
 }
 
+// mv = M v, M the copy of Q_0^{-1} that preconditions GMRES (mixed: emulated
+// or FP32; FP64 path with fp64_precond: FP64)
+void apply_m(mot_handle* h, const double* v, double* mv, cudaStream_t s) {
+    if (!mixed(h)) {
+        launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Minv64, v, h->B, mv, s);
+    } else if (h->emu_Minv.a16) {
+        launch_emu_gemm(h, h->emu_Minv, v, h->B, mv, s);
+    } else {
+        launch_d2f(h, (size_t)h->npad * 2 * h->B, v, h->d_xf, s);
+        launch_sgemm_d(h, 2 * h->npad, h->B, 2 * h->npad, h->d_Minvf, h->d_xf, mv, s);
+    }
+}
+
 // out = Q_0 v: dense Q_0 (mixed path: emulated, FP32 or FP64; FP64 path: the FP64
-// matrix formed at load), or the FP64 product form
-void apply_q0(mot_handle* h, const Work& W, const double* v, double* out, cudaStream_t s) {
+// matrix formed at load), or the FP64 product form. With mv: mv = M v, out = Q_0 mv.
+void apply_q0(mot_handle* h, const Work& W, const double* v, double* out, cudaStream_t s, double* mv = nullptr) {
     const int n = h->npad * 2 * h->B;
     const size_t bv = (size_t)n;
+    if (mv) {
+        apply_m(h, v, mv, s);
+        v = mv;
+    }
     if (mixed(h)) {
-        const double* in = v;
-        if (h->prec_active) {  // right preconditioning: Q_0 (M v)
-            if (h->emu_Minv.a16) {
-                launch_emu_gemm(h, h->emu_Minv, v, h->B, W.q1, s);
-            } else {
-                launch_d2f(h, bv, v, h->d_xf, s);
-                launch_sgemm_d(h, 2 * h->npad, h->B, 2 * h->npad, h->d_Minvf, h->d_xf, W.q1, s);
-            }
-            in = W.q1;
-        }
         if (mflag(h, MOT_MIX_Q032)) {
             if (h->emu_Q0s.a16) {
-                launch_emu_gemm(h, h->emu_Q0s, in, h->B, out, s);
+                launch_emu_gemm(h, h->emu_Q0s, v, h->B, out, s);
             } else {
-                launch_d2f(h, bv, in, h->d_xf, s);
+                launch_d2f(h, bv, v, h->d_xf, s);
                 launch_sgemm_d(h, 2 * h->npad, h->B, 2 * h->npad, h->d_Q0f, h->d_xf, out, s);
             }
         } else {
-            apply_q0_dense64(h, in, out, s);
+            apply_q0_dense64(h, v, out, s);
         }
         return;
-    }
-    if (h->prec_active && h->d_Minv64) {  // FP64 right preconditioning: Q_0 (M v), M = Q_0^{-1} in FP64
-        launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Minv64, v, h->B, W.q1, s);
-        v = W.q1;  // consumed before left_factor reuses W.q1
     }
     if (h->d_Q0 && !h->precomputing) {  // FP64 dense Q_0 formed at load
         launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Q0, v, h->B, out, s);
@@ -355,90 +348,81 @@ void apply_q0(mot_handle* h, const Work& W, const double* v, double* out, cudaSt
     left_factor(h, W, W.y1, W.y2, out, s);
 }
 
-// GMRES on Q_0 x = b, started from the x passed in (x0 = 0 when have_x0 is
-// false); the relative tolerance always refers to |b|.
-int gmres(mot_handle* h, const Work& W, const double* b, double* x, bool have_x0, double tol, cudaStream_t s) {
-    const int B = h->B;
+enum { GM_MAIN = 0, GM_REFINE = 1 };
+
+// GMRES on Q_0 x = b to |residual| <= tol |b|. r0 null: from x = 0; else x holds
+// the initial guess and r0 = b - Q_0 x. prec: right preconditioned, Q_0 M z = b,
+// x = M z, with the vectors M V_j kept (MOT_GM_ZCAP of them) so that x is their
+// combination; a longer solve applies M once more to the combination of the V_j.
+// GM_REFINE: the largest |r0| / |b| of the batch is left in last_gmres_resid, and
+// nothing more is done when it is within gmres_tol already.
+//
+// The iterations are queued without waiting for their residuals up to the
+// number that the last solve of this kind took; then the host looks after each.
+// A system that has converged is not changed by later iterations, so the
+// solution and the reported counts do not depend on when the host looked.
+// b must not be W.r, W.w or (prec) W.q1, W.t1.
+int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double* r0, bool prec, double tol, int kind,
+          cudaStream_t s) {
+    const int B = h->B, m = h->gm_m, maxit = h->opt.gmres_maxit;
     const size_t bv = (size_t)h->npad * 2 * B;
-    const int m = h->gm_m;
-    h->gm_tol = tol;
-    launch_gm_norm(h, b, W.beta, s);
-    launch_gm_init(h, W.beta, 1, s);  // records |b| as the reference norm
-    if (have_x0) {
-        apply_q0(h, W, x, W.r, s);
-        launch_axpby(h, (int)bv, 1.0, b, -1.0, W.r, W.r, s);
-        launch_gm_norm(h, W.r, W.beta, s);
-        launch_gm_init(h, W.beta, 0, s);
-        launch_gm_scale(h, W.r, W.beta, h->d_V, s);
-    } else {
-        CK(cudaMemsetAsync(x, 0, sizeof(double) * bv, s));
-        launch_gm_scale(h, b, W.beta, h->d_V, s);
-    }
+    const double* res = h->h_gmstat;
+    const int* act = (const int*)(res + 2 * B);
+    const int* jen = act + B;
+    launch_gm_begin(h, b, true, r0 ? r0 : b, h->d_V, s);
     int total = 0;
-    bool converged = false;
-    std::vector<int> act(B);
-    for (int cycle = 0; !converged && total < h->opt.gmres_maxit; cycle++) {
+    bool converged = false, add = r0 != nullptr;
+    double start = 0;  // largest |r0| / |b|
+    auto look = [&]() -> int {
+        CK(cudaMemcpyAsync(h->h_gmstat, h->d_resid, sizeof(double) * 3 * B, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        converged = true;
+        for (int k = 0; k < B; k++) {
+            converged &= act[k] == 0;
+            start = std::max(start, res[B + k]);
+        }
+        return MOT_OK;
+    };
+    for (;;) {
         int jend = 0;
-        for (int j = 0; j < m && total < h->opt.gmres_maxit; j++) {
-            const double* Vj = h->d_V + (size_t)j * bv;
-            apply_q0(h, W, Vj, W.w, s);
-            launch_gm_dots(h, h->d_V, j + 1, W.w, W.hc1, s);
-            launch_gm_update(h, h->d_V, j + 1, W.hc1, W.w, s);
-            launch_gm_dots(h, h->d_V, j + 1, W.w, W.hc2, s);
-            launch_gm_update(h, h->d_V, j + 1, W.hc2, W.w, s);
-            launch_axpby(h, (j + 1) * B, 1.0, W.hc1, 1.0, W.hc2, W.hsum, s);
-            launch_gm_norm(h, W.w, W.nrm, s);
-            launch_gm_arnoldi_finish(h, j, W.hsum, W.nrm, s);
-            launch_gm_scale(h, W.w, W.nrm, h->d_V + (size_t)(j + 1) * bv, s);
-            CK(cudaMemcpyAsync(act.data(), h->d_gm_active, sizeof(int) * B, cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            total++;
+        for (int j = 0; j < m && total < maxit && !converged; j++) {
+            double* mv = !prec ? nullptr : j < MOT_GM_ZCAP ? h->d_Z + (size_t)j * bv : W.q1;
+            apply_q0(h, W, h->d_V + (size_t)j * bv, W.w, s, mv);
+            launch_gm_iter(h, j, W.w, tol, kind == GM_REFINE ? 1e-6 : 0.0, s);
             jend = j + 1;
-            bool any = false;
-            for (int k = 0; k < B; k++) any |= act[k] != 0;
-            if (!any) {
-                converged = true;
-                break;
+            total++;
+            if (total >= h->gm_pred[kind] || jend == m || total == maxit) {
+                const int st = look();
+                if (st != MOT_OK) return st;
+                if (kind == GM_REFINE && start <= h->opt.gmres_tol) {
+                    h->last_gmres_resid = start;
+                    return MOT_OK;
+                }
             }
         }
-        if (jend > 0) launch_gm_solve_update(h, W.ygm, x, s);
-        if (converged || total >= h->opt.gmres_maxit) break;
+        // iterations past the last system's end did nothing: not counted
+        int used = 1;
+        for (int k = 0; k < B; k++) used = std::max(used, std::min(jen[k], jend));
+        total -= jend - used;
+        if (prec && used > MOT_GM_ZCAP) {
+            launch_gm_finish(h, h->d_V, used, false, W.ygm, W.q1, s);
+            apply_m(h, W.q1, W.t1, s);
+            launch_axpby(h, (int)bv, 1.0, W.t1, add ? 1.0 : 0.0, add ? x : nullptr, x, s);
+        } else {
+            launch_gm_finish(h, prec ? h->d_Z : h->d_V, used, add, W.ygm, x, s);
+        }
+        add = true;
+        if (converged || total >= maxit) break;
         // restart from the true residual
         apply_q0(h, W, x, W.r, s);
         launch_axpby(h, (int)bv, 1.0, b, -1.0, W.r, W.r, s);
-        launch_gm_norm(h, W.r, W.beta, s);
-        launch_gm_init(h, W.beta, 0, s);
-        launch_gm_scale(h, W.r, W.beta, h->d_V, s);
+        launch_gm_begin(h, b, false, W.r, h->d_V, s);
     }
-    std::vector<double> res(B);
-    CK(cudaMemcpyAsync(res.data(), h->d_resid, sizeof(double) * B, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    h->gm_pred[kind] = std::max(1, std::min(total, m));
     h->last_gmres_iters = total;
-    h->last_gmres_resid = 0;
-    for (double r : res) h->last_gmres_resid = std::max(h->last_gmres_resid, r);
+    h->last_gmres_resid = kind == GM_REFINE ? start : 0.0;
+    for (int k = 0; k < B && kind == GM_MAIN; k++) h->last_gmres_resid = std::max(h->last_gmres_resid, res[k]);
     return converged ? MOT_OK : fail(h, MOT_ENOCONV, "GMRES reached its iteration limit");
-}
-
-// x solves Q_0 x = rhs by right-preconditioned GMRES: Q_0 M z = rhs, x = M z,
-// with M the FP32 copy of Q_0^{-1} (mixed path) or its FP64 form (FP64 path
-// with fp64_precond). z lives in a buffer that apply_q0 does not touch: W.pd
-// on the mixed path (dense Q_0), W.s1 on the FP64 path (its product-form Q_0
-// uses W.pd inside the left factor; the history sums in W.s1 are consumed
-// before the solve). rhs must not be W.r, W.q1 or that buffer.
-int prec_solve(mot_handle* h, const Work& W, const double* rhs, double* x, double tol, cudaStream_t s) {
-    double* z = mixed(h) ? W.pd : W.s1;
-    h->prec_active = true;
-    int st = gmres(h, W, rhs, z, false, tol, s);
-    h->prec_active = false;
-    if (!mixed(h)) {
-        launch_gemm_rect(h, 2 * h->npad, 2 * h->npad, h->d_Minv64, z, h->B, x, s);
-    } else if (h->emu_Minv.a16) {
-        launch_emu_gemm(h, h->emu_Minv, W.pd, h->B, x, s);
-    } else {
-        launch_d2f(h, (size_t)h->npad * 2 * h->B, W.pd, h->d_xf, s);
-        launch_sgemm_d(h, 2 * h->npad, h->B, 2 * h->npad, h->d_Minvf, h->d_xf, x, s);
-    }
-    return st;
 }
 
 int ensure_state(mot_handle* h, int B) {
@@ -499,16 +483,18 @@ int ensure_state(mot_handle* h, int B) {
     h->d_g = (double*)dalloc(h, sizeof(double) * (size_t)B * (h->gm_m + 1));
     h->d_cs = (double*)dalloc(h, sizeof(double) * (size_t)B * h->gm_m);
     h->d_sn = (double*)dalloc(h, sizeof(double) * (size_t)B * h->gm_m);
-    h->red_bytes = sizeof(double) * (size_t)((h->npad + 255) / 256 + 1) * (h->gm_m + 1) * B;
-    h->d_red = (double*)dalloc(h, h->red_bytes);
-    h->d_resid = (double*)dalloc(h, sizeof(double) * B);
-    h->d_gm_active = (int*)dalloc(h, sizeof(int) * B);
-    h->d_gm_jend = (int*)dalloc(h, sizeof(int) * B);
+    const bool prec = !h->precomputing && (h->d_Minvf || h->d_Minv64);
+    if (prec) {
+        h->d_Z = (double*)dalloc(h, sizeof(double) * MOT_GM_ZCAP * bv);
+        if (!h->d_Z) return fail(h, MOT_EOOM, "device allocation of the march state");
+    }
+    h->d_resid = (double*)dalloc(h, sizeof(double) * 3 * B);
+    h->d_gm_active = (int*)(h->d_resid + 2 * B);
+    h->d_gm_jend = h->d_gm_active + B;
     h->d_gm_bnorm = (double*)dalloc(h, sizeof(double) * B);
     h->d_wscale = (double*)dalloc(h, sizeof(double) * B);
     if (!h->d_waves || !h->d_ring || !h->d_win || !h->d_cur || !h->d_dft || !h->d_work || !h->d_partial ||
-        !h->d_V || !h->d_H || !h->d_g || !h->d_cs || !h->d_sn || !h->d_red || !h->d_resid || !h->d_gm_active ||
-        !h->d_gm_jend || !h->d_gm_bnorm || !h->d_wscale)
+        !h->d_V || !h->d_H || !h->d_g || !h->d_cs || !h->d_sn || !h->d_resid || !h->d_gm_bnorm || !h->d_wscale)
         return fail(h, MOT_EOOM, "device allocation of the march state");
     h->h_waves.assign(10 * B, NAN);
     return MOT_OK;
@@ -516,8 +502,7 @@ int ensure_state(mot_handle* h, int B) {
 
 void free_state(mot_handle* h) {
     void* ptrs[] = {h->d_waves, h->d_ring, h->d_win, h->d_cur, h->d_dft, h->d_work, h->d_partial, h->d_V, h->d_H,
-                    h->d_g, h->d_cs, h->d_sn, h->d_red, h->d_resid, h->d_gm_active, h->d_gm_jend, h->d_gm_bnorm,
-                    h->d_wscale,
+                    h->d_g, h->d_cs, h->d_sn, h->d_Z, h->d_resid, h->d_gm_bnorm, h->d_wscale,
                     h->d_wprev1, h->d_wprev2};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -531,7 +516,7 @@ void free_state(mot_handle* h) {
     h->hist_tc = false;
     h->d_pcg_work = h->d_pcg_scal = nullptr;
     h->d_waves = h->d_ring = h->d_win = h->d_cur = h->d_dft = h->d_work = h->d_partial = nullptr;
-    h->d_V = h->d_H = h->d_g = h->d_cs = h->d_sn = h->d_red = h->d_resid = nullptr;
+    h->d_V = h->d_H = h->d_g = h->d_cs = h->d_sn = h->d_Z = h->d_resid = nullptr;
     h->d_gm_active = h->d_gm_jend = nullptr;
     h->d_gm_bnorm = nullptr;
     h->d_wscale = nullptr;
@@ -560,8 +545,8 @@ int upload_waves(mot_handle* h, const mot_wave* waves, int B, cudaStream_t s) {
     }
     // the step's input is copied every step (B x 80 bytes)
     h->h_waves = v;
+    // (pageable memory: the values are taken before the call returns)
     CK(cudaMemcpyAsync(h->d_waves, h->h_waves.data(), sizeof(double) * 10 * B, cudaMemcpyHostToDevice, s));
-    CK(cudaStreamSynchronize(s));
     return MOT_OK;
 }
 
@@ -640,11 +625,13 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
         left_factor(h, W, W.y1, W.y2, W.b, s);
     }
     PEV(3);
-    // initial guess: linear extrapolation of the last two solutions
-    bool have_x0 = i >= 2;
-    if (i >= 3)
+    const bool refine = mx && mflag(h, MOT_MIX_REFINE);
+    const bool prec = (mx && h->d_Minvf) || (!mx && h->d_Minv64);
+    // unpreconditioned: initial guess by linear extrapolation of the last two solutions
+    const bool have_x0 = i >= 2 && !prec;
+    if (have_x0 && i >= 3)
         launch_axpby(h, n, 2.0, h->d_wprev1, -1.0, h->d_wprev2, W.x, s);
-    else if (i == 2)
+    else if (have_x0)
         launch_axpby(h, n, 1.0, h->d_wprev1, 0.0, nullptr, W.x, s);
     // every wave's system is solved at O(1) magnitude: b and the initial
     // guess scaled by a power of two (exact), the solution scaled back. Late
@@ -654,11 +641,13 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
     launch_wave_scale(h, W.b, h->d_wscale, s);
     launch_wave_apply(h, h->d_wscale, false, W.b, s);
     if (have_x0) launch_wave_apply(h, h->d_wscale, false, W.x, s);
-    const bool refine = mx && mflag(h, MOT_MIX_REFINE);
-    const bool prec = (mx && h->d_Minvf) || (!mx && h->d_Minv64);
     // with refinement the reduced-precision solves only need 1e-6: each sweep gains ~6 digits
     const double tol_in = refine ? std::max(h->opt.gmres_tol, 1e-6) : h->opt.gmres_tol;
-    int st = prec ? prec_solve(h, W, W.b, W.x, tol_in, s) : gmres(h, W, W.b, W.x, have_x0, tol_in, s);
+    if (have_x0) {
+        apply_q0(h, W, W.x, W.r, s);
+        launch_axpby(h, n, 1.0, W.b, -1.0, W.r, W.r, s);
+    }
+    int st = gmres(h, W, W.b, W.x, have_x0 ? W.r : nullptr, prec, tol_in, GM_MAIN, s);
     if (st != MOT_OK && st != MOT_ENOCONV) return st;
     PEV(4);
     h->refine_sweeps = 0;
@@ -671,22 +660,12 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
         for (int sweep = 0; sweep < max_sweeps; sweep++) {
             apply_q0_dense64(h, W.x, W.r, s);
             launch_axpby(h, n, 1.0, W.b, -1.0, W.r, W.r, s);
-            launch_gm_norm(h, W.r, W.nrm, s);
-            launch_gm_norm(h, W.b, W.beta, s);
-            std::vector<double> rn(h->B), bn(h->B);
-            CK(cudaMemcpyAsync(rn.data(), W.nrm, sizeof(double) * h->B, cudaMemcpyDeviceToHost, s));
-            CK(cudaMemcpyAsync(bn.data(), W.beta, sizeof(double) * h->B, cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            double worst = 0;
-            for (int b = 0; b < h->B; b++) worst = std::max(worst, bn[b] > 0 ? rn[b] / bn[b] : 0.0);
-            h->last_gmres_resid = worst;
-            if (worst <= h->opt.gmres_tol) break;
-            h->refine_sweeps++;
-            // W.tmp receives the correction d of Q_0 d = r (r copied to W.dd: gmres uses W.r)
-            launch_axpby(h, n, 1.0, W.r, 0.0, nullptr, W.dd, s);
-            int st2 = prec ? prec_solve(h, W, W.dd, W.tmp, 1e-6, s) : gmres(h, W, W.dd, W.tmp, false, 1e-6, s);
+            // the correction's solve goes on to two digits below what is asked of the step's, or
+            // six digits below its own right-hand side
+            const int st2 = gmres(h, W, W.b, W.x, W.r, prec, 1e-2 * h->opt.gmres_tol, GM_REFINE, s);
             if (st2 != MOT_OK && st2 != MOT_ENOCONV) return st2;
-            launch_axpby(h, n, 1.0, W.x, 1.0, W.tmp, W.x, s);
+            if (h->last_gmres_resid <= h->opt.gmres_tol) break;
+            h->refine_sweeps++;
         }
         h->last_gmres_iters = gm_iters;
     }
@@ -923,6 +902,7 @@ MOT_API int mot_create(const mot_mesh* mesh, double eps_r, double mu_r, double d
     CK(cudaMemcpy(h->d_face_sgn, fs.data(), sizeof(double) * 3 * h->nf, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->d_iperm, h->iperm.data(), sizeof(int) * h->ne, cudaMemcpyHostToDevice));
     CK(cudaMallocHost(&h->h_cg_iters, sizeof(int) * 4));
+    CK(cudaMallocHost(&h->h_gmstat, sizeof(double) * 3 * MOT_MAX_B));
     CK(cudaEventCreateWithFlags(&h->ev_state, cudaEventDisableTiming));
     if (h->opt.timing) {
         CK(cudaEventCreate(&h->ev0));
@@ -2278,6 +2258,7 @@ MOT_API void mot_destroy(mot_handle* h) {
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (h->h_cg_iters) cudaFreeHost(h->h_cg_iters);
+    if (h->h_gmstat) cudaFreeHost(h->h_gmstat);
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
     if (h->ev_state) cudaEventDestroy(h->ev_state);

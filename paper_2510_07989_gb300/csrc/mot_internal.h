@@ -18,6 +18,8 @@
 #define MOT_TC_CHUNK 1024
 // Scatterers one launch of the tensor-core history kernel serves at most.
 #define MOT_TC_MAX_JOBS 32
+// Preconditioned Krylov vectors M V_j kept by a GMRES solve.
+#define MOT_GM_ZCAP 12
 // Size (doubles) of the fixed device array used by mot_fields_noalloc.
 #define MOT_NOALLOC_FIELD_DOUBLES 262144
 
@@ -139,14 +141,17 @@ struct mot_handle {
     double* d_g = nullptr;         // [B][m+1]
     double* d_cs = nullptr;
     double* d_sn = nullptr;
-    double* d_hcol = nullptr;      // [2][m+1][B] CGS2 coefficients
-    double* d_red = nullptr;       // reduction scratch
-    size_t red_bytes = 0;
-    double* d_resid = nullptr;     // [B]
-    double* h_resid = nullptr;     // pinned [B]
+    double* d_Z = nullptr;         // [GM_ZCAP][npad][2B] M V_j (preconditioned solves)
+    // what the host reads of a solve, one block: resid[B] (of the current
+    // iterate), resid0[B] (at its start), then the ints active[B], jend[B]
+    double* d_resid = nullptr;
+    double* h_gmstat = nullptr;    // pinned copy, MOT_MAX_B systems
+    // iterations the last solve of a kind took (0: main, 1: refinement): the
+    // host first looks whether the next one has converged after that many
+    int gm_pred[2] = {1, 1};
     int* d_iperm = nullptr;        // [ne] canonical edge -> internal row
-    int* d_gm_active = nullptr;    // [B] GMRES system still iterating
-    int* d_gm_jend = nullptr;      // [B] Krylov dimension reached
+    int* d_gm_active = nullptr;    // [B] GMRES system still iterating (in the block of d_resid)
+    int* d_gm_jend = nullptr;      // [B] Krylov dimension reached (in the block of d_resid)
     double* d_gm_bnorm = nullptr;  // [B] |b|
     double* d_wscale = nullptr;    // [B] power-of-two scale of each wave's Q_0 system in the step
     int* d_cg_iters = nullptr;     // [0] max CG iterations, [1] non-converged solves,
@@ -203,7 +208,6 @@ struct mot_handle {
     size_t emuws_bytes = 0;
     float* d_Minvf = nullptr;      // FP32 Q_0^{-1} (GMRES preconditioner), (2 npad)^2
     double* d_Minv64 = nullptr;    // FP64 Q_0^{-1} (preconditioner of the FP64 path, fp64_precond)
-    bool prec_active = false;      // apply_q0 computes Q_0 M v
     float* d_Lfinvf = nullptr;     // FP32 (Sigma^T Sigma + 11^T/N_f)^{-1}, nfpd x nfpd (CG preconditioner)
     int nfpd = 0;                  // N_f padded to 64
     double* d_pcg_work = nullptr;  // 5 x nfpd x 2B
@@ -211,7 +215,6 @@ struct mot_handle {
     float* d_pcg_f32 = nullptr;    // nfpd x 2B
     int last_pcg_iters = 0;
     bool precomputing = false;     // dense operators being assembled (use the product form)
-    double gm_tol = 1e-12;         // relative tolerance of the GMRES solve in progress
     int refine_sweeps = 0;         // FP64 refinement sweeps used by the last step
     // CUDA-event timing of the history launches (mot_options.timing)
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -301,16 +304,16 @@ void launch_window_sums(mot_handle* h, long long i, cudaStream_t s);
 void launch_recover(mot_handle* h, long long i, cudaStream_t s);
 void launch_pack_w(mot_handle* h, const double* x, double* out, cudaStream_t s);  // internal -> [B][2][ne]
 
-// GMRES pieces
-void launch_gm_dots(mot_handle* h, const double* V, int nvec, const double* w, double* out, cudaStream_t s);
-void launch_gm_update(mot_handle* h, const double* V, int nvec, const double* coef, double* w, cudaStream_t s);
-void launch_gm_norm(mot_handle* h, const double* w, double* out, cudaStream_t s);
-void launch_gm_scale(mot_handle* h, const double* w, const double* nrm, double* v, cudaStream_t s);
-void launch_gm_arnoldi_finish(mot_handle* h, int j, const double* hcol, const double* nrm, cudaStream_t s);
-void launch_gm_init(mot_handle* h, const double* beta, int first_cycle, cudaStream_t s);
+// GMRES (k_gmres.cu)
+// start of a cycle: V0 = r / |r| per system; first: also the reference norms |b|
+void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r, double* V0, cudaStream_t s);
+// iteration j: w = Q_0 V_j orthogonalised, V_{j+1}, rotated Hessenberg column, residual against
+// tol |b| and gain |r0|
+void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, cudaStream_t s);
+// x = (add ? x : 0) + sum_{v < nv} Z_v y_v, y the least-squares solution
+void launch_gm_finish(mot_handle* h, const double* Z, int nv, bool add, double* y, double* x, cudaStream_t s);
 // power-of-two scale of every wave's system (sc[b] = 2^-e) and its application
 void launch_wave_scale(mot_handle* h, const double* x, double* sc, cudaStream_t s);
 void launch_wave_apply(mot_handle* h, const double* sc, bool inverse, double* x, cudaStream_t s);
-void launch_gm_solve_update(mot_handle* h, double* y, double* x, cudaStream_t s);
 
 }  // namespace mot

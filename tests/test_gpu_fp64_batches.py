@@ -44,3 +44,17 @@ def test_fp64_march_over_batches(M, torus, B, kw):
     for b in sorted({0, B - 1}):
         ref = S.march(exc, n, b=b)
         assert np.abs(W[:, b].reshape(n, -1) - ref).max() < 1e-10 * np.abs(ref).max()
+
+
+def test_preconditioned_solve_past_the_kept_vectors(M, torus):
+    """A preconditioned solve longer than the Krylov vectors M V_j it keeps
+    (12): 14 iterations forced by a tolerance no residual reaches. The status
+    says so, and the iterate kept is the solution to the same 1e-10."""
+    ops, S = torus
+    exc = MS.fibonacci_batch(2, ops.dt, w_steps=20, t0_steps=20, r_obj=1.3)
+    n = 35
+    s = M.Solver(ops, fp64_precond=1, gmres_tol=1e-30, gmres_maxit=14)
+    W = s.run(exc, n)
+    assert s.noconv > 0 and s.info()["last_gmres_iters"] == 14
+    ref = S.march(exc, n, b=1)
+    assert np.abs(W[:, 1].reshape(n, -1) - ref).max() < 1e-10 * np.abs(ref).max()
