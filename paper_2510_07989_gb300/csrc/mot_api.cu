@@ -74,9 +74,7 @@ void launch_scatter_lf(mot_handle* h, long long Q0, long long Qend, const double
 // dense factorisation (k_dense.cu)
 int dense_lu(mot_handle* h, int n, double* A, int* piv, int* d_bad, cudaStream_t s);
 void dense_pad_identity(mot_handle* h, int n, int ne, double* A, cudaStream_t s);
-void dense_lap_plus_j(mot_handle* h, const DCsr& L, int npd, double* A, cudaStream_t s);
-int pcg_dense_prec(mot_handle* h, const DCsr& L, int npd, const float* M, const double* f, int C, double* z,
-                   double* work, double* d_scal, float* fstage, double tol, int maxit, cudaStream_t s);
+void dense_from_csr(mot_handle* h, const DCsr& L, double plus, int npd, double* A, cudaStream_t s);
 void dense_inverse_from_lu(mot_handle* h, int n, const double* LU, const int* piv, double* X, cudaStream_t s);
 void direct_laplacian_solve(mot_handle* h, int N, int npd, const double* Linv, const double* f, int C, double* r,
                             double* z, double* sc, cudaStream_t s);
@@ -232,26 +230,29 @@ size_t work_doubles(mot_handle* h) {
     return n;
 }
 
-// out = P^Sigma x  (C = 2B columns); Sigma^T x -> CG on Sigma^T Sigma -> Sigma z.
-// The mixed path preconditions the FP64 CG with an FP32 dense (L + 11^T/N_f)^{-1}.
+// out = P^Sigma x  (C = 2B columns): Sigma (Sigma^T Sigma)^+ Sigma^T x
 void project_sigma(mot_handle* h, const Work& W, const double* x, double* out, cudaStream_t s) {
     const int C = 2 * h->B;
+    if (h->d_Lfinvf) {
+        launch_project_refine(h, true, x, C, out, W.cgw, h->opt.cg_maxit, s);
+        return;
+    }
     launch_sigma_t(h, x, C, W.fvec, s);
     if (h->d_Lfinv64) {  // FP64 path with fp64_direct: the dense pseudo-inverse
         direct_laplacian_solve(h, h->nf, h->dfpd, h->d_Lfinv64, W.fvec, C, h->d_dir_r, h->d_dir_z, h->d_dir_sc, s);
         launch_sigma(h, h->d_dir_z, C, out, s);
         return;
     }
-    if (h->d_Lfinvf && h->d_pcg_work && !h->precomputing)
-        h->last_pcg_iters = pcg_dense_prec(h, h->Lf, h->nfpd, h->d_Lfinvf, W.fvec, C, W.zvec, h->d_pcg_work,
-                                           h->d_pcg_scal, h->d_pcg_f32, h->opt.cg_tol, 50, s);
-    else
-        launch_cg(h, h->Lf, nullptr, W.fvec, C, W.zvec, W.cgw, s);
+    launch_cg(h, h->Lf, nullptr, W.fvec, C, W.zvec, W.cgw, s);
     launch_sigma(h, W.zvec, C, out, s);
 }
 
 // out = P^Lambda x for C columns
 void project_lambda(mot_handle* h, const Work& W, const double* x, int C, double* out, cudaStream_t s) {
+    if (h->d_Lvinvf) {
+        launch_project_refine(h, false, x, C, out, W.cgw, h->opt.cg_maxit, s);
+        return;
+    }
     launch_lambda_t(h, x, C, W.fvec, s);
     if (h->d_Lvinv64) {  // FP64 path with fp64_direct: the dense pseudo-inverse
         direct_laplacian_solve(h, h->nv, h->dvpd, h->d_Lvinv64, W.fvec, C, h->d_dir_r, h->d_dir_z, h->d_dir_sc, s);
@@ -271,6 +272,8 @@ void left_factor(mot_handle* h, const Work& W, const double* y1, const double* y
     launch_pack2(h, y1, W.z2, C, W.Y4, s);
     if (h->d_Ginv64) {  // FP64 path with fp64_direct: X = G^{-1} Y with the dense inverse
         launch_gemm_rect(h, h->npad, h->npad, h->d_Ginv64, W.Y4, 2 * C, W.X4, s);
+    } else if (h->d_Ginvf) {
+        launch_gram_refine(h, W.Y4, 2 * C, W.X4, W.cgw, h->opt.cg_maxit, s);
     } else {
         launch_spmv(h, h->Gt, W.Y4, 2 * C, W.GY4, s);        // G^T Y
         launch_cg(h, h->G, &h->Gt, W.GY4, 2 * C, W.X4, W.cgw, s);  // (G^T G) X = G^T Y
@@ -460,14 +463,6 @@ int ensure_state(mot_handle* h, int B) {
         }
         h->d_xf = (float*)dalloc(h, sizeof(float) * 2 * bv);
         if (!h->d_xf) return fail(h, MOT_EOOM, "device allocation of the march state");
-        if (h->d_Lfinvf) {
-            const size_t blk = (size_t)h->nfpd * 2 * B;
-            h->d_pcg_work = (double*)dalloc(h, sizeof(double) * (4 * blk + (size_t)((h->nfpd + 63) / 64) * 2 * B));
-            h->d_pcg_scal = (double*)dalloc(h, sizeof(double) * 8 * 2 * B);
-            h->d_pcg_f32 = (float*)dalloc(h, sizeof(float) * blk);
-            if (!h->d_pcg_work || !h->d_pcg_scal || !h->d_pcg_f32)
-                return fail(h, MOT_EOOM, "device allocation of the march state");
-        }
     }
     h->d_wprev1 = (double*)dalloc(h, sizeof(double) * bv);
     h->d_wprev2 = (double*)dalloc(h, sizeof(double) * bv);
@@ -507,14 +502,12 @@ void free_state(mot_handle* h) {
     for (void* p : ptrs)
         if (p) cudaFree(p);
     h->d_wprev1 = h->d_wprev2 = nullptr;
-    void* fptrs[] = {h->d_ring32, h->d_win32, h->d_xf, h->d_pcg_work, h->d_pcg_scal, h->d_pcg_f32, h->d_ring16,
-                     h->d_win16};
+    void* fptrs[] = {h->d_ring32, h->d_win32, h->d_xf, h->d_ring16, h->d_win16};
     for (void* p : fptrs)
         if (p) cudaFree(p);
-    h->d_ring32 = h->d_win32 = h->d_xf = h->d_pcg_f32 = nullptr;
+    h->d_ring32 = h->d_win32 = h->d_xf = nullptr;
     h->d_ring16 = h->d_win16 = nullptr;
     h->hist_tc = false;
-    h->d_pcg_work = h->d_pcg_scal = nullptr;
     h->d_waves = h->d_ring = h->d_win = h->d_cur = h->d_dft = h->d_work = h->d_partial = nullptr;
     h->d_V = h->d_H = h->d_g = h->d_cs = h->d_sn = h->d_Z = h->d_resid = nullptr;
     h->d_gm_active = h->d_gm_jend = nullptr;
@@ -1400,32 +1393,6 @@ int precompute_mixed(mot_handle* h) {
         cudaFree(piv);
         h->device_bytes -= (int64_t)(2 * sizeof(double) * (size_t)n2 * n2 + sizeof(int) * (size_t)(n2 + 1));
     }
-    {
-        // preconditioner of the FP64 CG behind P^Sigma: (Sigma^T Sigma + 11^T/N_f)^{-1}, which is the
-        // pseudo-inverse on the range of the face Laplacian (connected surface), kept in FP32
-        const int npd = (h->nf + 63) / 64 * 64;
-        double* A = (double*)dalloc(h, sizeof(double) * (size_t)npd * npd);
-        double* inv = (double*)dalloc(h, sizeof(double) * (size_t)npd * npd);
-        int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(npd + 1));
-        h->d_Lfinvf = (float*)dalloc(h, sizeof(float) * (size_t)npd * npd);
-        if (!A || !inv || !piv || !h->d_Lfinvf) return fail(h, MOT_EOOM, "device allocation (Laplacian factorisation)");
-        dense_lap_plus_j(h, h->Lf, npd, A, s);
-        const int bad = dense_lu(h, npd, A, piv, piv + npd, s);
-        if (bad == 0) {
-            dense_inverse_from_lu(h, npd, A, piv, inv, s);
-            launch_d2f(h, (size_t)npd * npd, inv, h->d_Lfinvf, s);
-            h->nfpd = npd;
-        }
-        CK(cudaDeviceSynchronize());
-        cudaFree(A);
-        cudaFree(inv);
-        cudaFree(piv);
-        h->device_bytes -= (int64_t)(2 * sizeof(double) * (size_t)npd * npd + sizeof(int) * (size_t)(npd + 1));
-        if (bad != 0) {  // not connected: keep the plain CG
-            cudaFree(h->d_Lfinvf);
-            h->d_Lfinvf = nullptr;
-        }
-    }
     CK(cudaGetLastError());
     CK(cudaDeviceSynchronize());
     int it[2];
@@ -1523,6 +1490,65 @@ int precompute_fp64(mot_handle* h) {
     return MOT_OK;
 }
 
+// FP32 dense inverses for the projector and Gram solves: A (the CSR matrix plus
+// `plus` on every entry) factorised in FP64 and inverted, kept in FP32, then
+// tried on a right-hand side: eight sweeps must converge. If they do not (a
+// surface of several components, whose Laplacian has more than the constants in
+// its null space; a matrix singular to working precision) or there is no
+// memory, the solve stays plain CG.
+enum { INV_FACES = 0, INV_VERTS = 1, INV_GRAM = 2 };
+
+int form_refine_inverse(mot_handle* h, int kind) {
+    const DCsr& A = kind == INV_FACES ? h->Lf : kind == INV_VERTS ? h->Lv : h->G;
+    float** out = kind == INV_FACES ? &h->d_Lfinvf : kind == INV_VERTS ? &h->d_Lvinvf : &h->d_Ginvf;
+    if (!refine_fits(A.n)) return MOT_OK;
+    cudaStream_t s = 0;
+    const int npd = ((kind == INV_GRAM ? h->npad : A.n) + 63) / 64 * 64;
+    const size_t nn = (size_t)npd * npd;
+    const int64_t held = h->device_bytes;
+    double* a = (double*)dalloc(h, sizeof(double) * nn);
+    double* inv = (double*)dalloc(h, sizeof(double) * nn);
+    int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(npd + 1));
+    // trial: x and its result (2 columns), the solve's work
+    double* trial = (double*)dalloc(h, sizeof(double) * (4 * (size_t)h->npad + 6 * (size_t)A.n));
+    *out = (float*)dalloc(h, sizeof(float) * nn);
+    bool good = a && inv && piv && trial && *out;
+    if (good) {
+        dense_from_csr(h, A, kind == INV_GRAM ? 0.0 : 1.0 / A.n, npd, a, s);
+        good = dense_lu(h, npd, a, piv, piv + npd, s) == 0;
+    }
+    if (good) {
+        dense_inverse_from_lu(h, npd, a, piv, inv, s);
+        launch_d2f(h, nn, inv, *out, s);
+        std::vector<double> x(2 * (size_t)h->npad, 0.0);
+        uint32_t g = 12345u;
+        for (size_t i = 0; i < 2 * (size_t)h->ne; i++) {  // a fixed sequence in (-1, 1)
+            g = g * 1664525u + 1013904223u;
+            x[i] = (double)(int32_t)g / 2147483648.0;
+        }
+        CK(cudaMemcpy(trial, x.data(), sizeof(double) * x.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemsetAsync(h->d_cg_iters, 0, 2 * sizeof(int), s));
+        double* y = trial + 2 * (size_t)h->npad;
+        if (kind == INV_GRAM)
+            launch_gram_refine(h, trial, 2, y, y + 2 * (size_t)h->npad, 8, s);
+        else
+            launch_project_refine(h, kind == INV_FACES, trial, 2, y, y + 2 * (size_t)h->npad, 8, s);
+        int it[2];
+        CK(cudaMemcpy(it, h->d_cg_iters, 2 * sizeof(int), cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(x.data(), y, sizeof(double) * x.size(), cudaMemcpyDeviceToHost));
+        good = it[1] == 0;
+        for (double v : x) good = good && std::isfinite(v);
+    }
+    CK(cudaDeviceSynchronize());
+    CK(cudaGetLastError());
+    void* tmp[] = {a, inv, piv, trial, good ? nullptr : *out};
+    for (void* p : tmp)
+        if (p) cudaFree(p);
+    if (!good) *out = nullptr;
+    h->device_bytes = held + (good ? (int64_t)(sizeof(float) * nn) : 0);
+    return MOT_OK;
+}
+
 // FP64 path with fp64_direct: dense FP64 inverses of the Gram matrix and of
 // the two graph Laplacians (plus 11^T/N), formed once by LU with partial
 // pivoting, so the left factor and the projectors are exact to rounding
@@ -1561,7 +1587,7 @@ int prepare_fp64_direct(mot_handle* h, const std::vector<std::tuple<int, int, do
         int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(npd + 1));
         *out = (double*)dalloc(h, sizeof(double) * (size_t)npd * npd);
         if (!A || !piv || !*out) return fail(h, MOT_EOOM, "device allocation (dense Laplacian inverse)");
-        dense_lap_plus_j(h, L, npd, A, s);
+        dense_from_csr(h, L, 1.0 / L.n, npd, A, s);
         const int bad = dense_lu(h, npd, A, piv, piv + npd, s);
         if (bad == 0) dense_inverse_from_lu(h, npd, A, piv, *out, s);
         CK(cudaDeviceSynchronize());
@@ -1625,8 +1651,12 @@ MOT_API int mot_load_operators(mot_handle* h, const mot_operators* ops) {
     HostCsr G = csr_from_triplets(ne, ne, tg), Gt = csr_from_triplets(ne, ne, tgt);
     if ((st = upload_csr(h, G, h->G)) != MOT_OK) return st;
     if ((st = upload_csr(h, Gt, h->Gt)) != MOT_OK) return st;
-    if (h->opt.precision == MOT_PREC_FP64 && h->opt.fp64_direct && (st = prepare_fp64_direct(h, tg)) != MOT_OK)
-        return st;
+    if (h->opt.precision == MOT_PREC_FP64 && h->opt.fp64_direct) {
+        if ((st = prepare_fp64_direct(h, tg)) != MOT_OK) return st;
+    } else {
+        for (int kind : {INV_FACES, INV_VERTS, INV_GRAM})
+            if ((st = form_refine_inverse(h, kind)) != MOT_OK) return st;
+    }
     // RHS quadrature table
     h->nq = ops->nq;
     std::vector<double> x((size_t)np * h->nq * 3, 0.0), wf((size_t)np * h->nq * 3, 0.0);
@@ -2248,7 +2278,7 @@ MOT_API void mot_destroy(mot_handle* h) {
                     h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_x, h->d_rhs_wf, h->d_tiles, h->d_tmask,
                     h->hist.tasks, h->hist.chunks, h->hist.chunk_ptr, h->lag0.tasks, h->lag0.chunks,
                     h->lag0.chunk_ptr, h->d_omega, h->d_colidx, h->d_tiles32, h->d_Q0, h->d_Q0f, h->d_LF,
-                    h->d_LFf, h->d_Minvf, h->d_Minv64, h->d_Lfinvf, h->hist_tc_list.packed, h->hist_tc_list.chunks,
+                    h->d_LFf, h->d_Minvf, h->d_Minv64, h->d_Lfinvf, h->d_Lvinvf, h->d_Ginvf, h->hist_tc_list.packed, h->hist_tc_list.chunks,
                     h->hist_tc_list.rb_ptr, h->hist_tc_list.rb_chunks, h->d_tiles16, h->d_sgws, h->d_emuws,
                     h->d_Ginv64, h->d_Lfinv64, h->d_Lvinv64, h->d_dir_r, h->d_dir_z, h->d_dir_sc};
     emu_free(h, &h->emu_Q0);

@@ -208,12 +208,11 @@ struct mot_handle {
     size_t emuws_bytes = 0;
     float* d_Minvf = nullptr;      // FP32 Q_0^{-1} (GMRES preconditioner), (2 npad)^2
     double* d_Minv64 = nullptr;    // FP64 Q_0^{-1} (preconditioner of the FP64 path, fp64_precond)
-    float* d_Lfinvf = nullptr;     // FP32 (Sigma^T Sigma + 11^T/N_f)^{-1}, nfpd x nfpd (CG preconditioner)
-    int nfpd = 0;                  // N_f padded to 64
-    double* d_pcg_work = nullptr;  // 5 x nfpd x 2B
-    double* d_pcg_scal = nullptr;  // 6 x 2B doubles + 2B ints
-    float* d_pcg_f32 = nullptr;    // nfpd x 2B
-    int last_pcg_iters = 0;
+    // FP32 inverses behind the projector and Gram solves (k_project.cu), formed at
+    // load, leading dimension the order rounded up to 64; null: plain CG
+    float* d_Lfinvf = nullptr;     // (Sigma^T Sigma + 11^T/N_f)^{-1}
+    float* d_Lvinvf = nullptr;     // (Lambda^T Lambda + 11^T/N_v)^{-1}
+    float* d_Ginvf = nullptr;      // G^{-1}
     bool precomputing = false;     // dense operators being assembled (use the product form)
     int refine_sweeps = 0;         // FP64 refinement sweeps used by the last step
     // CUDA-event timing of the history launches (mot_options.timing)
@@ -295,6 +294,11 @@ void launch_lambda(mot_handle* h, const double* z, int C, double* x, cudaStream_
 void launch_spmv(mot_handle* h, const DCsr& A, const double* x, int C, double* y, cudaStream_t s);
 int launch_cg(mot_handle* h, const DCsr& A, const DCsr* A2, const double* f, int C, double* z, double* work,
               cudaStream_t s);  // returns max iterations or -1 on no convergence
+// projector and Gram solves by refinement with the FP32 inverses (k_project.cu)
+bool refine_fits(int N);
+void launch_project_refine(mot_handle* h, bool faces, const double* x, int C, double* out, double* work, int maxit,
+                           cudaStream_t s);
+void launch_gram_refine(mot_handle* h, const double* y, int C, double* out, double* work, int maxit, cudaStream_t s);
 void launch_gemm(mot_handle* h, const double* A, const double* X, int C, double* Y, cudaStream_t s);
 // Y[M][C] = A[M][K] X[K][C], FP64
 void launch_gemm_rect(mot_handle* h, int M, int K, const double* A, const double* X, int C, double* Y,
