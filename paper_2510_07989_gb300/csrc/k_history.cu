@@ -35,11 +35,7 @@ __device__ __forceinline__ const double* panel_ptr(int mode, const double* ring,
 // those: the lanes of a warp are columns of one row (2B a multiple of 32) and
 // walk its mask together; in other batches they walk the union of their rows'
 // masks. One full-depth launch at 432 edges, 53 lags, B = 64: 20.5 ms with
-// every entry multiplied, 8.7 ms with the masks. Below B = 4 (SKIP = false) a
-// warp spans eight rows or more, few entries are zero in all of them, and the
-// plain loop's loads overlap better: a step at 1920 edges, B = 1 is 2 % slower
-// with the masks, one at 270 edges, B = 5 is 2 % faster.
-template <bool SKIP>
+// every entry multiplied, 8.7 ms with the masks.
 __global__ void __launch_bounds__(NT) k_hist_f64(const HistTask* __restrict__ tasks,
                                                  const HistChunk* __restrict__ chunks,
                                                  const double* __restrict__ tiles,
@@ -68,12 +64,6 @@ __global__ void __launch_bounds__(NT) k_hist_f64(const HistTask* __restrict__ ta
             const int r = o < nout ? o / C2 : T - 1, c = o < nout ? o - r * C2 : 0;
             const double* sr = st + r * (T + 1);
             double s = acc[j];
-            if (!SKIP) {
-#pragma unroll 8
-                for (int n = 0; n < T; n++) s = fma(sr[n], sp[n * C2 + c], s);
-                acc[j] = s;
-                continue;
-            }
             uint32_t m = __reduce_or_sync(0xffffffffu, o < nout ? smask[r] : 0u);
             while (m) {  // two nonzeros at a time: their loads overlap
                 const int n0 = __ffs(m) - 1;
@@ -96,7 +86,7 @@ __global__ void __launch_bounds__(NT) k_hist_f64(const HistTask* __restrict__ ta
         const int* cols = colidx + (size_t)ch.rb * npad + (size_t)tk.cb * T;  // distance-sorted columns
         const double* tl = tiles + (size_t)tk.tile * T * T;
         __syncthreads();
-        if (SKIP && tid < T) smask[tid] = masks[(size_t)tk.tile * T + tid];
+        if (tid < T) smask[tid] = masks[(size_t)tk.tile * T + tid];
         for (int e = tid; e < T * T; e += NT) st[(e / T) * (T + 1) + (e % T)] = tl[e];
         for (int e = tid; e < T * C2; e += NT) {
             const int r = e / C2;
@@ -117,6 +107,88 @@ __global__ void __launch_bounds__(NT) k_hist_f64(const HistTask* __restrict__ ta
             dst[nout + o] = acc1[j];
         }
     }
+}
+
+// B <= 4 (C2 = 2, 4, 6 or 8 columns): a warp takes eight rows of a tile, its
+// lanes the 32 tile columns, and every lane keeps its products' sums over all
+// tasks of the chunk in registers -- the lanes are summed once per output and
+// chunk, not per tile, and nothing is staged: a tile row is one coalesced
+// 256-byte load, a lane gathers its own coefficient row, and the next task's
+// loads are in flight during this one's products. Bound by the FP64 units
+// (2B multiply-adds per tile entry) with the tile stream close behind. Four
+// warps cover a tile; the CTA's other four take every second task.
+template <int C2>
+__global__ void __launch_bounds__(NT) k_hist_f64_small(const HistTask* __restrict__ tasks,
+                                                       const HistChunk* __restrict__ chunks,
+                                                       const double* __restrict__ tiles,
+                                                       const double* __restrict__ ring, const double* __restrict__ win,
+                                                       const double* __restrict__ kry, int mode, long long step_i,
+                                                       int R, int npad, const int* __restrict__ colidx,
+                                                       double* __restrict__ partial) {
+    constexpr int RW = 8, NV = RW * C2;  // rows per warp, sums per lane
+    __shared__ double sums[2][2][T * C2];  // [task stream][target][row][column]
+    const HistChunk ch = chunks[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row0 = (warp & 3) * RW, half = warp >> 2;
+    for (int i = threadIdx.x; i < 4 * T * C2; i += NT) (&sums[0][0][0])[i] = 0.0;
+    __syncthreads();
+    double acc[RW][C2];
+#pragma unroll
+    for (int r = 0; r < RW; r++)
+#pragma unroll
+        for (int c = 0; c < C2; c++) acc[r][c] = 0.0;
+    // sums of the lanes into this warp's rows of target `out`
+    auto flush = [&](int out) {
+#pragma unroll
+        for (int r = 0; r < RW; r++)
+#pragma unroll
+            for (int c = 0; c < C2; c++) {
+                double v = acc[r][c];
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                if (lane == 0) sums[half][out][(row0 + r) * C2 + c] += v;
+                acc[r][c] = 0.0;
+            }
+    };
+    const int* cols = colidx + (size_t)ch.rb * npad;
+    const int end = ch.first + ch.count;
+    auto live = [&](int t) {  // the next task of this stream that takes part
+        while (t < end && mode == 0 && step_i - tasks[t].k < 1) t += 2;
+        return t;
+    };
+    double a[RW], x[C2];
+    int out = 0;
+    auto fetch = [&](int t) {
+        const HistTask tk = tasks[t];
+        out = (tk.code >> 4) & 1;
+        const double* pan = panel_ptr(mode, ring, win, kry, step_i, R, npad, C2, tk.k, tk.code & 3, (tk.code >> 2) & 3) +
+                            (size_t)cols[tk.cb * T + lane] * C2;
+        const double* tl = tiles + (size_t)tk.tile * T * T + row0 * T + lane;
+#pragma unroll
+        for (int r = 0; r < RW; r++) a[r] = tl[r * T];
+#pragma unroll
+        for (int c = 0; c < C2; c++) x[c] = pan[c];
+    };
+    int t = live(ch.first + half), cur = -1;
+    if (t < end) fetch(t);
+    while (t < end) {
+        if (cur >= 0 && out != cur) flush(cur);
+        cur = out;
+        double ca[RW], cx[C2];
+#pragma unroll
+        for (int r = 0; r < RW; r++) ca[r] = a[r];
+#pragma unroll
+        for (int c = 0; c < C2; c++) cx[c] = x[c];
+        t = live(t + 2);
+        if (t < end) fetch(t);
+#pragma unroll
+        for (int r = 0; r < RW; r++)
+#pragma unroll
+            for (int c = 0; c < C2; c++) acc[r][c] = fma(ca[r], cx[c], acc[r][c]);
+    }
+    if (cur >= 0) flush(cur);
+    __syncthreads();
+    double* dst = partial + (size_t)blockIdx.x * 2 * T * C2;
+    for (int i = threadIdx.x; i < 2 * T * C2; i += NT) dst[i] = (&sums[0][0][0])[i] + (&sums[1][0][0])[i];
 }
 
 // masks[tile][r]: bit n set where entry (r, n) of the tile is nonzero; one warp per row
@@ -161,9 +233,19 @@ void launch_history(mot_handle* h, const TaskList& tl, const double* tiles, cons
         size_t smem = sizeof(double) * (T * (T + 1) + T * C2);
         const bool timed = h->opt.timing && mode == 0 && h->ev0 && step_i > h->K;
         if (timed) cudaEventRecord(h->ev0, s);
-        auto* kernel = C2 >= 8 ? k_hist_f64<true> : k_hist_f64<false>;
-        kernel<<<tl.nchunks, NT, smem, s>>>(tl.tasks, tl.chunks, tiles, h->d_tmask, ring, win, kry, mode, step_i, h->R,
-                                            h->npad, C2, h->d_colidx, h->d_partial);
+#define MOT_HIST_SMALL(CV)                                                                                       \
+    k_hist_f64_small<CV><<<tl.nchunks, NT, 0, s>>>(tl.tasks, tl.chunks, tiles, ring, win, kry, mode, step_i, h->R, \
+                                                   h->npad, h->d_colidx, h->d_partial)
+        switch (C2) {
+            case 2: MOT_HIST_SMALL(2); break;
+            case 4: MOT_HIST_SMALL(4); break;
+            case 6: MOT_HIST_SMALL(6); break;
+            case 8: MOT_HIST_SMALL(8); break;
+            default:
+                k_hist_f64<<<tl.nchunks, NT, smem, s>>>(tl.tasks, tl.chunks, tiles, h->d_tmask, ring, win, kry, mode,
+                                                        step_i, h->R, h->npad, C2, h->d_colidx, h->d_partial);
+        }
+#undef MOT_HIST_SMALL
         if (timed) {
             cudaEventRecord(h->ev1, s);
             h->ev_pending = true;
