@@ -5,11 +5,12 @@
 // System b of the batch uses columns b and B + b of a block vector
 // [npad][2B]. A thread-block cluster owns G systems (4, so that a row's
 // columns fill a 32-byte sector; 1 for B = 1) and all rows: every CTA keeps its
-// part of the new vector in registers, and the dot products are summed over
+// part of the new vector in shared memory, and the dot products are summed over
 // the cluster through distributed shared memory, in rank order (every CTA
-// gets the same sums). What bounds it is the FP64 rate of an SM (two
-// multiply-adds per clock) and the latency of the cluster barriers: three
-// reductions per iteration.
+// gets the same sums). What bounds an iteration is latency: basis vectors from
+// L2, two cluster barriers, and chains of FP64 operations of a unit that does
+// two multiply-adds per clock and SM (a double-precision square root or
+// division costs a microsecond, so one thread per system does them).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -23,7 +24,7 @@ namespace cg = cooperative_groups;
 
 constexpr int GT = 256;      // threads per CTA
 constexpr int NW = GT / 32;
-constexpr int MAXE = 12;     // elements per thread kept in registers
+constexpr int SLICE = 12288; // elements of the new vector a CTA keeps in shared memory
 constexpr int MAXCL = 8;     // CTAs per cluster (the portable limit)
 
 struct GmState {
@@ -39,31 +40,21 @@ struct GmState {
     int m;
 };
 
-// Elements of group grp (G systems): index (row * 2 + part) * G + q; element e
-// of thread t of cluster rank rk is index (e * CL + rk) * GT + t.
+// Elements of a group of G systems: index (row * 2 + part) * G + q; local element
+// l of cluster rank rk is index ((l / GT) * CL + rk) * GT + l % GT, so a lane's
+// elements l = lane + 32 i belong to system lane % G of the group.
 template <int G>
 struct Part {
-    int npad, B, C2, g0, q, rk, cl, t;
-    __device__ Part(int npad_, int B_, int rk_, int cl_)
-        : npad(npad_), B(B_), C2(2 * B_), rk(rk_), cl(cl_), t(threadIdx.x) {
+    int npad, B, g0, rk, cl;
+    __device__ Part(int npad_, int B_, int rk_, int cl_) : npad(npad_), B(B_), rk(rk_), cl(cl_) {
         g0 = (int)(blockIdx.x / cl_) * G;
-        q = t % G;
     }
-    __device__ int elements() const { return (2 * npad * G + cl * GT - 1) / (cl * GT); }
+    __device__ int elements() const { return (2 * npad * G + cl * GT - 1) / (cl * GT) * GT; }
     // offset in a block vector, or -1 outside it
-    __device__ long long at(int e) const {
-        const long long rp = ((long long)(e * cl + rk) * GT + t) / G;
-        const long long row = rp >> 1;
-        const int part = (int)(rp & 1);
-        return row < npad && g0 + q < B ? row * C2 + part * B + g0 + q : -1;
+    __device__ int at(int l) const {
+        const int idx = (l / GT * cl + rk) * GT + l % GT, rp = idx / G, q = idx % G;
+        return rp < 2 * npad && g0 + q < B ? rp * B + g0 + q : -1;
     }
-};
-
-// The new vector's elements of a thread: in registers, or (more than MAXE per
-// thread) where it stands in global memory.
-template <bool REG>
-struct Elems {
-    double r[REG ? MAXE : 1];
 };
 
 // Sums of p[0 .. 3] over the lanes of a warp with the same lane % G: lane
@@ -83,245 +74,261 @@ __device__ __forceinline__ double warp_sum4(const double (&p)[4]) {
     return v;
 }
 
-// out[i] (i < n * G: sum i / G of system i % G) = the cluster's sums of what the
-// warps left in red[warp][i]; part is this CTA's own slot, read by the others
-// after the cluster barrier.
-__device__ __forceinline__ void cluster_sums(int n, const double* red, double* part, double* out, int cl) {
+// out[i] (i < n: sum i / G of system i % G) = the cluster's sums of what this
+// and the other CTAs left in red[0 .. parts)[i]; part is this CTA's own slot,
+// read by the others after the cluster barrier.
+__device__ __forceinline__ void cluster_sums(int n, int parts, const double* red, double* part, double* out, int cl) {
     __syncthreads();
+    double* own = cl == 1 ? out : part;
     for (int i = threadIdx.x; i < n; i += GT) {
-        double s = 0.0;
+        double v[NW];
 #pragma unroll
-        for (int w = 0; w < NW; w++) s += red[w * n + i];
-        part[i] = s;
+        for (int w = 0; w < NW; w++) v[w] = w < parts ? red[w * n + i] : 0.0;
+        own[i] = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
     }
-    cg::cluster_group c = cg::this_cluster();
-    c.sync();
-    for (int i = threadIdx.x; i < n; i += GT) {
-        double s = 0.0;
-        for (int r = 0; r < cl; r++) s += c.map_shared_rank(part, r)[i];
-        out[i] = s;
+    if (cl > 1) {
+        cg::cluster_group c = cg::this_cluster();
+        c.sync();
+        for (int i = threadIdx.x; i < n; i += GT) {
+            double v[MAXCL];
+#pragma unroll
+            for (int r = 0; r < MAXCL; r++) v[r] = r < cl ? c.map_shared_rank(part, r)[i] : 0.0;
+            out[i] = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        }
     }
     __syncthreads();
 }
 
-// red[warp][v * G + q] = this warp's part of <V_v, w>, v < nv
-template <int G, bool REG>
-__device__ __forceinline__ void dots(const Part<G>& P, int ne, const double* V, size_t vs, int nv, const double* w,
-                                     const Elems<REG>& E, double* red) {
-    const int lane = P.t & 31, warp = P.t >> 5, n = nv * G;
-    for (int v0 = 0; v0 < nv; v0 += 4) {
+// Warps that share a group of four sums: all of them for one group, one each
+// from NW groups on.
+__device__ __forceinline__ int shares(int groups) { return groups >= NW ? 1 : NW / groups; }
+
+// red[share][v * G + q] = the shares' parts of <V_v, w>, v < nv, and with `norm`
+// of |w|^2 as one more sum. A warp takes four vectors at a time over its share
+// of the elements: sixteen loads in flight a lane. (All warps over the same
+// vectors, eight at a time: 46 us an iteration at 1920 edges, B = 1, 17 vectors
+// on average.)
+template <int G, bool SM>
+__device__ __forceinline__ void dots(const Part<G>& P, int L, const double* V, size_t vs, int nv, bool norm,
+                                     const double* w, const double* ws, double* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ns = nv + (norm ? 1 : 0), n = ns * G, ng = (ns + 3) / 4, parts = shares(ng);
+    for (int gi = warp; gi < ng * parts; gi += NW) {
+        const int v0 = gi % ng * 4, share = gi / ng;
         double p[4] = {0.0, 0.0, 0.0, 0.0};
-        if (REG) {
+#pragma unroll 4
+        for (int l = share * 32 + lane; l < L; l += parts * 32) {
+            const int ix = P.at(l);
+            if (ix < 0) continue;
+            const double x = SM ? ws[l] : w[ix];
 #pragma unroll
-            for (int e = 0; e < MAXE; e++) {
-                const long long ix = e < ne ? P.at(e) : -1;
-                if (ix < 0) continue;
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-                    if (v0 + i < nv) p[i] = fma(V[(size_t)(v0 + i) * vs + ix], E.r[e], p[i]);
-            }
-        } else {
-            for (int e = 0; e < ne; e++) {
-                const long long ix = P.at(e);
-                if (ix < 0) continue;
-                const double x = w[ix];
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-                    if (v0 + i < nv) p[i] = fma(V[(size_t)(v0 + i) * vs + ix], x, p[i]);
-            }
+            for (int i = 0; i < 4; i++)
+                if (v0 + i < ns) p[i] = fma(v0 + i < nv ? V[(size_t)(v0 + i) * vs + ix] : x, x, p[i]);
         }
         const double s = warp_sum4<G>(p);
         const int v = v0 + (((lane >> 4) & 1) << 1 | ((lane >> 3) & 1));
-        if ((lane & 7) < G && v < nv) red[warp * n + v * G + (lane & 7)] = s;
+        if ((lane & 7) < G && v < ns) red[share * n + v * G + (lane & 7)] = s;
     }
 }
 
-// w -= sum_v V_v h[v]
-template <int G, bool REG>
-__device__ __forceinline__ void project_out(const Part<G>& P, int ne, const double* V, size_t vs, int nv, double* w,
-                                            Elems<REG>& E, const double* h) {
-    if (REG) {
-#pragma unroll
-        for (int e = 0; e < MAXE; e++) {
-            const long long ix = e < ne ? P.at(e) : -1;
-            if (ix < 0) continue;
-            double s = 0.0;
+// sum_v V_v[ix] h[v][q]
+template <int G>
+__device__ __forceinline__ double combine(const double* V, size_t vs, int nv, int ix, const double* h, int q) {
+    double s0 = 0.0, s1 = 0.0;
+    int v = 0;
 #pragma unroll 4
-            for (int v = 0; v < nv; v++) s = fma(V[(size_t)v * vs + ix], h[v * G + P.q], s);
-            E.r[e] -= s;
-        }
-    } else {
-        for (int e = 0; e < ne; e++) {
-            const long long ix = P.at(e);
-            if (ix < 0) continue;
-            double s = 0.0;
-#pragma unroll 4
-            for (int v = 0; v < nv; v++) s = fma(V[(size_t)v * vs + ix], h[v * G + P.q], s);
-            w[ix] -= s;
-        }
-    }
-}
-
-// red[warp][q] = this warp's part of |w|^2
-template <int G, bool REG>
-__device__ __forceinline__ void square(const Part<G>& P, int ne, const double* w, const Elems<REG>& E, double* red) {
-    double p[4] = {0.0, 0.0, 0.0, 0.0};
-    if (REG) {
+    for (; v + 4 <= nv; v += 4) {
+        double a[4];
 #pragma unroll
-        for (int e = 0; e < MAXE; e++)
-            if (e < ne) p[0] = fma(E.r[e], E.r[e], p[0]);
-    } else {
-        for (int e = 0; e < ne; e++) {
-            const long long ix = P.at(e);
-            const double x = ix >= 0 ? w[ix] : 0.0;
-            p[0] = fma(x, x, p[0]);
-        }
+        for (int i = 0; i < 4; i++) a[i] = V[(size_t)(v + i) * vs + ix];
+        s0 = fma(a[0], h[v * G + q], s0);
+        s1 = fma(a[1], h[(v + 1) * G + q], s1);
+        s0 = fma(a[2], h[(v + 2) * G + q], s0);
+        s1 = fma(a[3], h[(v + 3) * G + q], s1);
     }
-    const double s = warp_sum4<G>(p);
-    const int lane = P.t & 31;
-    if (lane < G) red[(P.t >> 5) * G + lane] = s;
+    for (; v < nv; v++) s0 = fma(V[(size_t)v * vs + ix], h[v * G + q], s0);
+    return s0 + s1;
 }
 
-template <int G, bool REG>
-__device__ __forceinline__ void load(const Part<G>& P, int ne, const double* w, Elems<REG>& E) {
-    if (!REG) return;
-#pragma unroll
-    for (int e = 0; e < MAXE; e++) {
-        const long long ix = e < ne ? P.at(e) : -1;
-        E.r[e] = ix >= 0 ? w[ix] : 0.0;
-    }
-}
-
-// v = w * f (the group's systems that are live), else 0
-template <int G, bool REG>
-__device__ __forceinline__ void store_scaled(const Part<G>& P, int ne, const double* w, const Elems<REG>& E, double f,
-                                             double* v) {
-    if (REG) {
-#pragma unroll
-        for (int e = 0; e < MAXE; e++) {
-            const long long ix = e < ne ? P.at(e) : -1;
-            if (ix >= 0) v[ix] = E.r[e] * f;
-        }
-    } else {
-        for (int e = 0; e < ne; e++) {
-            const long long ix = P.at(e);
-            if (ix >= 0) v[ix] = w[ix] * f;
-        }
-    }
-}
-
-// Below this norm a vector of an O(1) system is a breakdown: its system is done.
-constexpr double TINY_NORM = 1e-150;
+// Below this squared norm a vector of an O(1) system is a breakdown: its system is done.
+constexpr double TINY2 = 1e-300;
 
 // Start of a cycle: beta = |r| per system, V_0 = r / beta. On the first cycle
 // also the reference norm |b| (b == r: one vector).
-template <int G, bool REG>
+template <int G>
 __global__ void __launch_bounds__(GT) k_gm_begin(int npad, int B, const double* __restrict__ b, int first,
                                                  const double* __restrict__ r, double* __restrict__ V0, GmState S) {
-    extern __shared__ double sm[];
+    __shared__ double red[NW * 2 * G], part[2 * G], out[2 * G], inv_s[G];
     cg::cluster_group c = cg::this_cluster();
     const int cl = (int)c.num_blocks(), rk = (int)c.block_rank();
     const Part<G> P(npad, B, rk, cl);
-    const int ne = P.elements();
-    double* red = sm;                // NW x G
-    double* part = red + NW * G;     // 2 x G (one slot per reduction)
-    double* out = part + 2 * G;      // 2 x G
-    Elems<REG> E;
+    const int L = P.elements(), t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const bool other = first && b != r;
-    if (other) {
-        load<G, REG>(P, ne, b, E);
-        square<G, REG>(P, ne, b, E, red);
-        cluster_sums(G, red, part, out, cl);
+    double p[4] = {0.0, 0.0, 0.0, 0.0};  // |r|^2, |b|^2
+    for (int l = t; l < L; l += GT) {
+        const int ix = P.at(l);
+        if (ix < 0) continue;
+        const double x = r[ix];
+        p[0] = fma(x, x, p[0]);
+        if (other) {
+            const double y = b[ix];
+            p[1] = fma(y, y, p[1]);
+        }
     }
-    load<G, REG>(P, ne, r, E);
-    square<G, REG>(P, ne, r, E, red);
-    cluster_sums(G, red, part + G, out + G, cl);
-    const int sys = P.g0 + P.q;
-    const double beta = sqrt(out[G + P.q]);
-    double bn = 0.0;
-    if (sys < B) bn = first ? (other ? sqrt(out[P.q]) : beta) : S.bnorm[sys];
-    const bool live = beta > 0.0 && bn > 0.0;
-    store_scaled<G, REG>(P, ne, r, E, live && beta > TINY_NORM ? 1.0 / beta : 0.0, V0);
-    if (rk == 0 && P.t < G && sys < B) {
-        S.g[(size_t)sys * (S.m + 1)] = beta;
-        if (first) S.bnorm[sys] = bn;
-        if (first) S.resid0[sys] = bn > 0.0 ? beta / bn : 0.0;
-        S.active[sys] = live ? 1 : 0;
-        S.jend[sys] = 0;
-        S.resid[sys] = bn > 0.0 ? beta / bn : 0.0;
+    const double s = warp_sum4<G>(p);
+    if ((lane & 7) < G && lane < 16) red[warp * 2 * G + (lane >> 3) * G + (lane & 7)] = s;
+    cluster_sums(2 * G, NW, red, part, out, cl);
+    c.barrier_arrive();  // this CTA has read what it needs of the others' shared memory
+    if (t < G) {
+        const int sys = P.g0 + t;
+        const double n2 = out[t], iv = n2 > TINY2 ? rsqrt(n2) : 0.0;
+        const double beta = n2 > TINY2 ? n2 * iv : sqrt(n2);
+        double bn = 0.0;
+        if (sys < B) bn = !first ? S.bnorm[sys] : other ? sqrt(out[G + t]) : beta;
+        const bool live = beta > 0.0 && bn > 0.0;
+        inv_s[t] = live ? iv : 0.0;
+        if (rk == 0 && sys < B) {
+            const double rel = bn > 0.0 ? beta / bn : 0.0;
+            S.g[(size_t)sys * (S.m + 1)] = beta;
+            if (first) S.bnorm[sys] = bn;
+            if (first) S.resid0[sys] = rel;
+            S.active[sys] = live ? 1 : 0;
+            S.jend[sys] = 0;
+            S.resid[sys] = rel;
+        }
     }
-    c.sync();  // every read of a CTA's shared memory by the others is done
+    __syncthreads();
+    for (int l = t; l < L; l += GT) {
+        const int ix = P.at(l);
+        if (ix >= 0) V0[ix] = r[ix] * inv_s[l % G];
+    }
+    c.barrier_wait();  // ... and they of this one's
 }
 
 // Iteration j: w (= Q_0 V_j) orthogonalised against V_0 .. V_j (classical
 // Gram-Schmidt twice), V_{j+1} = w / |w|, and the new column of the rotated
-// Hessenberg matrix. A system is done at a residual of tol |b|, or of gain times
-// its residual at the start. A system that is done writes V_{j+1} = 0 from its next
-// iteration on and keeps its state, so iterations past its end change nothing.
-template <int G, bool REG>
+// Hessenberg matrix. |w|^2 after the second pass is the sum of squares before
+// it less that pass's coefficients (summed with them: two reductions, not
+// three), unless it took most of the vector away. A system is done at a residual
+// of tol |b|, or of gain times its residual at the start. A system that is done
+// writes V_{j+1} = 0 from its next iteration on and keeps its state, so
+// iterations past its end change nothing.
+template <int G, bool SM>
 __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const double* __restrict__ V, size_t vs,
                                                 double* __restrict__ w, double* __restrict__ Vnext, double tol,
                                                 double gain, GmState S) {
     extern __shared__ double sm[];
+    __shared__ double inv_s[G], n2_s[G];
+    __shared__ int lost_s[G];
     cg::cluster_group c = cg::this_cluster();
     const int cl = (int)c.num_blocks(), rk = (int)c.block_rank();
     const Part<G> P(npad, B, rk, cl);
-    const int ne = P.elements(), nv = j + 1, n = nv * G;
-    double* red = sm;               // NW x n
-    double* part = red + NW * n;    // 2 n + G (one slot per reduction)
-    double* h1 = part + 2 * n + G;  // n
-    double* h2 = h1 + n;            // n
-    double* nr = h2 + n;            // G
-    double* rot = nr + G;           // 2 x j x G: cosines, sines of the earlier rotations
-    const int sys = P.g0 + P.q;
-    const bool valid = sys < B;
-    const bool live = valid && S.active[sys] != 0;  // read before the first barrier, written after the last
-    if (rk == 0)
-        for (int i = P.t; i < j * G; i += GT) {
+    const int L = P.elements(), nv = j + 1, n = nv * G, t = threadIdx.x;
+    double* red = sm;                // NW (n + G)
+    double* part = red + NW * (n + G);  // 2 n + 2 G (one slot per reduction)
+    double* h1 = part + 2 * n + 2 * G;  // n
+    double* h2 = h1 + n;             // n + G: coefficients, |w|^2
+    double* sq = h2 + n + G;         // G
+    double* rot = sq + G;            // 2 x j x G: cosines, sines of the earlier rotations
+    double* ws = rot + 2 * j * G;    // L (SM)
+    const int sys = P.g0 + t;        // of threads t < G
+    const bool mine = t < G && sys < B;
+    // read before the first barrier, written after the last by rank 0
+    const bool live = mine && S.active[sys] != 0;
+    double gj = 0.0, ibn = 0.0, floor_r = 0.0;
+    if (rk == 0) {
+        for (int i = t; i < j * G; i += GT) {
             const int b = P.g0 + i % G;
             rot[i] = b < B ? S.cs[(size_t)b * S.m + i / G] : 1.0;
             rot[j * G + i] = b < B ? S.sn[(size_t)b * S.m + i / G] : 0.0;
         }
-    Elems<REG> E;
-    load<G, REG>(P, ne, w, E);
-    dots<G, REG>(P, ne, V, vs, nv, w, E, red);
-    cluster_sums(n, red, part, h1, cl);
-    project_out<G, REG>(P, ne, V, vs, nv, w, E, h1);
-    dots<G, REG>(P, ne, V, vs, nv, w, E, red);
-    cluster_sums(n, red, part + n, h2, cl);
-    project_out<G, REG>(P, ne, V, vs, nv, w, E, h2);
-    square<G, REG>(P, ne, w, E, red);
-    cluster_sums(G, red, part + 2 * n, nr, cl);
-    const double nrm = sqrt(nr[P.q]);
-    store_scaled<G, REG>(P, ne, w, E, live && nrm > TINY_NORM ? 1.0 / nrm : 0.0, Vnext);
-    if (rk == 0 && P.t < G && live) {
+        if (live) {
+            gj = S.g[(size_t)sys * (S.m + 1) + j];
+            ibn = 1.0 / S.bnorm[sys];
+            floor_r = fmax(tol, gain * S.resid0[sys]);
+        }
+    }
+    if (SM)
+        for (int l = t; l < L; l += GT) {
+            const int ix = P.at(l);
+            ws[l] = ix >= 0 ? w[ix] : 0.0;
+        }
+    __syncthreads();
+    dots<G, SM>(P, L, V, vs, nv, false, w, ws, red);
+    cluster_sums(n, shares((nv + 3) / 4), red, part, h1, cl);
+    for (int l = t; l < L; l += GT) {
+        const int ix = P.at(l);
+        if (ix < 0) continue;
+        const double s = combine<G>(V, vs, nv, ix, h1, l % G);
+        if (SM) ws[l] -= s;
+        else w[ix] -= s;
+    }
+    __syncthreads();
+    dots<G, SM>(P, L, V, vs, nv, true, w, ws, red);
+    cluster_sums(n + G, shares((nv + 4) / 4), red, part + n, h2, cl);
+    if (t < G) {
+        double s = h2[n + t], m = s;
+        for (int v = 0; v < nv; v++) m -= h2[v * G + t] * h2[v * G + t];
+        n2_s[t] = m;
+        lost_s[t] = !(m >= 0.5 * s);  // the second pass took most of it away
+    }
+    __syncthreads();
+    bool again = false;
+#pragma unroll
+    for (int q = 0; q < G; q++) again |= lost_s[q] != 0;
+    if (again) {  // the same in every CTA of the cluster: it follows from the sums
+        double p[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int l = t; l < L; l += GT) {
+            const int ix = P.at(l);
+            if (ix < 0) continue;
+            const double x = (SM ? ws[l] : w[ix]) - combine<G>(V, vs, nv, ix, h2, l % G);
+            p[0] = fma(x, x, p[0]);
+        }
+        const double s = warp_sum4<G>(p);
+        if ((t & 31) < G) red[(t >> 5) * G + (t & 31)] = s;
+        cluster_sums(G, NW, red, part + 2 * n + G, sq, cl);
+        if (t < G) n2_s[t] = sq[t];
+    }
+    c.barrier_arrive();  // this CTA has read what it needs of the others' shared memory
+    if (t < G) inv_s[t] = live && n2_s[t] > TINY2 ? rsqrt(n2_s[t]) : 0.0;
+    __syncthreads();
+    for (int l = t; l < L; l += GT) {
+        const int ix = P.at(l);
+        if (ix < 0) continue;
+        const double iv = inv_s[l % G];
+        const double x = (SM ? ws[l] : w[ix]) - combine<G>(V, vs, nv, ix, h2, l % G);
+        Vnext[ix] = iv != 0.0 ? x * iv : 0.0;
+    }
+    if (rk == 0 && live) {
         double* Hb = S.H + (size_t)sys * (S.m + 1) * S.m;
-        double* gb = S.g + (size_t)sys * (S.m + 1);
-        double a = h1[P.q] + h2[P.q];
+        double a = h1[t] + h2[t];
         for (int i = 0; i < j; i++) {
-            const double x = h1[(i + 1) * G + P.q] + h2[(i + 1) * G + P.q];
-            const double cc = rot[i * G + P.q], ss = rot[(j + i) * G + P.q];
+            const double x = h1[(i + 1) * G + t] + h2[(i + 1) * G + t];
+            const double cc = rot[i * G + t], ss = rot[(j + i) * G + t];
             Hb[(size_t)i * S.m + j] = cc * a + ss * x;
             a = -ss * a + cc * x;
         }
-        const double d = hypot(a, nrm);
-        double cc = 1.0, ss = 0.0;
-        if (d > 0.0) {
-            cc = a / d;
-            ss = nrm / d;
+        const double n2 = fmax(n2_s[t], 0.0), nrm = n2 > TINY2 ? n2 * inv_s[t] : sqrt(n2);
+        const double d2 = fma(a, a, n2);  // all O(1) or less: b is scaled to O(1)
+        double d = 0.0, cc = 1.0, ss = 0.0;
+        if (d2 > 0.0) {
+            const double id = rsqrt(d2);
+            d = d2 * id;
+            cc = a * id;
+            ss = nrm * id;
         }
         S.cs[(size_t)sys * S.m + j] = cc;
         S.sn[(size_t)sys * S.m + j] = ss;
         Hb[(size_t)j * S.m + j] = d;
-        const double gj = gb[j];
+        double* gb = S.g + (size_t)sys * (S.m + 1);
         gb[j + 1] = -ss * gj;
         gb[j] = cc * gj;
-        const double rr = fabs(ss * gj) / S.bnorm[sys];
+        const double rr = fabs(ss * gj) * ibn;
         S.resid[sys] = rr;
         S.jend[sys] = j + 1;
-        if (rr <= fmax(tol, gain * S.resid0[sys]) || !(nrm > 0.0)) S.active[sys] = 0;
+        if (rr <= floor_r || !(nrm > 0.0)) S.active[sys] = 0;
     }
-    c.sync();
+    c.barrier_wait();  // ... and they of this one's
 }
 
 // y = H^{-1} g (upper triangular, size jend[b]) into y[i][b], i < nv (0 past
@@ -366,13 +373,6 @@ GmState state_of(mot_handle* h) {
     return GmState{h->d_H, h->d_g, h->d_cs, h->d_sn, h->d_gm_bnorm, h->d_resid, h->d_resid + h->B, h->d_gm_active, h->d_gm_jend, h->gm_m};
 }
 
-// Cluster size: about two elements per thread, at most the portable eight CTAs.
-int cluster_of(long long elements) {
-    int cl = 1;
-    while (cl < MAXCL && elements > (long long)cl * GT * 2) cl *= 2;
-    return cl;
-}
-
 template <class K, class... A>
 void launch_cluster(K kernel, int groups, int cl, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
@@ -403,15 +403,17 @@ void set_attributes(mot_handle* h) {
 
 struct Shape {
     int G, groups, cl;
-    bool reg;
+    long long per_cta;  // elements
 };
-Shape shape_of(const mot_handle* h) {
+// Cluster size: about `per` elements per CTA, at most the portable eight CTAs.
+Shape shape_of(const mot_handle* h, int per) {
     Shape p;
     p.G = h->B == 1 ? 1 : 4;
     p.groups = (h->B + p.G - 1) / p.G;
     const long long el = 2LL * h->npad * p.G;
-    p.cl = cluster_of(el);
-    p.reg = el <= (long long)p.cl * GT * MAXE;
+    p.cl = 1;
+    while (p.cl < MAXCL && el > (long long)p.cl * per) p.cl *= 2;
+    p.per_cta = (el + p.cl * GT - 1) / (p.cl * GT) * GT;
     return p;
 }
 
@@ -420,22 +422,22 @@ Shape shape_of(const mot_handle* h) {
 namespace mot {
 
 void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r, double* V0, cudaStream_t s) {
-    const Shape p = shape_of(h);
-    auto* k = p.G == 1 ? (p.reg ? k_gm_begin<1, true> : k_gm_begin<1, false>)
-                       : (p.reg ? k_gm_begin<4, true> : k_gm_begin<4, false>);
-    launch_cluster(k, p.groups, p.cl, sizeof(double) * (NW + 4) * p.G, s, h->npad, h->B, b, first ? 1 : 0, r, V0,
-                   state_of(h));
+    const Shape p = shape_of(h, 2048);
+    launch_cluster(p.G == 1 ? k_gm_begin<1> : k_gm_begin<4>, p.groups, p.cl, 0, s, h->npad, h->B, b, first ? 1 : 0, r,
+                   V0, state_of(h));
     h->launches++;
 }
 
 void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, cudaStream_t s) {
     set_attributes(h);
-    const Shape p = shape_of(h);
+    const Shape p = shape_of(h, 512);
     const size_t vs = (size_t)h->npad * 2 * h->B;
     const int n = (j + 1) * p.G;
-    const size_t smem = sizeof(double) * ((size_t)NW * n + 4 * n + 2 * p.G + 2 * (size_t)j * p.G);
-    auto* k = p.G == 1 ? (p.reg ? k_gm_iter<1, true> : k_gm_iter<1, false>)
-                       : (p.reg ? k_gm_iter<4, true> : k_gm_iter<4, false>);
+    const bool sm = p.per_cta <= SLICE;
+    const size_t smem = sizeof(double) * ((size_t)NW * (n + p.G) + 4 * n + 4 * p.G + 2 * (size_t)j * p.G +
+                                          (sm ? (size_t)p.per_cta : 0));
+    auto* k = p.G == 1 ? (sm ? k_gm_iter<1, true> : k_gm_iter<1, false>)
+                       : (sm ? k_gm_iter<4, true> : k_gm_iter<4, false>);
     launch_cluster(k, p.groups, p.cl, smem, s, h->npad, h->B, j, (const double*)h->d_V, vs, w,
                    h->d_V + (size_t)(j + 1) * vs, tol, gain, state_of(h));
     h->launches++;

@@ -306,7 +306,8 @@ __global__ void k_split_sum(long long n, int S, const double* __restrict__ W, do
 
 // Y[n][C] = A[n][K] X[K][C] for C <= 8: one warp per row, lanes over the
 // contraction index (coalesced rows of A), warp-shuffle reduction. Bound by
-// reading A (C <= 2) or the FP64 units.
+// reading A (C <= 2) or the FP64 units; 16-byte loads, four of A in flight per
+// lane (8-byte loads: 57 us at 3840 x 3840, C = 1, 2.0 TB/s).
 template <int CC>
 __global__ void __launch_bounds__(256) k_gemv_small(int n, int K, const double* __restrict__ A,
                                                     const double* __restrict__ X, double* __restrict__ Y) {
@@ -316,11 +317,17 @@ __global__ void __launch_bounds__(256) k_gemv_small(int n, int K, const double* 
 #pragma unroll
         for (int c = 0; c < CC; c++) acc[c] = 0.0;
         const double* a = A + (size_t)row * K;
-#pragma unroll 8
-        for (int k = lane; k < K; k += 32) {
-            const double av = a[k];
+#pragma unroll 4
+        for (int k = 2 * lane; k < K; k += 64) {  // K is even, rows 16-byte aligned
+            const double2 av = *reinterpret_cast<const double2*>(a + k);
+            double2 x[CC];  // X rows k, k + 1
 #pragma unroll
-            for (int c = 0; c < CC; c++) acc[c] = fma(av, X[(size_t)k * CC + c], acc[c]);
+            for (int c = 0; c < CC; c++) x[c] = *reinterpret_cast<const double2*>(X + (size_t)k * CC + 2 * c);
+            const double* xs = reinterpret_cast<const double*>(x);
+#pragma unroll
+            for (int c = 0; c < CC; c++) acc[c] = fma(av.x, xs[c], acc[c]);
+#pragma unroll
+            for (int c = 0; c < CC; c++) acc[c] = fma(av.y, xs[CC + c], acc[c]);
         }
 #pragma unroll
         for (int c = 0; c < CC; c++) {

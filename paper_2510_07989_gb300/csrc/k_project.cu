@@ -37,7 +37,6 @@ namespace cg = cooperative_groups;
 constexpr int PT = 512;  // threads per CTA
 constexpr int PW = PT / 32;
 constexpr int CL = 8;    // CTAs per cluster
-constexpr int RPW = 4;   // rows of M a warp multiplies together
 constexpr int REFINE_SMEM = 220 * 1024;
 
 enum { FACES = 0, VERTS = 1, GRAM = 2 };
@@ -84,6 +83,7 @@ template <int CW, int MODE>
 __global__ void __launch_bounds__(PT) k_refine_solve(Problem Q, const double* __restrict__ x, double* __restrict__ out,
                                                      double* __restrict__ work, double tol, int maxit,
                                                      int* __restrict__ it_max, int* __restrict__ noconv) {
+    constexpr int RPW = CW == 8 ? 4 : 8;         // rows of M a warp multiplies together: 16 to 32 loads in flight a lane
     extern __shared__ __align__(16) float rs[];  // [N][CW] r in FP32 (CW = 8: two halves of 4 columns)
     __shared__ double red[PW][CW];
     __shared__ double col[3][CW];                // this CTA's column values of the three reductions
