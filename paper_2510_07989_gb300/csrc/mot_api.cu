@@ -928,9 +928,13 @@ const int kKindFamily[NTK] = {0, 0, 0, 1, 1, 1, 2, 2, 2, 3};  // 0 A, 1 Ah, 2 At
 // lags. Within a piece: coefficient transform (variant; windowed sums
 // separately), lag, column block.
 // cap: most tasks per chunk; lag_frac: the fraction of the L2 that the ring
-// slots of one lag range may fill (sets the lags per range).
+// slots of one lag range may fill (sets the lags per range); launch_tasks: tasks
+// of the launch the list is for, over all scatterers it serves (0: this one's).
+// A launch of few tasks is cut into smaller chunks than cap, at least four a
+// CTA slot: a chunk is one CTA's work, and at 1024 tasks the 14 046 tasks of a
+// 216-edge torus were 14 CTAs on 152 SMs (750 us a launch).
 int make_tc_list(mot_handle* h, const std::vector<HistTask>& tasks, const std::vector<int>& rbs, int cap,
-                 double lag_frac) {
+                 double lag_frac, int64_t launch_tasks = 0) {
     const int nrb = h->nrb;
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->dev);
@@ -979,6 +983,11 @@ int make_tc_list(mot_handle* h, const std::vector<HistTask>& tasks, const std::v
         return a.cb < b.cb;
     });
     cap = std::max(1, std::min(cap, MOT_TC_CHUNK));  // tasks per chunk (staged in the CTA's shared memory)
+    h->tc_cap = cap;
+    int nsm = 148;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    const int64_t all = std::max<int64_t>(launch_tasks, (int64_t)m.size());
+    cap = (int)std::min<int64_t>(cap, std::max<int64_t>(16, all / (4 * nsm)));
     int maxcount = 0;
     std::vector<HistChunk> chunks;
     std::vector<std::vector<int>> per_rb(nrb);
@@ -1008,7 +1017,6 @@ int make_tc_list(mot_handle* h, const std::vector<HistTask>& tasks, const std::v
     tl.ntasks = (int)m.size();
     tl.nchunks = (int)chunks.size();
     tl.cap = std::max(1, maxcount);
-    h->tc_cap = cap;
     h->tc_lag_frac = lag_frac;
     tl.packed = (uint4*)dalloc(h, sizeof(uint4) * std::max<size_t>(1, packed.size()));
     tl.chunks = (HistChunk*)dalloc(h, sizeof(HistChunk) * std::max<size_t>(1, chunks.size()));
@@ -1814,6 +1822,8 @@ int tune_tc(mot_handle* const* hs, int n, cudaStream_t s) {
         max_npad = std::max(max_npad, hs[k]->npad);
     }
     const bool bulk = hs[0]->tc_bulk;
+    int64_t all = 0;
+    for (int k = 0; k < n; k++) all += hs[k]->hist_tc_list.ntasks;
     float best = 1e30f;
     int bcap = MOT_TC_CHUNK, bns = 0, bepi = 4, btp = 1;
     double blf = 0.4;
@@ -1823,7 +1833,8 @@ int tune_tc(mot_handle* const* hs, int n, cudaStream_t s) {
         for (double lf : fracs) {
             int st;
             for (int k = 0; k < n; k++) {
-                if ((st = make_tc_list(hs[k], hs[k]->tc_tasks_host, hs[k]->tc_rbs_host, cap, lf)) != MOT_OK) return st;
+                if ((st = make_tc_list(hs[k], hs[k]->tc_tasks_host, hs[k]->tc_rbs_host, cap, lf, all)) != MOT_OK)
+                    return st;
                 if (!hs[k]->hist_tc_list.packed) return fail(hs[k], MOT_EINVAL, "tensor-core list not available");
                 if ((st = fit_partial(hs[k])) != MOT_OK) return st;
             }
@@ -1857,7 +1868,7 @@ int tune_tc(mot_handle* const* hs, int n, cudaStream_t s) {
         }
     for (int k = 0; k < n; k++) {
         int st;
-        if ((st = make_tc_list(hs[k], hs[k]->tc_tasks_host, hs[k]->tc_rbs_host, bcap, blf)) != MOT_OK) return st;
+        if ((st = make_tc_list(hs[k], hs[k]->tc_tasks_host, hs[k]->tc_rbs_host, bcap, blf, all)) != MOT_OK) return st;
         if ((st = fit_partial(hs[k])) != MOT_OK) return st;
         hs[k]->tc_stages = bns;
         hs[k]->tc_tps = btp;

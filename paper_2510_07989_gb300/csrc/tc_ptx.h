@@ -42,6 +42,19 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+// whether the phase has completed (no suspension)
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // try_wait with a suspend-time hint: the thread sleeps until the phase
 // completes or about `ns` nanoseconds pass, instead of spinning on the issue
 // slots the working warps of its sub-partition need.
@@ -75,6 +88,7 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
 }
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err,
                                           int code, unsigned long long bound = WAIT_NS) {
+    if (mbar_test(bar, parity)) return true;
     // fast path: up to 1024 tries of at most ~1 us of suspension each (~1 ms),
     // then the time-bounded slow path
 #pragma unroll 1
