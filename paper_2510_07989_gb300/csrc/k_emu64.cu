@@ -33,6 +33,7 @@
 // TMEM and issues the MMAs (lane 0), warps 2-5 fold TMEM into the sums (one
 // output row per thread, 64 columns). Every mbarrier wait is bounded in time
 // and ends in an error status.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -43,6 +44,7 @@
 namespace {
 
 using namespace tcx;
+namespace cg = cooperative_groups;
 
 constexpr int EM = 128;           // rows of A per CTA
 constexpr int EN = 64;            // columns of X per CTA
@@ -139,51 +141,86 @@ __global__ void k_slice_rows(int M, int Mp, int K, const double* __restrict__ A,
     }
 }
 
-// exponent of every column of X (K x N, row-major)
-__global__ void k_col_exponents(int K, int N, const double* __restrict__ X, int* __restrict__ ex) {
-    const int j = blockIdx.x;
-    double m = 0.0;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) m = fmax(m, fabs(X[(size_t)k * N + j]));
-    __shared__ double red[256];
-    red[threadIdx.x] = m;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        int e = 0;
-        if (red[0] > 0.0) frexp(red[0], &e);
-        ex[j] = e;
-    }
-}
-
-// X (K x N) -> slices of X^T in [NH][K / 32][S][64 x 32, 64-byte swizzle]
+// X (K x N, row-major) -> the exponent of every column (|x| / 2^e < 1, 0 for a
+// zero column) and the slices of X^T in [NH][K / 32][S][64 x 32, 64-byte
+// swizzle]. A cluster owns eight columns (one 64-byte sector pair per row of X):
+// each CTA takes a share of the rows, the column maxima are combined through
+// distributed shared memory, and the rows are read again (L1 / L2) and sliced:
+// one launch where maxima (a CTA per column, 8-byte strided loads) and slices
+// were two (20 us at 1848 x 64).
+//
+// The slices are the balanced base-128 digits of the value rounded once to
+// 7 S - 1 bits below the column's scale: one multiplication and one conversion
+// per value in the double-precision unit (two operations per clock and SM), the
+// digits in integer arithmetic; a slice at a time by rounding and subtracting
+// took five double-precision operations for each. |digit| <= 64, and the digits
+// sum to the same rounded value. Non-finite values go on as NaN.
+constexpr int XCOLS = 8, XT = 256;
 template <int NSL>
-__global__ void k_slice_cols(int K, int N, int NH, const double* __restrict__ X, const int* __restrict__ ex,
-                             __nv_bfloat16* __restrict__ X16) {
-    const int KT = K / EK;
-    const long long total = (long long)NH * EN * (K / 8);
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int n = (int)(idx % (NH * EN)), k8 = (int)(idx / (NH * EN));
-        float s[8][NSL];
+__global__ void __launch_bounds__(XT) k_slice_x(int K, int N, const double* __restrict__ X, int* __restrict__ ex,
+                                                __nv_bfloat16* __restrict__ X16) {
+    cg::cluster_group c = cg::this_cluster();
+    const int cl = (int)c.num_blocks(), rk = (int)c.block_rank();
+    __shared__ double red[XT / 32][XCOLS], top[XCOLS];
+    const int n0 = (int)(blockIdx.x / cl) * XCOLS, KT = K / EK, K8 = K / 8;
+    const int t = threadIdx.x, q = t % XCOLS, n = n0 + q, lane = t & 31, warp = t >> 5;
+    const int g = t / XCOLS, GR = XT / XCOLS;  // row groups of eight
+    double m = 0.0;
+    if (n < N)
+        for (int k8 = rk * GR + g; k8 < K8; k8 += cl * GR)
 #pragma unroll
-        for (int e = 0; e < 8; e++) {
-            const double x = n < N ? ldexp(X[(size_t)(k8 * 8 + e) * N + n], -ex[n]) : 0.0;
-            slice_n<NSL>(x, s[e]);
+            for (int e = 0; e < 8; e++) m = fmax(m, fabs(X[(size_t)(k8 * 8 + e) * N + n]));
+    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 8));
+    if (lane < XCOLS) red[warp][lane] = m;
+    __syncthreads();
+    if (t < XCOLS) {
+        for (int w = 0; w < XT / 32; w++) m = fmax(m, red[w][t]);
+        top[t] = m;
+    }
+    c.sync();
+    m = 0.0;
+    for (int r = 0; r < cl; r++) m = fmax(m, c.map_shared_rank(top, r)[q]);
+    c.barrier_arrive();
+    int e2 = 0;
+    if (m > 0.0) frexp(m, &e2);
+    if (rk == 0 && t < XCOLS && n < N) ex[n] = e2;
+    const int up = 7 * NSL - 1 - e2;  // the value times 2^up is rounded to an integer
+    const bool plain = up > -1000 && up < 1000;
+    const double f = plain ? __longlong_as_double((long long)(up + 1023) << 52) : 0.0;
+    const int nh = n / EN, r = n % EN;
+    for (int k8 = rk * GR + g; k8 < K8; k8 += cl * GR) {
+        uint32_t w[NSL][4];
+#pragma unroll
+        for (int p = 0; p < NSL; p++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) w[p][i] = 0u;
+        if (n < N) {
+            double x[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) x[e] = X[(size_t)(k8 * 8 + e) * N + n];
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const double y = plain ? x[e] * f : ldexp(x[e], up);
+                long long v = __double2ll_rn(y);
+                const bool bad = !(fabs(y) < 1e15);  // NaN or infinite
+#pragma unroll
+                for (int p = NSL - 1; p >= 0; p--) {
+                    const int d = p > 0 ? (int)((v + 64) & 127) - 64 : (int)v;
+                    v = (v - d) >> 7;
+                    const uint32_t h = bad ? 0x7fc0u : (uint32_t)__bfloat16_as_ushort(__int2bfloat16_rn(d));  // exact
+                    w[p][e >> 1] |= h << (16 * (e & 1));
+                }
+            }
         }
-        const int nh = n / EN, r = n % EN, kt = (k8 * 8) / EK, kc = ((k8 * 8) % EK) / 8;
+        const int kt = k8 * 8 / EK, kc = k8 * 8 % EK / 8;
         unsigned char* base = reinterpret_cast<unsigned char*>(X16 + (((size_t)nh * KT + kt) * NSL) * (EN * EK));
 #pragma unroll
-        for (int q = 0; q < NSL; q++) {
-            __nv_bfloat16 b[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) b[e] = __float2bfloat16_rn(s[e][q]);
-            *reinterpret_cast<uint4*>(base + (size_t)q * B_TILE + sw64_chunk(r, kc)) =
-                make_uint4(pack2(b[0], b[1]), pack2(b[2], b[3]), pack2(b[4], b[5]), pack2(b[6], b[7]));
-        }
+        for (int p = 0; p < NSL; p++)
+            *reinterpret_cast<uint4*>(base + (size_t)p * B_TILE + sw64_chunk(r, kc)) =
+                make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
     }
+    c.barrier_wait();
 }
 
 // Y[z] (M x N, rows < M, columns < N) = partial product over the k-tiles
@@ -406,9 +443,22 @@ int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, doub
     double* ws = reinterpret_cast<double*>(h->d_emuws);
     __nv_bfloat16* d_x16 = reinterpret_cast<__nv_bfloat16*>(h->d_emuws + part);
     int* d_ex = reinterpret_cast<int*>(h->d_emuws + part + x16);
-    k_col_exponents<<<N, 256, 0, s>>>(K, N, X, d_ex);
-    const long long total = (long long)NH * EN * (K / 8);
-    const int blocks = (int)std::min<long long>((total + 255) / 256, 152 * 32);
+    {
+        cudaLaunchConfig_t cfg = {};
+        // a CTA takes 32 groups of eight rows at a time
+        int cl = 1;
+        while (cl < 8 && K / 8 > cl * XT / XCOLS) cl *= 2;
+        cfg.gridDim = dim3(NH * EN / XCOLS * cl);
+        cfg.blockDim = dim3(XT);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = cl;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, NSL == 6 ? k_slice_x<6> : k_slice_x<4>, K, N, X, d_ex, d_x16);
+    }
     static std::atomic<unsigned long long> attr{0};
     once_per_device(attr, h->dev, [] {
         cudaFuncSetAttribute(k_emu_gemm<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EmuCfg<6>::SMEM);
@@ -418,15 +468,13 @@ int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, doub
     const auto* a16 = reinterpret_cast<const __nv_bfloat16*>(A.a16);
     double* out = S > 1 ? ws : Y;
     if (NSL == 6) {
-        k_slice_cols<6><<<blocks, 256, 0, s>>>(K, N, NH, X, d_ex, d_x16);
         k_emu_gemm<6><<<grid, E_THREADS, EmuCfg<6>::SMEM, s>>>(A.M, N, K, kts, a16, A.ea, d_x16, d_ex, out,
                                                                h->d_cg_iters + 2);
     } else {
-        k_slice_cols<4><<<blocks, 256, 0, s>>>(K, N, NH, X, d_ex, d_x16);
         k_emu_gemm<4><<<grid, E_THREADS, EmuCfg<4>::SMEM, s>>>(A.M, N, K, kts, a16, A.ea, d_x16, d_ex, out,
                                                                h->d_cg_iters + 2);
     }
-    h->launches += 3;
+    h->launches += 2;
     if (S > 1) {
         const size_t n = (size_t)A.M * N;
         k_emu_reduce<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256, 0, s>>>(n, S, ws, Y);

@@ -202,10 +202,11 @@ __global__ void k_tile_masks(long long rows, const double* __restrict__ tiles, u
 }
 
 // out_s[rb*T + r][c] = sum over the chunks of row block rb of partial[chunk][target][r][c],
-// in order. One thread per output: with one CTA per row block (a few dozen) the
+// in order; with rho, rho - that sum. One thread per output: with one CTA per row block (a few dozen) the
 // chunk loop ran at a fraction of the memory rate (321 us at 432 edges, B = 64).
 __global__ void __launch_bounds__(256) k_hist_reduce(const int* __restrict__ chunk_ptr,
                                                      const double* __restrict__ partial, int C2,
+                                                     const double* __restrict__ rho1, const double* __restrict__ rho2,
                                                      double* __restrict__ s1, double* __restrict__ s2) {
     const int rb = blockIdx.y;
     const int nout = T * C2;
@@ -215,10 +216,9 @@ __global__ void __launch_bounds__(256) k_hist_reduce(const int* __restrict__ chu
     double a = 0.0;
 #pragma unroll 4
     for (int c = chunk_ptr[rb]; c < c1; c++) a += partial[(size_t)c * 2 * nout + o];
-    if (o < nout)
-        s1[(size_t)rb * nout + o] = a;
-    else
-        s2[(size_t)rb * nout + o - nout] = a;
+    const size_t ix = (size_t)rb * nout + (o < nout ? o : o - nout);
+    if (rho1) a = (o < nout ? rho1 : rho2)[ix] - a;
+    (o < nout ? s1 : s2)[ix] = a;
 }
 
 }  // namespace
@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(256) k_hist_reduce(const int* __restrict__ chu
 namespace mot {
 
 void launch_history(mot_handle* h, const TaskList& tl, const double* tiles, const double* ring, const double* win,
-                    const double* kry, int mode, long long step_i, double* out_s1, double* out_s2,
-                    cudaStream_t s) {
+                    const double* kry, int mode, long long step_i, const double* rho1, const double* rho2,
+                    double* out_s1, double* out_s2, cudaStream_t s) {
     const int C2 = 2 * h->B;
     if (tl.nchunks > 0) {
         size_t smem = sizeof(double) * (T * (T + 1) + T * C2);
@@ -252,13 +252,13 @@ void launch_history(mot_handle* h, const TaskList& tl, const double* tiles, cons
         }
         h->launches++;
     }
-    launch_history_reduce(h, tl, C2, out_s1, out_s2, s);
+    launch_history_reduce(h, tl, C2, rho1, rho2, out_s1, out_s2, s);
 }
 
-void launch_history_reduce(mot_handle* h, const TaskList& tl, int C2, double* out_s1, double* out_s2,
-                           cudaStream_t s) {
+void launch_history_reduce(mot_handle* h, const TaskList& tl, int C2, const double* rho1, const double* rho2,
+                           double* out_s1, double* out_s2, cudaStream_t s) {
     const dim3 grid((2 * T * C2 + 255) / 256, h->nrb);
-    k_hist_reduce<<<grid, 256, 0, s>>>(tl.chunk_ptr, h->d_partial, C2, out_s1, out_s2);
+    k_hist_reduce<<<grid, 256, 0, s>>>(tl.chunk_ptr, h->d_partial, C2, rho1, rho2, out_s1, out_s2);
     h->launches++;
 }
 

@@ -343,9 +343,35 @@ __global__ void __launch_bounds__(256) k_gemv_small(int n, int K, const double* 
 // rho1[e][b] (u-part) / rho1[e][B+b] (v-part): (1/dt) int p_i (e, h) tested;
 // rho2: (1/T_max) (d/dt^-1 (e, h))(i dt) tested, 0 after t_trunc.
 // Testing with n x f_m gives -<f_m, .>. Section V-C, Eq. (hin).
-__global__ void k_rhs(int ne, int npad, int B, int nq, const double* __restrict__ xq, const double* __restrict__ wf,
-                      const double* __restrict__ waves, double ti, double tprev, double dt, double tmax, double c,
-                      double eta, double* __restrict__ rho1, double* __restrict__ rho2) {
+//
+// The incident field's time integral needs two error functions per point and
+// wave, FP64 work of a unit that does two operations per clock and SM. A
+// triangle's points are those of its three edges' functions, so they are
+// evaluated once per distinct point of the quadrature table (a third of it;
+// found at load), and beyond |argument| = 6 the error function is 1 to the last
+// bit: before the pulse arrives and after it has passed nothing is evaluated.
+// F[pt][0][b] = (A/2c) (erf(a1) - erf(a0)),  F[pt][1][b] = (A/2c) (1 + erf(a1))
+__global__ void __launch_bounds__(128) k_rhs_points(int npts, int B, const double* __restrict__ pts,
+                                                    const double* __restrict__ waves, double ti, double tprev, double c,
+                                                    double* __restrict__ F) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= npts * B) return;
+    const int pt = i / B, b = i - pt * B;
+    const double* wv = waves + 10 * b;
+    const double A = wv[0], w = wv[7], t0 = wv[8];
+    const double kd = wv[4] * pts[3 * pt] + wv[5] * pts[3 * pt + 1] + wv[6] * pts[3 * pt + 2];
+    auto erf_sat = [](double a) { return a >= 6.0 ? 1.0 : a <= -6.0 ? -1.0 : erf(a); };
+    const double f = 4.0 / w;
+    const double e1 = erf_sat(f * (c * (ti - t0) - kd)), e0 = erf_sat(f * (c * (tprev - t0) - kd));
+    const double g = A / (2.0 * c);
+    F[((size_t)pt * 2) * B + b] = g * (e1 - e0);
+    F[((size_t)pt * 2 + 1) * B + b] = g * (1.0 + e1);
+}
+
+__global__ void k_rhs_edges(int ne, int npad, int B, int nq, const int* __restrict__ ptidx,
+                            const double* __restrict__ wf, const double* __restrict__ F,
+                            const double* __restrict__ waves, double ti, double dt, double tmax, double eta,
+                            double* __restrict__ rho1, double* __restrict__ rho2) {
     const int C2 = 2 * B;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npad * B; i += gridDim.x * blockDim.x) {
         const int r = i / B, b = i - r * B;
@@ -354,31 +380,26 @@ __global__ void k_rhs(int ne, int npad, int B, int nq, const double* __restrict_
             rho2[(size_t)r * C2 + b] = rho2[(size_t)r * C2 + B + b] = 0.0;
             continue;
         }
-        const double* wv = waves + 10 * b;
-        const double A = wv[0], px = wv[1], py = wv[2], pz = wv[3], kx = wv[4], ky = wv[5], kz = wv[6];
-        const double w = wv[7], t0 = wv[8], ttr = wv[9];
-        const double hx = (ky * pz - kz * py) / eta, hy = (kz * px - kx * pz) / eta, hz = (kx * py - ky * px) / eta;
-        double e1 = 0, h1 = 0, e2 = 0, h2 = 0;
+        double d[3] = {0, 0, 0}, s[3] = {0, 0, 0};
+#pragma unroll 2
         for (int q = 0; q < nq; q++) {
-            const double* x = xq + ((size_t)r * nq + q) * 3;
             const double* f = wf + ((size_t)r * nq + q) * 3;
-            const double kd = kx * x[0] + ky * x[1] + kz * x[2];
-            const double a1 = (4.0 / w) * (c * (ti - t0) - kd);
-            const double a0 = (4.0 / w) * (c * (tprev - t0) - kd);
-            const double s1 = (A / (2.0 * c)) * (1.0 + erf(a1));
-            const double ds = (A / (2.0 * c)) * (erf(a1) - erf(a0));
-            const double fp = f[0] * px + f[1] * py + f[2] * pz;
-            const double fh = f[0] * hx + f[1] * hy + f[2] * hz;
-            e1 += fp * ds;
-            h1 += fh * ds;
-            e2 += fp * s1;
-            h2 += fh * s1;
+            const double* v = F + (size_t)ptidx[r * nq + q] * 2 * B + b;
+            const double ds = v[0], s1 = v[B];
+#pragma unroll
+            for (int t = 0; t < 3; t++) {
+                d[t] = fma(f[t], ds, d[t]);
+                s[t] = fma(f[t], s1, s[t]);
+            }
         }
-        rho1[(size_t)r * C2 + b] = -e1 / dt;
-        rho1[(size_t)r * C2 + B + b] = -h1 / dt;
-        const bool on = ti <= ttr;
-        rho2[(size_t)r * C2 + b] = on ? -e2 / tmax : 0.0;
-        rho2[(size_t)r * C2 + B + b] = on ? -h2 / tmax : 0.0;
+        const double* wv = waves + 10 * b;
+        const double px = wv[1], py = wv[2], pz = wv[3], kx = wv[4], ky = wv[5], kz = wv[6];
+        const double hx = (ky * pz - kz * py) / eta, hy = (kz * px - kx * pz) / eta, hz = (kx * py - ky * px) / eta;
+        rho1[(size_t)r * C2 + b] = -(px * d[0] + py * d[1] + pz * d[2]) / dt;
+        rho1[(size_t)r * C2 + B + b] = -(hx * d[0] + hy * d[1] + hz * d[2]) / dt;
+        const bool on = ti <= wv[9];
+        rho2[(size_t)r * C2 + b] = on ? -(px * s[0] + py * s[1] + pz * s[2]) / tmax : 0.0;
+        rho2[(size_t)r * C2 + B + b] = on ? -(hx * s[0] + hy * s[1] + hz * s[2]) / tmax : 0.0;
     }
 }
 
@@ -717,10 +738,12 @@ void launch_gemm(mot_handle* h, const double* A, const double* X, int C, double*
 }
 
 void launch_rhs(mot_handle* h, long long i, double* rho1, double* rho2, cudaStream_t s) {
-    k_rhs<<<grid_for((long long)h->npad * h->B), 256, 0, s>>>(h->ne, h->npad, h->B, h->nq, h->d_rhs_x, h->d_rhs_wf,
-                                                              h->d_waves, i * h->dt, (i - 1) * h->dt, h->dt,
-                                                              h->tmax, h->c, h->eta, rho1, rho2);
-    h->launches++;
+    k_rhs_points<<<(h->npts * h->B + 127) / 128, 128, 0, s>>>(h->npts, h->B, h->d_pts, h->d_waves, i * h->dt,
+                                                              (i - 1) * h->dt, h->c, h->d_ptfield);
+    k_rhs_edges<<<grid_for((long long)h->npad * h->B, 128), 128, 0, s>>>(
+        h->ne, h->npad, h->B, h->nq, h->d_ptidx, h->d_rhs_wf, h->d_ptfield, h->d_waves, i * h->dt, h->dt, h->tmax,
+        h->eta, rho1, rho2);
+    h->launches += 2;
 }
 
 void launch_window_sums(mot_handle* h, long long i, cudaStream_t s) {

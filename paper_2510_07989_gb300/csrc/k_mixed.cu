@@ -392,8 +392,8 @@ inline int grid_for(size_t n, int bs = 256) {
 namespace mot {
 
 void launch_history32(mot_handle* h, const TaskList& tl, const float* tiles, const float* ring, const float* win,
-                      const float* kry, int mode, long long step_i, double* out_s1, double* out_s2,
-                      cudaStream_t s) {
+                      const float* kry, int mode, long long step_i, const double* rho1, const double* rho2,
+                      double* out_s1, double* out_s2, cudaStream_t s) {
     const int C2 = 2 * h->B;
     if (tl.nchunks > 0) {
         const bool timed = h->opt.timing && mode == 0 && h->ev0 && step_i > h->K;
@@ -416,7 +416,7 @@ void launch_history32(mot_handle* h, const TaskList& tl, const float* tiles, con
         }
         h->launches++;
     }
-    launch_history_reduce(h, tl, C2, out_s1, out_s2, s);
+    launch_history_reduce(h, tl, C2, rho1, rho2, out_s1, out_s2, s);
 }
 
 double* split_workspace(mot_handle* h, size_t bytes) {

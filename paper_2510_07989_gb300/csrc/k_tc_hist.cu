@@ -134,6 +134,17 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16& a, __nv_bfloat16&
     c = __float2bfloat16_rn(r2);
 }
 
+// the same of an FP64 value: split in FP32 (exact differences), the value's
+// rounding to FP32 added to the last slice. Four operations of the
+// double-precision unit, which does two per clock and SM.
+__device__ __forceinline__ void split3d(double x, __nv_bfloat16& a, __nv_bfloat16& b, __nv_bfloat16& c) {
+    const float f = (float)x, rem = (float)(x - (double)f);
+    a = __float2bfloat16_rn(f);
+    const float r1 = f - __bfloat162float(a);
+    b = __float2bfloat16_rn(r1);
+    c = __float2bfloat16_rn((r1 - __bfloat162float(b)) + rem);
+}
+
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
     return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
@@ -601,35 +612,46 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     }
 }
 
-// src: npanels panels of n doubles; dst: npanels x 3 bf16 slices of n values.
-// Blocked (bulk-form) panels: n = npad x 2B values per panel become three
-// slices of npad x 128 bf16 each, in 32-row blocks of blk_elem layout (the
-// first B columns of a row in the first half, the next B in the second; the
-// other columns stay as allocated, zero).
-__global__ void k_split3(size_t n, int npanels, int C2, int blocked, const double* __restrict__ src,
-                         __nv_bfloat16* __restrict__ dst) {
-    const size_t total = n * (size_t)npanels;
-    const size_t ns = blocked ? n / C2 * 128 : n;  // elements of one slice
-    const int B = C2 / 2;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t p = i / n, r = i - p * n;
-        const double x = src[i];
-        const __nv_bfloat16 a = __double2bfloat16(x);
-        const double r1 = x - (double)__bfloat162float(a);
-        const __nv_bfloat16 b = __double2bfloat16(r1);
-        const double r2 = r1 - (double)__bfloat162float(b);
-        const __nv_bfloat16 c = __double2bfloat16(r2);
-        size_t e = r;
-        if (blocked) {
-            const size_t row = r / C2;
-            const int m = (int)(r - row * C2);
-            const int mm = m < B ? m : 64 + m - B;
-            e = (row >> 5) * (T * 128) + blk_elem((int)(row & 31), mm);
+// Windowed sums of the K~ tail straight to their bf16 slices, two columns a
+// thread: W_a = sum_{k=a}^{kmax-1} of the loop part's [-v, u] panel of step i-k
+// (steps >= 1), a = 1 .. amax, into dst [a][3 slices][npad][2B] or, in the bulk
+// form, [a][3][npad x 128] in 32-row blocks of blk_elem layout (the first B
+// columns of a row in the first half, the next B in the second; the other
+// columns stay as allocated, zero). Bound by the ring's FP64 panels (read once)
+// and the slices written; through FP64 sums in memory it was two kernels and
+// three times the bytes (117 us at 924 edges, 52 windows, B = 64).
+__global__ void __launch_bounds__(128) k_window_split(int npad, int B, int kmax, int amax, long long step_i, int R,
+                                                      int blocked, const double* __restrict__ ring,
+                                                      __nv_bfloat16* __restrict__ dst) {
+    const int C2 = 2 * B;
+    const size_t ps = (size_t)npad * C2, ns = blocked ? (size_t)npad * 128 : ps;
+    const size_t i = 2 * (blockIdx.x * (size_t)128 + threadIdx.x);
+    if (i >= ps) return;
+    size_t e = i;
+    if (blocked) {
+        const size_t row = i / C2;
+        const int m = (int)(i - row * C2);
+        e = (row >> 5) * (T * 128) + blk_elem((int)(row & 31), m < B ? m : 64 + m - B);
+    }
+    double2 acc = make_double2(0.0, 0.0);
+    const int slot_i = (int)(step_i % R);
+#pragma unroll 4
+    for (int k = kmax - 1; k >= 1; k--) {
+        if (step_i - k >= 1) {
+            const int slot = slot_i - k + (slot_i < k ? R : 0);
+            const double2 v = *reinterpret_cast<const double2*>(ring + ((size_t)slot * 6 + 2) * ps + i);
+            acc.x += v.x;
+            acc.y += v.y;
         }
-        __nv_bfloat16* d = dst + p * 3 * ns + e;
-        d[0] = a;
-        d[ns] = b;
-        d[2 * ns] = c;
+        if (k <= amax) {
+            __nv_bfloat16 x0, x1, x2, y0, y1, y2;
+            split3d(acc.x, x0, x1, x2);
+            split3d(acc.y, y0, y1, y2);
+            uint32_t* d = reinterpret_cast<uint32_t*>(dst + (size_t)k * 3 * ns + e);
+            d[0] = pack2(x0, y0);
+            d[ns / 2] = pack2(x1, y1);
+            d[ns] = pack2(x2, y2);
+        }
     }
 }
 
@@ -671,34 +693,34 @@ __global__ void k_split_ring(int npad, int B, int blocked, const double* __restr
         const int m = (int)(i - part * ps - r * C2);
         const double* v2 = ring_slot + ((size_t)part * 3 + 2) * ps + r * C2;  // [-v, u]
         const double x = m < B ? v2[B + m] : -v2[m - B];
-        const __nv_bfloat16 a = __double2bfloat16(x);
-        const double r1 = x - (double)__bfloat162float(a);
-        const __nv_bfloat16 b = __double2bfloat16(r1);
-        const double r2 = r1 - (double)__bfloat162float(b);
+        __nv_bfloat16 a, b, c;
+        split3d(x, a, b, c);
         const size_t e = blocked ? (r >> 5) * (T * 128) + blk_elem((int)(r & 31), m < B ? m : 64 + m - B) : r * C2 + m;
         __nv_bfloat16* d = dst + (size_t)part * 3 * ds + e;
         d[0] = a;
         d[ds] = b;
-        d[2 * ds] = __double2bfloat16(r2);
+        d[2 * ds] = c;
     }
 }
 
 // s1, s2 of row block rb = sum of the partial results of its chunks, in the
-// order of the row block's chunk list. One thread per output, eight chunks'
+// order of the row block's chunk list; with rho, rho - that sum. One thread per output, eight chunks'
 // loads in flight: with one CTA per row block the sum of 36 row blocks' chunks
 // (B = 64) took 220 us.
 __global__ void __launch_bounds__(256) k_hist_reduce_idx(const int* __restrict__ rb_ptr,
                                                          const int* __restrict__ rb_chunks,
                                                          const double* __restrict__ partial, int C2,
-                                                         double* __restrict__ s1, double* __restrict__ s2) {
+                                                         const double* __restrict__ rho1,
+                                                         const double* __restrict__ rho2, double* __restrict__ s1, double* __restrict__ s2) {
     const int rb = blockIdx.y, nout = T * C2, o = blockIdx.x * 256 + threadIdx.x;  // o over both targets
     if (o >= 2 * nout) return;
     const int c0 = rb_ptr[rb], c1 = rb_ptr[rb + 1];
     double a = 0.0;
 #pragma unroll 8
     for (int ci = c0; ci < c1; ci++) a += partial[(size_t)rb_chunks[ci] * 2 * nout + o];
-    double* dst = o < nout ? s1 + (size_t)rb * nout + o : s2 + (size_t)rb * nout + o - nout;
-    *dst = a;
+    const size_t ix = (size_t)rb * nout + (o < nout ? o : o - nout);
+    if (rho1) a = (o < nout ? rho1 : rho2)[ix] - a;
+    (o < nout ? s1 : s2)[ix] = a;
 }
 
 }  // namespace
@@ -756,12 +778,12 @@ int history_tc_stages(int npad, bool bulk, int cap) {
 
 bool history_tc_fits(int npad, bool bulk) { return history_tc_stages(npad, bulk, MOT_TC_CHUNK) > 0; }
 
-void launch_split3(mot_handle* h, int npanels, const double* src, uint16_t* dst, cudaStream_t s) {
-    const size_t n = (size_t)h->npad * 2 * h->B;
-    const size_t total = n * (size_t)npanels;
-    if (total == 0) return;
-    const int blocks = (int)std::min<size_t>((total + 255) / 256, 152 * 16);
-    k_split3<<<blocks, 256, 0, s>>>(n, npanels, 2 * h->B, h->tc_bulk ? 1 : 0, src, reinterpret_cast<__nv_bfloat16*>(dst));
+void launch_window_split(mot_handle* h, long long i, cudaStream_t s) {
+    if (h->max_tail_lag < 1) return;
+    const size_t n = (size_t)h->npad * h->B;  // pairs of columns
+    k_window_split<<<(int)((n + 127) / 128), 128, 0, s>>>(h->npad, h->B, h->kmax, h->max_tail_lag, i, h->R,
+                                                          h->tc_bulk ? 1 : 0, h->d_ring,
+                                                          reinterpret_cast<__nv_bfloat16*>(h->d_win16));
     h->launches++;
 }
 
@@ -840,8 +862,8 @@ void launch_jobs(mot_handle* h0, TcJobs& jobs, int nctas, int max_npad, int cap,
 
 }  // namespace
 
-void launch_history_tc(mot_handle* h, const TaskList& tl, long long step_i, double* out_s1, double* out_s2,
-                       cudaStream_t s) {
+void launch_history_tc(mot_handle* h, const TaskList& tl, long long step_i, const double* rho1, const double* rho2,
+                       double* out_s1, double* out_s2, cudaStream_t s) {
     const int C2 = 2 * h->B;
     if (tl.nchunks > 0) {
         const bool timed = h->opt.timing && h->ev0 && step_i > h->K;
@@ -860,16 +882,16 @@ void launch_history_tc(mot_handle* h, const TaskList& tl, long long step_i, doub
         }
     }
     k_hist_reduce_idx<<<dim3((2 * T * C2 + 255) / 256, h->nrb), 256, 0, s>>>(tl.rb_ptr, tl.rb_chunks, h->d_partial, C2,
-                                                                             out_s1, out_s2);
+                                                                             rho1, rho2, out_s1, out_s2);
     h->launches++;
 }
 
 // The history of n scatterers (all on the tensor-core path, one form) in one
 // launch of the history kernel: step i of handle k is hs[k]->step + 1; the
-// chunk sums of every handle are then reduced into s1[k], s2[k]. All on
-// stream s. Returns the launch's duration in ms when `timed` (events on s).
-float launch_history_tc_many(mot_handle* const* hs, int n, double* const* s1, double* const* s2, cudaStream_t s,
-                             bool timed) {
+// chunk sums of every handle are then reduced into s1[k], s2[k] (with rho:
+// subtracted from rho1[k], rho2[k]). All on stream s. Returns the launch's duration in ms when `timed` (events on s).
+float launch_history_tc_many(mot_handle* const* hs, int n, const double* const* rho1, const double* const* rho2,
+                             double* const* s1, double* const* s2, cudaStream_t s, bool timed) {
     TcJobs jobs;
     jobs.njobs = n;
     int nctas = 0, max_npad = 0, cap = 1;
@@ -895,7 +917,8 @@ float launch_history_tc_many(mot_handle* const* hs, int n, double* const* s1, do
     for (int k = 0; k < n; k++) {
         mot_handle* h = hs[k];
         k_hist_reduce_idx<<<dim3((4 * T * h->B + 255) / 256, h->nrb), 256, 0, s>>>(
-            h->hist_tc_list.rb_ptr, h->hist_tc_list.rb_chunks, h->d_partial, 2 * h->B, s1[k], s2[k]);
+            h->hist_tc_list.rb_ptr, h->hist_tc_list.rb_chunks, h->d_partial, 2 * h->B,
+            rho1 ? rho1[k] : nullptr, rho2 ? rho2[k] : nullptr, s1[k], s2[k]);
         h->launches++;
     }
     float ms = 0.f;

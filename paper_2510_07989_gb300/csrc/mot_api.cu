@@ -12,6 +12,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <cstdio>
 #include <cstdlib>
 #include <map>
@@ -61,7 +62,8 @@ void* dalloc(mot_handle* h, size_t bytes) {
 
 // mixed-precision kernels (k_mixed.cu)
 void launch_history32(mot_handle* h, const TaskList& tl, const float* tiles, const float* ring, const float* win,
-                      const float* kry, int mode, long long step_i, double* out_s1, double* out_s2, cudaStream_t s);
+                      const float* kry, int mode, long long step_i, const double* rho1, const double* rho2,
+                      double* out_s1, double* out_s2, cudaStream_t s);
 void launch_sgemm_d(mot_handle* h, int M, int N, int K, const float* A, const float* X, double* Y, cudaStream_t s);
 void launch_d2f(mot_handle* h, size_t n, const double* x, float* y, cudaStream_t s);
 void launch_unit_cols(mot_handle* h, long long J0, long long Jend, double* X, cudaStream_t s);
@@ -347,7 +349,7 @@ void apply_q0(mot_handle* h, const Work& W, const double* v, double* out, cudaSt
     launch_axpby(h, n, 1.0, v, -1.0, W.sig, W.ell, s);
     launch_variants(h, W.ell, W.kry, h->eta, h->etap, s);
     launch_variants(h, W.sig, W.kry + 3 * bv, h->eta, h->etap, s);
-    launch_history(h, h->lag0, h->d_tiles, nullptr, nullptr, W.kry, 1, 0, W.y1, W.y2, s);
+    launch_history(h, h->lag0, h->d_tiles, nullptr, nullptr, W.kry, 1, 0, nullptr, nullptr, W.y1, W.y2, s);
     left_factor(h, W, W.y1, W.y2, out, s);
 }
 
@@ -436,7 +438,7 @@ int ensure_state(mot_handle* h, int B) {
     h->gm_m = std::min(std::max(h->opt.gmres_maxit, 1), 100);
     h->d_waves = (double*)dalloc(h, sizeof(double) * 10 * B);
     h->d_ring = (double*)dalloc(h, sizeof(double) * (size_t)h->R * 6 * bv);
-    h->d_win = (double*)dalloc(h, sizeof(double) * (size_t)(h->max_tail_lag + 1) * bv);
+    h->d_ptfield = (double*)dalloc(h, sizeof(double) * 2 * (size_t)h->npts * B);
     h->d_cur = (double*)dalloc(h, sizeof(double) * 4 * (size_t)h->npad * B);
     if (h->opt.precision == MOT_PREC_MIXED && !h->precomputing) {
         int major = 0;
@@ -464,6 +466,10 @@ int ensure_state(mot_handle* h, int B) {
         h->d_xf = (float*)dalloc(h, sizeof(float) * 2 * bv);
         if (!h->d_xf) return fail(h, MOT_EOOM, "device allocation of the march state");
     }
+    if (!h->hist_tc) {
+        h->d_win = (double*)dalloc(h, sizeof(double) * (size_t)(h->max_tail_lag + 1) * bv);
+        if (!h->d_win) return fail(h, MOT_EOOM, "device allocation of the march state");
+    }
     h->d_wprev1 = (double*)dalloc(h, sizeof(double) * bv);
     h->d_wprev2 = (double*)dalloc(h, sizeof(double) * bv);
     if (!h->d_wprev1 || !h->d_wprev2) return fail(h, MOT_EOOM, "device allocation of the march state");
@@ -488,7 +494,7 @@ int ensure_state(mot_handle* h, int B) {
     h->d_gm_jend = h->d_gm_active + B;
     h->d_gm_bnorm = (double*)dalloc(h, sizeof(double) * B);
     h->d_wscale = (double*)dalloc(h, sizeof(double) * B);
-    if (!h->d_waves || !h->d_ring || !h->d_win || !h->d_cur || !h->d_dft || !h->d_work || !h->d_partial ||
+    if (!h->d_waves || !h->d_ring || !h->d_ptfield || !h->d_cur || !h->d_dft || !h->d_work || !h->d_partial ||
         !h->d_V || !h->d_H || !h->d_g || !h->d_cs || !h->d_sn || !h->d_resid || !h->d_gm_bnorm || !h->d_wscale)
         return fail(h, MOT_EOOM, "device allocation of the march state");
     h->h_waves.assign(10 * B, NAN);
@@ -496,7 +502,7 @@ int ensure_state(mot_handle* h, int B) {
 }
 
 void free_state(mot_handle* h) {
-    void* ptrs[] = {h->d_waves, h->d_ring, h->d_win, h->d_cur, h->d_dft, h->d_work, h->d_partial, h->d_V, h->d_H,
+    void* ptrs[] = {h->d_waves, h->d_ring, h->d_win, h->d_ptfield, h->d_cur, h->d_dft, h->d_work, h->d_partial, h->d_V, h->d_H,
                     h->d_g, h->d_cs, h->d_sn, h->d_Z, h->d_resid, h->d_gm_bnorm, h->d_wscale,
                     h->d_wprev1, h->d_wprev2};
     for (void* p : ptrs)
@@ -508,7 +514,7 @@ void free_state(mot_handle* h) {
     h->d_ring32 = h->d_win32 = h->d_xf = nullptr;
     h->d_ring16 = h->d_win16 = nullptr;
     h->hist_tc = false;
-    h->d_waves = h->d_ring = h->d_win = h->d_cur = h->d_dft = h->d_work = h->d_partial = nullptr;
+    h->d_waves = h->d_ring = h->d_win = h->d_ptfield = h->d_cur = h->d_dft = h->d_work = h->d_partial = nullptr;
     h->d_V = h->d_H = h->d_g = h->d_cs = h->d_sn = h->d_Z = h->d_resid = nullptr;
     h->d_gm_active = h->d_gm_jend = nullptr;
     h->d_gm_bnorm = nullptr;
@@ -554,7 +560,7 @@ bool is_device_ptr(const void* p) {
 
 // One MOT step in three phases (a full step runs all of them on one stream):
 //   STEP_INPUTS   right-hand side, windowed sums of the K~ tail, reduced-precision panels
-//   STEP_HISTORY  the history contraction into W.s1, W.s2
+//   STEP_HISTORY  the history contraction, subtracted from the right-hand side: W.y1, W.y2
 //   STEP_SOLVE    combine, left factor, Q_0 solve, ring update, recovery
 // mot_run_many runs the history of several scatterers as one launch between
 // their STEP_INPUTS and STEP_SOLVE phases.
@@ -575,11 +581,11 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
         launch_rhs(h, i, W.rho1, W.rho2, s);
         PEV(1);
         if (i >= 2) {
-            launch_window_sums(h, i, s);
             if (h->hist_tc) {
-                if (h->max_tail_lag >= 1) launch_split3(h, h->max_tail_lag + 1, h->d_win, h->d_win16, s);
-            } else if (h32) {
-                if (h->max_tail_lag >= 1)
+                launch_window_split(h, i, s);
+            } else {
+                launch_window_sums(h, i, s);
+                if (h32 && h->max_tail_lag >= 1)
                     launch_d2f(h, (size_t)(h->max_tail_lag + 1) * bv, h->d_win, h->d_win32, s);
             }
         }
@@ -588,17 +594,15 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
         if (h->hist_tc && !(h->hist_tc_list.packed && h->hist_tc_list.rb_ptr && h->hist_tc_list.rb_chunks))
             return fail(h, MOT_ESTATE, "tensor-core history: no task list (a re-cut of the list failed)");
         if (h->hist_tc)
-            launch_history_tc(h, h->hist_tc_list, i, W.s1, W.s2, s);
+            launch_history_tc(h, h->hist_tc_list, i, W.rho1, W.rho2, W.y1, W.y2, s);
         else if (h32)
-            launch_history32(h, h->hist, h->d_tiles32, h->d_ring32, h->d_win32, nullptr, 0, i, W.s1, W.s2, s);
+            launch_history32(h, h->hist, h->d_tiles32, h->d_ring32, h->d_win32, nullptr, 0, i, W.rho1, W.rho2, W.y1,
+                             W.y2, s);
         else
-            launch_history(h, h->hist, h->d_tiles, h->d_ring, h->d_win, nullptr, 0, i, W.s1, W.s2, s);
+            launch_history(h, h->hist, h->d_tiles, h->d_ring, h->d_win, nullptr, 0, i, W.rho1, W.rho2, W.y1, W.y2, s);
     }
     if (!(phases & STEP_SOLVE)) return MOT_OK;
-    if (i >= 2) {
-        launch_axpby(h, n, 1.0, W.rho1, -1.0, W.s1, W.y1, s);
-        launch_axpby(h, n, 1.0, W.rho2, -1.0, W.s2, W.y2, s);
-    } else {
+    if (i < 2) {  // else the history left y1, y2 = rho1 - s1, rho2 - s2
         launch_axpby(h, n, 1.0, W.rho1, 0.0, nullptr, W.y1, s);
         launch_axpby(h, n, 1.0, W.rho2, 0.0, nullptr, W.y2, s);
     }
@@ -1676,6 +1680,24 @@ MOT_API int mot_load_operators(mot_handle* h, const mot_operators* ops) {
             if (!std::isfinite(x[d + i]) || !std::isfinite(wf[d + i])) return fail(h, MOT_EINVAL, "non-finite RHS table");
         }
     }
+    // the distinct points of the table, by their exact coordinates
+    std::vector<double> pts;
+    std::vector<int> ptidx((size_t)np * h->nq, 0);
+    {
+        std::map<std::array<double, 3>, int> seen;
+        for (size_t e = 0; e < (size_t)ne * h->nq; e++) {
+            const std::array<double, 3> k = {x[3 * e], x[3 * e + 1], x[3 * e + 2]};
+            const auto it = seen.emplace(k, (int)seen.size());
+            if (it.second) pts.insert(pts.end(), k.begin(), k.end());
+            ptidx[e] = it.first->second;
+        }
+    }
+    h->npts = (int)(pts.size() / 3);
+    h->d_pts = (double*)dalloc(h, sizeof(double) * pts.size());
+    h->d_ptidx = (int*)dalloc(h, sizeof(int) * ptidx.size());
+    if (!h->d_pts || !h->d_ptidx) return fail(h, MOT_EOOM, "device allocation (RHS points)");
+    CK(cudaMemcpy(h->d_pts, pts.data(), sizeof(double) * pts.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_ptidx, ptidx.data(), sizeof(int) * ptidx.size(), cudaMemcpyHostToDevice));
     h->d_rhs_x = (double*)dalloc(h, sizeof(double) * x.size());
     h->d_rhs_wf = (double*)dalloc(h, sizeof(double) * wf.size());
     if (!h->d_rhs_x || !h->d_rhs_wf) return fail(h, MOT_EOOM, "device allocation (RHS table)");
@@ -1850,9 +1872,10 @@ int tune_tc(mot_handle* const* hs, int n, cudaStream_t s) {
                         hs[k]->tc_tps = tp;
                         hs[k]->tc_epi = epi;
                     }
-                    launch_history_tc_many(hs, n, s1.data(), s2.data(), s, false);
+                    launch_history_tc_many(hs, n, nullptr, nullptr, s1.data(), s2.data(), s, false);
                     float t[3];
-                    for (int r = 0; r < 3; r++) t[r] = launch_history_tc_many(hs, n, s1.data(), s2.data(), s, true);
+                    for (int r = 0; r < 3; r++)
+                        t[r] = launch_history_tc_many(hs, n, nullptr, nullptr, s1.data(), s2.data(), s, true);
                     std::sort(t, t + 3);
                     if (cudaGetLastError() != cudaSuccess)
                         return fail(hs[0], MOT_ECUDA, "mot_tune: trial launch failed");
@@ -1985,7 +2008,8 @@ MOT_API int mot_run_many(mot_handle* const* hs, int n, int n_steps, const mot_wa
     // the group's history of the coming step, by the first member's thread
     auto group_history = [&]() {
         std::vector<mot_handle*> hm;
-        std::vector<double*> s1, s2;
+        std::vector<double*> y1, y2;
+        std::vector<const double*> rho1, rho2;
         bool full = true;
         for (int g = 0; g < ng; g++) {
             mot_handle* h = hs[group[g]];
@@ -1993,8 +2017,10 @@ MOT_API int mot_run_many(mot_handle* const* hs, int n, int n_steps, const mot_wa
             cudaStreamWaitEvent(gs, ev_in[g], 0);
             Work W = work_of(h);
             hm.push_back(h);
-            s1.push_back(W.s1);
-            s2.push_back(W.s2);
+            y1.push_back(W.y1);
+            y2.push_back(W.y2);
+            rho1.push_back(W.rho1);
+            rho2.push_back(W.rho2);
             full = full && h->step + 1 > h->K;
         }
         if (!hm.empty()) {
@@ -2006,7 +2032,8 @@ MOT_API int mot_run_many(mot_handle* const* hs, int n, int n_steps, const mot_wa
                 if (t != MOT_OK) group_status = t;
             }
             const bool timed = full && hm[0]->opt.timing;
-            const float ms = launch_history_tc_many(hm.data(), (int)hm.size(), s1.data(), s2.data(), gs, timed);
+            const float ms = launch_history_tc_many(hm.data(), (int)hm.size(), rho1.data(), rho2.data(), y1.data(),
+                                                    y2.data(), gs, timed);
             if (timed)
                 for (mot_handle* h : hm) {
                     h->timed_ms += ms;
@@ -2286,7 +2313,7 @@ MOT_API void mot_destroy(mot_handle* h) {
     void* ptrs[] = {h->d_edge_faces, h->d_edge_verts, h->d_face_edges, h->d_face_sgn, h->d_iperm, h->d_cg_iters,
                     h->vtx_edges.rowptr, h->vtx_edges.col, h->vtx_edges.val, h->Lf.rowptr, h->Lf.col, h->Lf.val,
                     h->Lv.rowptr, h->Lv.col, h->Lv.val, h->G.rowptr, h->G.col, h->G.val, h->Gt.rowptr,
-                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_x, h->d_rhs_wf, h->d_tiles, h->d_tmask,
+                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_x, h->d_rhs_wf, h->d_pts, h->d_ptidx, h->d_tiles, h->d_tmask,
                     h->hist.tasks, h->hist.chunks, h->hist.chunk_ptr, h->lag0.tasks, h->lag0.chunks,
                     h->lag0.chunk_ptr, h->d_omega, h->d_colidx, h->d_tiles32, h->d_Q0, h->d_Q0f, h->d_LF,
                     h->d_LFf, h->d_Minvf, h->d_Minv64, h->d_Lfinvf, h->d_Lvinvf, h->d_Ginvf, h->hist_tc_list.packed, h->hist_tc_list.chunks,

@@ -103,6 +103,10 @@ struct mot_handle {
     int nq = 0;
     double* d_rhs_x = nullptr;     // [npad][nq][3]
     double* d_rhs_wf = nullptr;
+    int npts = 0;                  // distinct quadrature points (edges share their triangles')
+    double* d_pts = nullptr;       // [npts][3]
+    int* d_ptidx = nullptr;        // [npad][nq] point of every entry of the table
+    double* d_ptfield = nullptr;   // [npts][2][B] incident field integrals of the step
 
     // block-sparse history
     double* d_tiles = nullptr;     // FP64 tiles (mixed path: lag 0 only, compact numbering, until set-up ends)
@@ -252,19 +256,21 @@ double* split_workspace(mot_handle* h, size_t bytes);
 
 // history
 void launch_history(mot_handle* h, const TaskList& tl, const double* tiles, const double* ring, const double* win,
-                    const double* kry, int mode, long long step_i, double* out_s1, double* out_s2, cudaStream_t s);
+                    const double* kry, int mode, long long step_i, const double* rho1, const double* rho2,
+                    double* out_s1, double* out_s2, cudaStream_t s);
 
 // nonzero masks of ntiles FP64 tiles (k_hist_f64)
 void launch_tile_masks(mot_handle* h, int64_t ntiles, const double* tiles, uint32_t* masks, cudaStream_t s);
 
 // tensor-core history (mixed path, B a multiple of 8): tiles from d_tiles16, panels from d_ring16/d_win16
-void launch_history_tc(mot_handle* h, const TaskList& tl, long long step_i, double* out_s1, double* out_s2,
-                       cudaStream_t s);
-// sum of the chunk partial results of a history launch into out_s1 / out_s2
-void launch_history_reduce(mot_handle* h, const TaskList& tl, int C2, double* out_s1, double* out_s2,
-                           cudaStream_t s);
-// npanels FP64 panels of npad x 2B values -> three bf16 slices each
-void launch_split3(mot_handle* h, int npanels, const double* src, uint16_t* dst, cudaStream_t s);
+void launch_history_tc(mot_handle* h, const TaskList& tl, long long step_i, const double* rho1, const double* rho2,
+                       double* out_s1, double* out_s2, cudaStream_t s);
+// sum of the chunk partial results of a history launch into out_s1 / out_s2 (rho1, rho2
+// not null: subtracted from them)
+void launch_history_reduce(mot_handle* h, const TaskList& tl, int C2, const double* rho1, const double* rho2,
+                           double* out_s1, double* out_s2, cudaStream_t s);
+// windowed sums of the K~ tail of step i as bf16 slices (d_win16)
+void launch_window_split(mot_handle* h, long long i, cudaStream_t s);
 // bf16 slices of the FP32 tiles in the tensor core's B layout (d_tiles32 -> d_tiles16)
 void launch_split_tiles(mot_handle* h, cudaStream_t s);
 // bf16 slices of l and s of ring slot `slot` (from the FP64 ring's [-v, u] variant)
@@ -274,8 +280,8 @@ size_t history_tc_ring_slot_elems(const mot_handle* h);  // bf16 elements of one
 int history_tc_stages(int npad, bool bulk, int cap);
 // whether (ns stages of tp tasks) fits the kernel's shared memory with cap staged tasks
 bool history_tc_config_fits(int npad, bool bulk, int cap, int ns, int tp);
-float launch_history_tc_many(mot_handle* const* hs, int n, double* const* s1, double* const* s2, cudaStream_t s,
-                             bool timed);
+float launch_history_tc_many(mot_handle* const* hs, int n, const double* const* rho1, const double* const* rho2,
+                             double* const* s1, double* const* s2, cudaStream_t s, bool timed);
 
 // emulated FP64 products on tensor cores (k_emu64.cu): Y (M x N) = A X with A
 // prepared once by emu_prepare from the device FP64 matrix A (M x K, ld K)
