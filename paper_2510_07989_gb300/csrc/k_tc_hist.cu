@@ -56,14 +56,15 @@
 // thread waits once and commits once per stage, so two tasks per stage halve
 // the barrier hand-offs (NS stages: 4 or 5 of one task, 2 or 3 of two).
 //
-// Warp roles (224 threads with four epilogue warps, 352 with eight; one CTA
-// per SM):
-//   warps 0-1  gather: coefficient rows by cp.async (each lane's arrival fires
-//              on completion of its copies, so the warps never wait for them)
-//              and the tile copies
-//   warp  2    TMEM allocation; lane 0 issues the MMAs
-//   warps 3-6  epilogue (TMEM -> registers, compensated sums on packed FP32
-//   (or 3-10)  pairs, partial results)
+// Warp roles (224 threads with four epilogue warps, 512 with eight; one CTA
+// per SM; numbers with four, in brackets with eight):
+//   warps 0-1 (0-5)   gather, in pairs that take tasks in turn: coefficient rows
+//                     by cp.async (each lane's arrival fires on completion of
+//                     its copies, so the warps never wait for them)
+//   (warp 6)          tile copies (with four epilogue warps, thread 0's work)
+//   warp 2 (7)        TMEM allocation; lane 0 issues the MMAs
+//   warps 3-6 (8-15)  epilogue (TMEM -> registers, compensated sums on packed
+//                     FP32 pairs, partial results)
 // Arrivals on a barrier are shared-memory atomics on one word: the epilogue
 // warps arrive once per warp, after a warp-level sync.
 // Every mbarrier wait is bounded in time; a wait that runs out raises the
@@ -91,12 +92,20 @@ constexpr int B_SLICE = T * T * 2;          // 2048 bytes: one bf16 slice of a t
 constexpr int STAGE_A = 3 * A_SLICE;        // 24576
 constexpr int STAGE_B = 6 * B_SLICE;        // 12288: both tiles' slices, ordered X0 hi, X1 hi, X0 mid, X1 mid, X0 lo, X1 lo
 constexpr int STAGE = STAGE_A + STAGE_B;    // 36864
-constexpr int NPROD = 64;
-// threads of a CTA with EW epilogue warps: warps 0-1 gather, 2 MMA, 3 .. 2 + EW
-// epilogue (EW = 4: each warp folds both outputs of its TMEM lane quarter;
-// EW = 8: two warps per quarter, one output each)
+// Warps of a CTA with EW epilogue warps: first the pairs that gather the
+// coefficient rows, then (EW = 8) the warp that copies the tiles, the MMA warp, the
+// epilogue. EW = 8: three pairs, two epilogue warps per TMEM lane quarter, one
+// output each, sixteen warps of at most 128 registers a thread. EW = 4: one pair
+// that also copies the tiles; its epilogue warps fold both outputs of a quarter
+// and need 252 registers a thread, eight warps at most.
 template <int EW>
-__host__ __device__ constexpr int tc_threads() { return NPROD + 32 + 32 * EW; }
+struct Roles {
+    static constexpr int PAIRS = EW == 8 ? 3 : 1;
+    static constexpr int TILE_WARP = EW == 8 ? 2 * PAIRS : -1;
+    static constexpr int MMA_WARP = 2 * PAIRS + (EW == 8 ? 1 : 0);
+};
+template <int EW>
+__host__ __device__ constexpr int tc_threads() { return 32 * (Roles<EW>::MMA_WARP + 1 + EW); }
 constexpr int TC_CHUNK = MOT_TC_CHUNK;      // tasks per CTA (staged in shared memory)
 constexpr size_t TC_SMEM_MAX = 227 * 1024;
 
@@ -167,8 +176,6 @@ __device__ __forceinline__ void two_sum2(float2& s, float2& c, float2 v) {
     c = f2add(c, e);
 }
 __device__ __forceinline__ float2 pair_of(const float (&v)[32], int n) { return make_float2(v[2 * n], v[2 * n + 1]); }
-
-__device__ __forceinline__ void producer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 // Merged task of the tensor-core list: x, y = tiles of s1 and s2 (the zero
 // tile if absent), z = cb | k << 16 | (part | variant << 2) << 26.
@@ -242,6 +249,7 @@ template <int NS, bool BULK, int EW, int TP>
 __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     k_hist_tc(const __grid_constant__ TcJobs jobs, int cap, int stall_task, unsigned long long stall_bound) {
     constexpr int TC_THREADS = tc_threads<EW>();
+    constexpr int PAIRS = Roles<EW>::PAIRS, MMA_WARP = Roles<EW>::MMA_WARP, TILE_WARP = Roles<EW>::TILE_WARP;
     using L = TcLayout<NS, BULK, TP>;
     constexpr uint32_t SSTAGE = TP * STAGE;  // bytes of one pipeline stage (TP task slots of STAGE bytes)
     int jb = 0;
@@ -265,7 +273,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     const uint32_t bar0 = sbase + (uint32_t)L::BARS;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::SLOT);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    int* issued_slot = reinterpret_cast<int*>(tmem_slot + 2);  // stages whose copies the producers issued
+    int* issued_slot = reinterpret_cast<int*>(tmem_slot + 2);  // stages whose tile copies were issued
     uint4* sdesc = reinterpret_cast<uint4*>(smem + L::DESC);
     uint16_t* scol = reinterpret_cast<uint16_t*>(smem + L::DESC + 16 * (size_t)cap);
     // FULL: the coefficient rows (one arrival per copying thread, when its
@@ -293,7 +301,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     const int* __restrict__ gcol = colidx + (size_t)ch.rb * npad;  // the same order in global memory
     if (tid == 0) {
         for (int s = 0; s < NS; s++) {
-            mbar_init(FULL(s), BULK ? 1 : NPROD);
+            mbar_init(FULL(s), BULK ? 1 : PAIRS > 1 ? TP * 64 + 1 : 64);
             mbar_init(EMPTY(s), 1);
         }
         for (int b = 0; b < NB; b++) {
@@ -305,7 +313,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
         *issued_slot = 0;
         fence_barrier_init();
     }
-    if (warp == 2) {
+    if (warp == MMA_WARP) {
         tmem_alloc(su32(tmem_slot), TMEM_COLS);
         tmem_relinquish();
     }
@@ -314,7 +322,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (BULK && warp < 2) {
+    if (BULK && warp < MMA_WARP) {
         // ---------------- bulk producer: one thread moves every stage ----------------
         if (tid == 0) {
             const int slot_i = (int)(step_i % R);
@@ -365,18 +373,54 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
             // a last stage with fewer than TP tasks
             if (v > 0 && v % TP != 0 && !(stall_cta && (v - 1) / TP == stall_task)) mbar_arrive(FULL(s));
         }
-    } else if (!BULK && warp < 2) {
-        // ---------------- gather: coefficient rows and the tile copy ----------------
-        const int t = tid;
+    } else if (!BULK && warp == TILE_WARP) {
+        // ---------------- tile copies ----------------
+        if (lane == 0) {
+            int v = 0;
+            for (int ti = 0; ti < ntask; ti++) {
+                const uint4 d = sdesc[ti];
+                if (step_i - pk_k(d) < 1) continue;
+                const int j = v / TP, u = v % TP, s = j % NS;
+                v++;
+                if (u == 0) {
+                    if (!mbar_wait(EMPTY(s), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound)) {
+                        v = 0;
+                        break;
+                    }
+                    *issued_slot = j + 1;
+                }
+                if (stall_cta && j == stall_task) continue;  // failure test: this stage is never filled
+                const uint32_t bdst = sbase + s * SSTAGE + u * STAGE + STAGE_A;
+                mbar_add_tx(FULL(s), STAGE_B);  // before the stage's arrival
+#pragma unroll
+                for (int q = 0; q < 3; q++) {  // slices in the order Y0 Z0 Y1 Z1 Y2 Z2
+                    bulk_g2s(bdst + (2 * q) * B_SLICE, tiles16 + ((size_t)d.x * 3 + q) * (T * T), B_SLICE, FULL(s));
+                    bulk_g2s(bdst + (2 * q + 1) * B_SLICE, tiles16 + ((size_t)d.y * 3 + q) * (T * T), B_SLICE,
+                             FULL(s));
+                }
+                if (u == TP - 1) mbar_arrive(FULL(s));
+            }
+            // a last stage with fewer than TP tasks
+            if (v % TP != 0 && !(stall_cta && v / TP == stall_task)) mbar_arrive(FULL(v / TP % NS));
+        }
+        __syncwarp();
+    } else if (!BULK && warp < 2 * PAIRS) {
+        // ---------------- gather: coefficient rows (one pair: and the tile copies) ----------------
+        // A task is some 900 cycles of a pair's instructions, whatever it copies,
+        // so several pairs take tasks in turn; an arrival per thread and task. One
+        // pair, two and three pairs with the tile copies in a warp of their own:
+        // 2.40, 2.02 (two pairs, tiles by their first threads), 1.96 and 1.92 ms
+        // for 448 303 tasks (1512 edges, B = 64).
+        const int t = tid & 63, pair = warp >> 1, wp = warp & 1;
         const int l8 = lane & 7, l3 = lane >> 3;
         const int slot_i = (int)(step_i % R);  // ring slot of step i; lag k (< R) is slot_i - k mod R
         // this lane's 16-byte pieces: slices q = 0..2, row groups ro, column quads mq of
-        // its warp's half (mq = 2 warp + 0/1); destination offsets do not depend on the task
+        // its warp's half (mq = 2 wp + 0/1); destination offsets do not depend on the task
         uint32_t dofs[4][2];
 #pragma unroll
         for (int ro = 0; ro < 4; ro++)
 #pragma unroll
-            for (int h = 0; h < 2; h++) dofs[ro][h] = a_chunk(ro * 8 + l8, (2 * warp + h) * 4 + l3);
+            for (int h = 0; h < 2; h++) dofs[ro][h] = a_chunk(ro * 8 + l8, (2 * wp + h) * 4 + l3);
         const size_t pstride = (size_t)npad * C2;  // elements of one bf16 slice of one panel
         // 16-byte pieces per coefficient row (C2 / 8); a batch below 64 waves
         // leaves the panel's upper columns uncopied (their TMEM lanes are never
@@ -387,7 +431,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
         bool has[2];
 #pragma unroll
         for (int h = 0; h < 2; h++) {
-            const int mg = (2 * warp + h) * 4 + l3;
+            const int mg = (2 * wp + h) * 4 + l3;
             has[h] = mg < nch;
             const int sw = mg + (nch >> 1) < nch ? mg + (nch >> 1) : mg + (nch >> 1) - nch;
             soff0[h] = mg * 8;
@@ -402,16 +446,16 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
             const int j = v / TP, u = v % TP;
             s = j % NS;
             v++;
-            if (u == 0) {
-                if (!mbar_wait(EMPTY(s), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound)) {
-                    v = -1;
-                    break;
-                }
-                if (t == 0) *issued_slot = j + 1;
+            if (PAIRS > 1 && (v - 1) % PAIRS != pair) continue;
+            if ((PAIRS > 1 || u == 0) &&
+                !mbar_wait(EMPTY(s), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound)) {
+                v = -1;
+                break;
             }
+            if (PAIRS == 1 && t == 0) *issued_slot = j + 1;
             if (stall_cta && j == stall_task) continue;  // failure test: this stage is never filled
             const uint32_t adst = sbase + s * SSTAGE + u * STAGE;
-            if (t == 0) {  // slices in the order Y0 Z0 Y1 Z1 Y2 Z2; bytes added before this thread's arrival
+            if (PAIRS == 1 && t == 0) {  // slices in the order Y0 Z0 Y1 Z1 Y2 Z2; bytes added before this thread's arrival
                 mbar_add_tx(FULL(s), STAGE_B);
 #pragma unroll
                 for (int q = 0; q < 3; q++) {
@@ -438,12 +482,22 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
                 }
             }
             // this thread's arrival on the stage fires when its copies have landed
-            if (u == TP - 1) cp_async_arrive_noinc(FULL(s));
+            if (PAIRS > 1 || u == TP - 1) cp_async_arrive_noinc(FULL(s));
         }
-        // a last stage with fewer than TP tasks
-        if (v > 0 && v % TP != 0 && !(stall_cta && (v - 1) / TP == stall_task)) cp_async_arrive_noinc(FULL(s));
+        // a last stage of one task of two: the pair's arrivals, or those of the pair
+        // whose turn it would be (once the stage is free, so that they count for
+        // this use of it)
+        if (TP == 2 && v > 0 && v % 2 != 0 && v % PAIRS == pair) {
+            const int j = v / 2;
+            if (PAIRS == 1) {
+                if (!(stall_cta && j == stall_task)) cp_async_arrive_noinc(FULL(s));
+            } else if (mbar_wait(EMPTY(j % NS), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound) &&
+                       !(stall_cta && j == stall_task)) {
+                mbar_arrive(FULL(j % NS));
+            }
+        }
         cp_async_wait_all();  // this thread's row copies have landed
-    } else if (warp == 2) {
+    } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
             int v = 0, g = -1, ing = 0, cur = -1, s = 0;
@@ -497,9 +551,9 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
         const int quarter = warp & 3;  // TMEM lanes [32 quarter, 32 quarter + 32)
         const int m = quarter * 32 + lane;
         const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
-        // outputs this warp folds: both (EW = 4), or one (EW = 8: warps 3-6 s1, 7-10 s2)
+        // outputs this warp folds: both (EW = 4), or one (EW = 8: the first four s1, the others s2)
         constexpr int NO = EW == 8 ? 1 : 2;
-        const int o0 = EW == 8 ? (warp - 3) >> 2 : 0;
+        const int o0 = EW == 8 ? (warp - MMA_WARP - 1) >> 2 : 0;
         float2 hs[NO][16], hc[NO][16];  // compensated sums, tile rows 2n and 2n + 1 in a pair
 #pragma unroll
         for (int o = 0; o < NO; o++)
@@ -597,7 +651,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 2) {
+    if (warp == MMA_WARP) {
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }
