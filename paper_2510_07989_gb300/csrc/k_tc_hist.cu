@@ -56,14 +56,15 @@
 // thread waits once and commits once per stage, so two tasks per stage halve
 // the barrier hand-offs (NS stages: 4 or 5 of one task, 2 or 3 of two).
 //
-// Warp roles (224 threads with four epilogue warps, 512 with eight; one CTA
+// Warp roles (256 threads with four epilogue warps, 512 with eight; one CTA
 // per SM; numbers with four, in brackets with eight):
-//   warps 0-1 (0-5)   gather, in pairs that take tasks in turn: coefficient rows
-//                     by cp.async (each lane's arrival fires on completion of
-//                     its copies, so the warps never wait for them)
-//   (warp 6)          tile copies (with four epilogue warps, thread 0's work)
-//   warp 2 (7)        TMEM allocation; lane 0 issues the MMAs
-//   warps 3-6 (8-15)  epilogue (TMEM -> registers, compensated sums on packed
+//   warps 0-2 (0-5)   three gather workers of one (two) warps that take tasks in
+//                     turn: coefficient rows by cp.async (each lane's arrival
+//                     fires on completion of its copies, so the warps never
+//                     wait for them)
+//   (warp 6)          tile copies (with four epilogue warps, the workers' work)
+//   warp 3 (7)        TMEM allocation; lane 0 issues the MMAs
+//   warps 4-7 (8-15)  epilogue (TMEM -> registers, compensated sums on packed
 //                     FP32 pairs, partial results)
 // Arrivals on a barrier are shared-memory atomics on one word: the epilogue
 // warps arrive once per warp, after a warp-level sync.
@@ -92,17 +93,18 @@ constexpr int B_SLICE = T * T * 2;          // 2048 bytes: one bf16 slice of a t
 constexpr int STAGE_A = 3 * A_SLICE;        // 24576
 constexpr int STAGE_B = 6 * B_SLICE;        // 12288: both tiles' slices, ordered X0 hi, X1 hi, X0 mid, X1 mid, X0 lo, X1 lo
 constexpr int STAGE = STAGE_A + STAGE_B;    // 36864
-// Warps of a CTA with EW epilogue warps: first the pairs that gather the
+// Warps of a CTA with EW epilogue warps: first the three workers that gather the
 // coefficient rows, then (EW = 8) the warp that copies the tiles, the MMA warp, the
-// epilogue. EW = 8: three pairs, two epilogue warps per TMEM lane quarter, one
-// output each, sixteen warps of at most 128 registers a thread. EW = 4: one pair
-// that also copies the tiles; its epilogue warps fold both outputs of a quarter
-// and need 252 registers a thread, eight warps at most.
+// epilogue. EW = 8: two warps a worker, two epilogue warps per TMEM lane quarter,
+// one output each, sixteen warps of at most 128 registers a thread. EW = 4: one
+// warp a worker, which also copies its tasks' tiles; the epilogue warps fold both
+// outputs of a quarter and need 252 registers a thread, eight warps at most.
 template <int EW>
 struct Roles {
-    static constexpr int PAIRS = EW == 8 ? 3 : 1;
-    static constexpr int TILE_WARP = EW == 8 ? 2 * PAIRS : -1;
-    static constexpr int MMA_WARP = 2 * PAIRS + (EW == 8 ? 1 : 0);
+    static constexpr int WORKERS = 3;
+    static constexpr int WW = EW == 8 ? 2 : 1;  // warps per worker
+    static constexpr int TILE_WARP = EW == 8 ? WORKERS * WW : -1;
+    static constexpr int MMA_WARP = WORKERS * WW + (EW == 8 ? 1 : 0);
 };
 template <int EW>
 __host__ __device__ constexpr int tc_threads() { return 32 * (Roles<EW>::MMA_WARP + 1 + EW); }
@@ -249,7 +251,8 @@ template <int NS, bool BULK, int EW, int TP>
 __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     k_hist_tc(const __grid_constant__ TcJobs jobs, int cap, int stall_task, unsigned long long stall_bound) {
     constexpr int TC_THREADS = tc_threads<EW>();
-    constexpr int PAIRS = Roles<EW>::PAIRS, MMA_WARP = Roles<EW>::MMA_WARP, TILE_WARP = Roles<EW>::TILE_WARP;
+    constexpr int WORKERS = Roles<EW>::WORKERS, WW = Roles<EW>::WW, MMA_WARP = Roles<EW>::MMA_WARP,
+                  TILE_WARP = Roles<EW>::TILE_WARP;
     using L = TcLayout<NS, BULK, TP>;
     constexpr uint32_t SSTAGE = TP * STAGE;  // bytes of one pipeline stage (TP task slots of STAGE bytes)
     int jb = 0;
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
     const int* __restrict__ gcol = colidx + (size_t)ch.rb * npad;  // the same order in global memory
     if (tid == 0) {
         for (int s = 0; s < NS; s++) {
-            mbar_init(FULL(s), BULK ? 1 : PAIRS > 1 ? TP * 64 + 1 : 64);
+            mbar_init(FULL(s), BULK ? 1 : TP * WW * 32 + (TILE_WARP >= 0 ? 1 : 0));
             mbar_init(EMPTY(s), 1);
         }
         for (int b = 0; b < NB; b++) {
@@ -404,34 +407,34 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
             if (v % TP != 0 && !(stall_cta && v / TP == stall_task)) mbar_arrive(FULL(v / TP % NS));
         }
         __syncwarp();
-    } else if (!BULK && warp < 2 * PAIRS) {
-        // ---------------- gather: coefficient rows (one pair: and the tile copies) ----------------
-        // A task is some 900 cycles of a pair's instructions, whatever it copies,
-        // so several pairs take tasks in turn; an arrival per thread and task. One
-        // pair, two and three pairs with the tile copies in a warp of their own:
-        // 2.40, 2.02 (two pairs, tiles by their first threads), 1.96 and 1.92 ms
-        // for 448 303 tasks (1512 edges, B = 64).
-        const int t = tid & 63, pair = warp >> 1, wp = warp & 1;
+    } else if (!BULK && warp < WORKERS * WW) {
+        // ---------------- gather: coefficient rows (and, without a tile warp, the tiles) ----------------
+        // A task is some 900 cycles of a pair of warps, whatever it copies, so
+        // three workers take tasks in turn; an arrival per thread and task. For
+        // 448 303 tasks (1512 edges, B = 64), EW = 8: one pair 2.40 ms, two 2.02,
+        // three with the tile copies in a warp of their own 1.92.
+        const int worker = warp / WW, wp = warp % WW, t = wp * 32 + lane;
+        constexpr int NH = 4 / WW;  // column quads of a lane: mq = NH wp + 0 ..
         const int l8 = lane & 7, l3 = lane >> 3;
         const int slot_i = (int)(step_i % R);  // ring slot of step i; lag k (< R) is slot_i - k mod R
         // this lane's 16-byte pieces: slices q = 0..2, row groups ro, column quads mq of
-        // its warp's half (mq = 2 wp + 0/1); destination offsets do not depend on the task
-        uint32_t dofs[4][2];
+        // its warp; destination offsets do not depend on the task
+        uint32_t dofs[4][NH];
 #pragma unroll
         for (int ro = 0; ro < 4; ro++)
 #pragma unroll
-            for (int h = 0; h < 2; h++) dofs[ro][h] = a_chunk(ro * 8 + l8, (2 * wp + h) * 4 + l3);
+            for (int h = 0; h < NH; h++) dofs[ro][h] = a_chunk(ro * 8 + l8, (NH * wp + h) * 4 + l3);
         const size_t pstride = (size_t)npad * C2;  // elements of one bf16 slice of one panel
         // 16-byte pieces per coefficient row (C2 / 8); a batch below 64 waves
         // leaves the panel's upper columns uncopied (their TMEM lanes are never
         // read). Source offsets of this lane's two pieces, as stored and with
         // the u and v halves exchanged ([-v, u]), fixed for the whole chunk.
         const int nch = C2 >> 3;
-        int soff0[2], soff1[2];
-        bool has[2];
+        int soff0[NH], soff1[NH];
+        bool has[NH];
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int mg = (2 * wp + h) * 4 + l3;
+        for (int h = 0; h < NH; h++) {
+            const int mg = (NH * wp + h) * 4 + l3;
             has[h] = mg < nch;
             const int sw = mg + (nch >> 1) < nch ? mg + (nch >> 1) : mg + (nch >> 1) - nch;
             soff0[h] = mg * 8;
@@ -446,16 +449,15 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
             const int j = v / TP, u = v % TP;
             s = j % NS;
             v++;
-            if (PAIRS > 1 && (v - 1) % PAIRS != pair) continue;
-            if ((PAIRS > 1 || u == 0) &&
-                !mbar_wait(EMPTY(s), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound)) {
+            if ((v - 1) % WORKERS != worker) continue;
+            if (!mbar_wait(EMPTY(s), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound)) {
                 v = -1;
                 break;
             }
-            if (PAIRS == 1 && t == 0) *issued_slot = j + 1;
+            if (TILE_WARP < 0 && t == 0) atomicMax(issued_slot, j + 1);
             if (stall_cta && j == stall_task) continue;  // failure test: this stage is never filled
             const uint32_t adst = sbase + s * SSTAGE + u * STAGE;
-            if (PAIRS == 1 && t == 0) {  // slices in the order Y0 Z0 Y1 Z1 Y2 Z2; bytes added before this thread's arrival
+            if (TILE_WARP < 0 && t == 0) {  // slices in the order Y0 Z0 Y1 Z1 Y2 Z2; bytes added before this thread's arrival
                 mbar_add_tx(FULL(s), STAGE_B);
 #pragma unroll
                 for (int q = 0; q < 3; q++) {
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
                 const int c = cb * T + ro * 8 + l8;
                 const __nv_bfloat16* row = pan + (size_t)(L::SCOL ? (int)scol[c] : __ldg(gcol + c)) * C2;
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
+                for (int h = 0; h < NH; h++) {
                     if (!has[h]) continue;
                     const __nv_bfloat16* src = row + (swap ? soff1[h] : soff0[h]);
 #pragma unroll
@@ -482,19 +484,15 @@ __global__ void __launch_bounds__(tc_threads<EW>(), 1)
                 }
             }
             // this thread's arrival on the stage fires when its copies have landed
-            if (PAIRS > 1 || u == TP - 1) cp_async_arrive_noinc(FULL(s));
+            cp_async_arrive_noinc(FULL(s));
         }
-        // a last stage of one task of two: the pair's arrivals, or those of the pair
-        // whose turn it would be (once the stage is free, so that they count for
-        // this use of it)
-        if (TP == 2 && v > 0 && v % 2 != 0 && v % PAIRS == pair) {
+        // a last stage of one task of two: the arrivals of the worker whose turn it
+        // would be (once the stage is free, so that they count for this use of it)
+        if (TP == 2 && v > 0 && v % 2 != 0 && v % WORKERS == worker) {
             const int j = v / 2;
-            if (PAIRS == 1) {
-                if (!(stall_cta && j == stall_task)) cp_async_arrive_noinc(FULL(s));
-            } else if (mbar_wait(EMPTY(j % NS), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound) &&
-                       !(stall_cta && j == stall_task)) {
+            if (mbar_wait(EMPTY(j % NS), ((uint32_t)(j / NS) & 1u) ^ 1u, abort_flag, err, 2, bound) &&
+                !(stall_cta && j == stall_task))
                 mbar_arrive(FULL(j % NS));
-            }
         }
         cp_async_wait_all();  // this thread's row copies have landed
     } else if (warp == MMA_WARP) {
