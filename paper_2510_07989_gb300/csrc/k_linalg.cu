@@ -6,6 +6,7 @@
 //
 // Block vectors are row-major [rows][C]: row = edge (or face / vertex),
 // column = one right-hand side component (u-part columns 0..B-1, v-part B..2B-1).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -13,6 +14,8 @@
 #include "mot_internal.h"
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 // ----------------------------------------------------------------- helpers
 __global__ void k_axpby(int n, double a, const double* __restrict__ x, double b, const double* __restrict__ y,
@@ -530,64 +533,126 @@ __global__ void k_pack_cur(int ne, int npad, int B, const int* __restrict__ iper
     }
 }
 
-// Far field E_inf(r) = (j k / 4 pi) [eta r x (r x N) + r x L] / S(w) for every
-// (direction, frequency, wave); N, L from the Fourier sums of j and m (loop and
-// star parts summed here, after separate accumulation). One CTA per output.
-__global__ void k_far_field(int ne, int npad, int B, int nq, int nfreq, int ndir, const double* __restrict__ xq,
-                            const double* __restrict__ wf, const double* __restrict__ dft,
-                            const double* __restrict__ omega, const double* __restrict__ dirs,
-                            const double* __restrict__ waves, double c, double eta, double* __restrict__ E) {
-    const int o = blockIdx.x;
-    const int d = o % ndir, f = (o / ndir) % nfreq, b = o / (ndir * nfreq);
-    const double w = omega[f], k = w / c;
-    const double rx = dirs[3 * d], ry = dirs[3 * d + 1], rz = dirs[3 * d + 2];
+// Point currents of one frequency: the Fourier sums of j and m (loop and star
+// parts summed here, after separate accumulation) times the quadrature's weight *
+// basis function, summed over the edges whose tables share the point.
+// cur[pt][12][b]: j_x re, im, j_y .., then m
+__global__ void __launch_bounds__(128) k_point_currents(int npts, int npad, int B, int nq,
+                                                        const int* __restrict__ ptr, const int* __restrict__ ent,
+                                                        const double* __restrict__ wf, const double* __restrict__ D,
+                                                        double* __restrict__ cur) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= npts * B) return;
+    const int pt = i / B, b = i - pt * B;
     const size_t nb = (size_t)npad * B;
-    const double* D = dft + (size_t)f * 4 * nb * 2;
-    double acc[12];
-    for (int j = 0; j < 12; j++) acc[j] = 0.0;
-    for (int r = threadIdx.x; r < ne; r += blockDim.x) {
-        const size_t ix = (size_t)r * B + b;
-        const double jr = D[(0 * nb + ix) * 2] + D[(1 * nb + ix) * 2];
-        const double ji = D[(0 * nb + ix) * 2 + 1] + D[(1 * nb + ix) * 2 + 1];
+    double a[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) a[k] = 0.0;
+    for (int e = ptr[pt]; e < ptr[pt + 1]; e++) {
+        const size_t ix = (size_t)(ent[e] / nq) * B + b;
+        const double jr = D[ix * 2] + D[(nb + ix) * 2], ji = D[ix * 2 + 1] + D[(nb + ix) * 2 + 1];
         const double mr = D[(2 * nb + ix) * 2] + D[(3 * nb + ix) * 2];
         const double mi = D[(2 * nb + ix) * 2 + 1] + D[(3 * nb + ix) * 2 + 1];
-        for (int q = 0; q < nq; q++) {
-            const double* x = xq + ((size_t)r * nq + q) * 3;
-            const double* fv = wf + ((size_t)r * nq + q) * 3;
-            double sp, cp;
-            sincos(k * (rx * x[0] + ry * x[1] + rz * x[2]), &sp, &cp);
-            const double ar = jr * cp - ji * sp, ai = jr * sp + ji * cp;
-            const double br = mr * cp - mi * sp, bi = mr * sp + mi * cp;
-            for (int t = 0; t < 3; t++) {
-                acc[2 * t] += ar * fv[t];
-                acc[2 * t + 1] += ai * fv[t];
-                acc[6 + 2 * t] += br * fv[t];
-                acc[6 + 2 * t + 1] += bi * fv[t];
-            }
+#pragma unroll
+        for (int t = 0; t < 3; t++) {
+            const double f = wf[(size_t)ent[e] * 3 + t];
+            a[2 * t] = fma(jr, f, a[2 * t]);
+            a[2 * t + 1] = fma(ji, f, a[2 * t + 1]);
+            a[6 + 2 * t] = fma(mr, f, a[6 + 2 * t]);
+            a[6 + 2 * t + 1] = fma(mi, f, a[6 + 2 * t + 1]);
         }
     }
-    __shared__ double red[12][256];
-    for (int j = 0; j < 12; j++) red[j][threadIdx.x] = acc[j];
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st)
-            for (int j = 0; j < 12; j++) red[j][threadIdx.x] += red[j][threadIdx.x + st];
+#pragma unroll
+    for (int k = 0; k < 12; k++) cur[((size_t)pt * 12 + k) * B + b] = a[k];
+}
+
+// Far field E_inf(r) = (j k / 4 pi) [eta r x (r x N) + r x L] / S(w) of one
+// frequency; N, L the sums of the point currents times e^{j k r.x}. Bound by
+// the FP64 units: 24 multiply-adds per point, direction and wave, and one
+// sine and cosine per point and direction, shared by the waves (and by the
+// three edges of a point's triangle; per edge and wave they were 24 times as
+// many: 2.62 ms at 480 edges, 8 waves, 3 frequencies, 181 directions). A cluster
+// of eight CTAs takes DT directions: its threads are (share of the points,
+// direction, wave), the shares are summed in shared memory and then over the
+// cluster, in order.
+constexpr int FT = 256, FCL = 8;
+__global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, int f, int ndir, int DT,
+                                                  const double* __restrict__ pts, const double* __restrict__ cur,
+                                                  const double* __restrict__ omega, const double* __restrict__ dirs,
+                                                  const double* __restrict__ waves, double c, double eta,
+                                                  double* __restrict__ E) {
+    __shared__ double2 phase[FT];
+    __shared__ double sums[FT * 12];  // shares, then this CTA's sums [12][DT * B]
+    cg::cluster_group cl = cg::this_cluster();
+    const int rk = (int)cl.block_rank(), t = threadIdx.x;
+    const int G = DT * B, nsub = FT / G, sub = t / G, l = t - sub * G, d = l / B, b = l - d * B;
+    const bool on = sub < nsub;
+    const int dir = blockIdx.x / FCL * DT + d;
+    const double w = omega[f], k = w / c;
+    double r[3] = {0, 0, 0};
+    if (on && dir < ndir)
+        for (int i = 0; i < 3; i++) r[i] = dirs[3 * dir + i];
+    double acc[12];
+#pragma unroll
+    for (int j = 0; j < 12; j++) acc[j] = 0.0;
+    // a share takes B consecutive points at a time: thread (d, b) the phase of point b
+    const int step = FCL * nsub * B;
+    for (int p0 = 0; p0 < npts; p0 += step) {
+        const int first = p0 + (rk * nsub + sub) * B, n = on ? max(0, min(B, npts - first)) : 0;
+        if (b < n) {
+            const double* x = pts + 3 * (size_t)(first + b);
+            double sn, cs;
+            sincos(k * (r[0] * x[0] + r[1] * x[1] + r[2] * x[2]), &sn, &cs);
+            phase[t] = make_double2(cs, sn);
+        }
+        __syncthreads();
+        for (int i = 0; i < n; i++) {
+            const double2 e = phase[t - b + i];
+            const double* v = cur + (size_t)(first + i) * 12 * B + b;
+#pragma unroll
+            for (int j = 0; j < 6; j++) {
+                const double re = v[(2 * j) * B], im = v[(2 * j + 1) * B];
+                acc[2 * j] = fma(re, e.x, fma(-im, e.y, acc[2 * j]));
+                acc[2 * j + 1] = fma(re, e.y, fma(im, e.x, acc[2 * j + 1]));
+            }
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const double r[3] = {rx, ry, rz};
+#pragma unroll
+    for (int j = 0; j < 12; j++) sums[j * FT + t] = acc[j];
+    __syncthreads();
+    double own[12];
+    if (t < G)
+#pragma unroll
+        for (int j = 0; j < 12; j++) {
+            double s = 0.0;
+            for (int u = 0; u < nsub; u++) s += sums[j * FT + u * G + t];
+            own[j] = s;
+        }
+    __syncthreads();
+    if (t < G)
+#pragma unroll
+        for (int j = 0; j < 12; j++) sums[j * FT + t] = own[j];
+    cl.sync();
+    if (t < G && t % FCL == rk && dir < ndir) {
+        double v[12];
+#pragma unroll
+        for (int j = 0; j < 12; j++) {
+            v[j] = 0.0;
+            for (int q = 0; q < FCL; q++) v[j] += cl.map_shared_rank(sums, q)[j * FT + t];
+        }
         double out[6];
         for (int part = 0; part < 2; part++) {  // real, imag
             double N[3], Lv[3];
-            for (int t = 0; t < 3; t++) {
-                N[t] = red[2 * t + part][0];
-                Lv[t] = red[6 + 2 * t + part][0];
+            for (int i = 0; i < 3; i++) {
+                N[i] = v[2 * i + part];
+                Lv[i] = v[6 + 2 * i + part];
             }
             const double rN = r[0] * N[0] + r[1] * N[1] + r[2] * N[2];
             // r x (r x N) = r (r.N) - N ; r x L
             const double rxL[3] = {r[1] * Lv[2] - r[2] * Lv[1], r[2] * Lv[0] - r[0] * Lv[2],
                                    r[0] * Lv[1] - r[1] * Lv[0]};
-            for (int t = 0; t < 3; t++) out[2 * t + part] = eta * (r[t] * rN - N[t]) + rxL[t];
+            for (int i = 0; i < 3; i++) out[2 * i + part] = eta * (r[i] * rN - N[i]) + rxL[i];
         }
         // multiply by j k / (4 pi) and divide by S = (A/c) e^{-j w t0} exp(-(w w_p / 8c)^2)
         const double* wv = waves + 10 * b;
@@ -598,14 +663,16 @@ __global__ void k_far_field(int ne, int npad, int B, int nq, int nfreq, int ndir
         const double Sr = mag * cs, Si = mag * ss;
         const double den = Sr * Sr + Si * Si;
         const double fac = k / (4.0 * 3.14159265358979323846);
-        for (int t = 0; t < 3; t++) {
-            const double vr = -fac * out[2 * t + 1], vi = fac * out[2 * t];  // j k/(4 pi) * (vr + j vi)
+        const size_t o = ((size_t)b * nfreq + f) * ndir + dir;
+        for (int i = 0; i < 3; i++) {
+            const double vr = -fac * out[2 * i + 1], vi = fac * out[2 * i];  // j k/(4 pi) * (vr + j vi)
             const double er = den > 0 ? (vr * Sr + vi * Si) / den : 0.0;
             const double ei = den > 0 ? (vi * Sr - vr * Si) / den : 0.0;
-            E[((size_t)o * 3 + t) * 2] = er;
-            E[((size_t)o * 3 + t) * 2 + 1] = ei;
+            E[(o * 3 + i) * 2] = er;
+            E[(o * 3 + i) * 2 + 1] = ei;
         }
     }
+    cl.sync();  // every read of a CTA's shared memory by the others is done
 }
 
 inline int grid_for(long long n, int bs = 256) {
@@ -793,11 +860,28 @@ void launch_pack_cur(mot_handle* h, double* out, cudaStream_t s) {
 }
 
 void launch_far_field(mot_handle* h, int n_dir, const double* dirs, double* E, cudaStream_t s) {
-    const int n = h->B * h->nfreq * n_dir;
-    if (n == 0) return;
-    k_far_field<<<n, 256, 0, s>>>(h->ne, h->npad, h->B, h->nq, h->nfreq, n_dir, h->d_rhs_x, h->d_rhs_wf, h->d_dft,
-                                  h->d_omega, dirs, h->d_waves, h->c, h->eta, E);
-    h->launches++;
+    if (h->B * h->nfreq * n_dir == 0) return;
+    const int DT = std::max(1, std::min(8, FT / h->B));
+    const size_t nb = (size_t)h->npad * h->B;
+    for (int f = 0; f < h->nfreq; f++) {
+        k_point_currents<<<(h->npts * h->B + 127) / 128, 128, 0, s>>>(h->npts, h->npad, h->B, h->nq, h->d_ptptr,
+                                                                      h->d_ptent, h->d_rhs_wf,
+                                                                      h->d_dft + (size_t)f * 4 * nb * 2, h->d_ptcur);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((n_dir + DT - 1) / DT * FCL);
+        cfg.blockDim = dim3(FT);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = FCL;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, k_far_field, h->npts, h->B, h->nfreq, f, n_dir, DT, (const double*)h->d_pts,
+                           (const double*)h->d_ptcur, (const double*)h->d_omega, dirs, (const double*)h->d_waves, h->c,
+                           h->eta, E);
+        h->launches += 2;
+    }
 }
 
 }  // namespace mot

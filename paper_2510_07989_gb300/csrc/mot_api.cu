@@ -439,6 +439,10 @@ int ensure_state(mot_handle* h, int B) {
     h->d_waves = (double*)dalloc(h, sizeof(double) * 10 * B);
     h->d_ring = (double*)dalloc(h, sizeof(double) * (size_t)h->R * 6 * bv);
     h->d_ptfield = (double*)dalloc(h, sizeof(double) * 2 * (size_t)h->npts * B);
+    if (h->nfreq > 0) {
+        h->d_ptcur = (double*)dalloc(h, sizeof(double) * 12 * (size_t)h->npts * B);
+        if (!h->d_ptcur) return fail(h, MOT_EOOM, "device allocation of the march state");
+    }
     h->d_cur = (double*)dalloc(h, sizeof(double) * 4 * (size_t)h->npad * B);
     if (h->opt.precision == MOT_PREC_MIXED && !h->precomputing) {
         int major = 0;
@@ -502,7 +506,7 @@ int ensure_state(mot_handle* h, int B) {
 }
 
 void free_state(mot_handle* h) {
-    void* ptrs[] = {h->d_waves, h->d_ring, h->d_win, h->d_ptfield, h->d_cur, h->d_dft, h->d_work, h->d_partial, h->d_V, h->d_H,
+    void* ptrs[] = {h->d_waves, h->d_ring, h->d_win, h->d_ptfield, h->d_ptcur, h->d_cur, h->d_dft, h->d_work, h->d_partial, h->d_V, h->d_H,
                     h->d_g, h->d_cs, h->d_sn, h->d_Z, h->d_resid, h->d_gm_bnorm, h->d_wscale,
                     h->d_wprev1, h->d_wprev2};
     for (void* p : ptrs)
@@ -514,7 +518,7 @@ void free_state(mot_handle* h) {
     h->d_ring32 = h->d_win32 = h->d_xf = nullptr;
     h->d_ring16 = h->d_win16 = nullptr;
     h->hist_tc = false;
-    h->d_waves = h->d_ring = h->d_win = h->d_ptfield = h->d_cur = h->d_dft = h->d_work = h->d_partial = nullptr;
+    h->d_waves = h->d_ring = h->d_win = h->d_ptfield = h->d_ptcur = h->d_cur = h->d_dft = h->d_work = h->d_partial = nullptr;
     h->d_V = h->d_H = h->d_g = h->d_cs = h->d_sn = h->d_Z = h->d_resid = nullptr;
     h->d_gm_active = h->d_gm_jend = nullptr;
     h->d_gm_bnorm = nullptr;
@@ -1693,15 +1697,25 @@ MOT_API int mot_load_operators(mot_handle* h, const mot_operators* ops) {
         }
     }
     h->npts = (int)(pts.size() / 3);
+    std::vector<int> ptptr(h->npts + 1, 0), ptent((size_t)ne * h->nq);
+    for (size_t e = 0; e < ptent.size(); e++) ptptr[ptidx[e] + 1]++;
+    for (int k = 0; k < h->npts; k++) ptptr[k + 1] += ptptr[k];
+    {
+        std::vector<int> at(ptptr.begin(), ptptr.end() - 1);
+        for (size_t e = 0; e < ptent.size(); e++) ptent[at[ptidx[e]]++] = (int)e;
+    }
     h->d_pts = (double*)dalloc(h, sizeof(double) * pts.size());
     h->d_ptidx = (int*)dalloc(h, sizeof(int) * ptidx.size());
-    if (!h->d_pts || !h->d_ptidx) return fail(h, MOT_EOOM, "device allocation (RHS points)");
+    h->d_ptptr = (int*)dalloc(h, sizeof(int) * ptptr.size());
+    h->d_ptent = (int*)dalloc(h, sizeof(int) * ptent.size());
+    if (!h->d_pts || !h->d_ptidx || !h->d_ptptr || !h->d_ptent)
+        return fail(h, MOT_EOOM, "device allocation (quadrature points)");
+    CK(cudaMemcpy(h->d_ptptr, ptptr.data(), sizeof(int) * ptptr.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_ptent, ptent.data(), sizeof(int) * ptent.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->d_pts, pts.data(), sizeof(double) * pts.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->d_ptidx, ptidx.data(), sizeof(int) * ptidx.size(), cudaMemcpyHostToDevice));
-    h->d_rhs_x = (double*)dalloc(h, sizeof(double) * x.size());
     h->d_rhs_wf = (double*)dalloc(h, sizeof(double) * wf.size());
-    if (!h->d_rhs_x || !h->d_rhs_wf) return fail(h, MOT_EOOM, "device allocation (RHS table)");
-    CK(cudaMemcpy(h->d_rhs_x, x.data(), sizeof(double) * x.size(), cudaMemcpyHostToDevice));
+    if (!h->d_rhs_wf) return fail(h, MOT_EOOM, "device allocation (RHS table)");
     CK(cudaMemcpy(h->d_rhs_wf, wf.data(), sizeof(double) * wf.size(), cudaMemcpyHostToDevice));
     h->tc_bulk = h->opt.precision == MOT_PREC_MIXED && mflag(h, MOT_MIX_TC) && mflag(h, MOT_MIX_TCBULK);
     if ((st = build_tiles(h, ops)) != MOT_OK) return st;
@@ -2313,7 +2327,8 @@ MOT_API void mot_destroy(mot_handle* h) {
     void* ptrs[] = {h->d_edge_faces, h->d_edge_verts, h->d_face_edges, h->d_face_sgn, h->d_iperm, h->d_cg_iters,
                     h->vtx_edges.rowptr, h->vtx_edges.col, h->vtx_edges.val, h->Lf.rowptr, h->Lf.col, h->Lf.val,
                     h->Lv.rowptr, h->Lv.col, h->Lv.val, h->G.rowptr, h->G.col, h->G.val, h->Gt.rowptr,
-                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_x, h->d_rhs_wf, h->d_pts, h->d_ptidx, h->d_tiles, h->d_tmask,
+                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_wf, h->d_pts, h->d_ptidx,
+                    h->d_ptptr, h->d_ptent, h->d_tiles, h->d_tmask,
                     h->hist.tasks, h->hist.chunks, h->hist.chunk_ptr, h->lag0.tasks, h->lag0.chunks,
                     h->lag0.chunk_ptr, h->d_omega, h->d_colidx, h->d_tiles32, h->d_Q0, h->d_Q0f, h->d_LF,
                     h->d_LFf, h->d_Minvf, h->d_Minv64, h->d_Lfinvf, h->d_Lvinvf, h->d_Ginvf, h->hist_tc_list.packed, h->hist_tc_list.chunks,

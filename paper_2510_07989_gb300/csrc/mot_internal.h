@@ -101,11 +101,13 @@ struct mot_handle {
     double* d_T0s = nullptr;       // [npad][npad]
     double* d_T0h = nullptr;
     int nq = 0;
-    double* d_rhs_x = nullptr;     // [npad][nq][3]
-    double* d_rhs_wf = nullptr;
+    double* d_rhs_wf = nullptr;    // [npad][nq][3] weight * area * f_m
     int npts = 0;                  // distinct quadrature points (edges share their triangles')
     double* d_pts = nullptr;       // [npts][3]
     int* d_ptidx = nullptr;        // [npad][nq] point of every entry of the table
+    int* d_ptptr = nullptr;        // [npts+1] entries (row * nq + q) of the table at each point ..
+    int* d_ptent = nullptr;        // .. [ne * nq]
+    double* d_ptcur = nullptr;     // [npts][12][B] point currents of one frequency (far field)
     double* d_ptfield = nullptr;   // [npts][2][B] incident field integrals of the step
 
     // block-sparse history

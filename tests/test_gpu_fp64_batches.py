@@ -59,3 +59,30 @@ def test_preconditioned_solve_past_the_kept_vectors(M, torus):
     assert s.noconv > 0 and s.info()["last_gmres_iters"] == 14
     ref = S.march(exc, n, b=1)
     assert np.abs(W[:, 1].reshape(n, -1) - ref).max() < 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("B,n_dir", [(1, 1), (1, 17), (9, 9), (48, 6), (64, 3)])
+def test_far_field_over_batches(M, torus, B, n_dir):
+    """The far field for batches and direction counts that fill a CTA's threads
+    (direction, wave, share of the points) in different ways, ragged last
+    direction tiles among them: against the oracle's radiation integrals of the
+    currents recovered from the same steps, the 1e-9 of the parity test."""
+    from oracle import farfield as FF
+    ops, S = torus
+    exc = MS.fibonacci_batch(B, ops.dt, w_steps=20, t0_steps=20, r_obj=1.3)
+    n, omegas = 30, np.array([0.0, 0.7])
+    s = M.Solver(ops, fp64_precond=1)
+    M.mot_set_frequencies(s.h, omegas)
+    W = s.run(exc, n)
+    t = np.linspace(0.1, 3.0, n_dir)
+    dirs = np.stack([np.sin(t) * np.cos(2 * t), np.sin(t) * np.sin(2 * t), np.cos(t)], axis=1)
+    E = M.mot_fields(s.h, M.mot_waves(exc), dirs, 2, B)
+    for b in sorted({0, B - 1}):
+        parts = [S.split(w) for w in W[:, b].reshape(n, -1)]
+        ell = np.array([p[0] for p in parts])
+        sg = np.array([p[1] for p in parts])
+        cur = ell + ops.tmax / ops.dt * np.diff(sg, axis=0, prepend=np.zeros((1, sg.shape[1])))
+        for f, w in enumerate(omegas):
+            X = cur.T @ FF.dft_weights(w, ops.dt, n)
+            ref = FF.far_field(ops.rwg, X[:ops.ne], X[ops.ne:], w, 1.0, dirs) / FF.pulse_spectrum(exc, b, w)
+            assert np.abs(E[b, f] - ref).max() <= 1e-9 * np.abs(ref).max()
