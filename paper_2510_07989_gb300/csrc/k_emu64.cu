@@ -223,14 +223,16 @@ __global__ void __launch_bounds__(XT) k_slice_x(int K, int N, const double* __re
     c.barrier_wait();
 }
 
-// Y[z] (M x N, rows < M, columns < N) = partial product over the k-tiles
+// W[z] (M x N, rows < M, columns < N) = partial product over the k-tiles
 // [z * kts, (z + 1) * kts) of CTA split z (gridDim.z splits; kts a multiple
-// of KC_TILES).
+// of KC_TILES), as compensated FP32 pairs before the scaling: k_emu_reduce sums
+// the splits and converts. (Converted here, an output took some ten operations
+// of a double-precision unit that does two per clock and SM, about half of the
+// kernel at 1848 x 1848 x 64: 32 us, now 15.)
 template <int NSL>
 __global__ void __launch_bounds__(E_THREADS, 1)
-    k_emu_gemm(int M, int N, int K, int kts, const __nv_bfloat16* __restrict__ A16, const int* __restrict__ ea,
-               const __nv_bfloat16* __restrict__ X16, const int* __restrict__ ex, double* __restrict__ Y,
-               int* __restrict__ err) {
+    k_emu_gemm(int M, int N, int K, int kts, const __nv_bfloat16* __restrict__ A16,
+               const __nv_bfloat16* __restrict__ X16, float2* __restrict__ W, int* __restrict__ err) {
     using C = EmuCfg<NSL>;
     constexpr int E_NS = C::NS, E_STAGE = C::STAGE, A_STAGE = C::A_STAGE, B_STAGE = C::B_STAGE;
     constexpr int NLEV = NSL;
@@ -359,11 +361,16 @@ __global__ void __launch_bounds__(E_THREADS, 1)
         }
         const int gi = mt * EM + row;
         if (ok && gi < M) {
-            double* out = Y + (size_t)z * M * N + (size_t)gi * N;
+            float2* out = W + (size_t)z * M * N + (size_t)gi * N + nh * EN;
+            const int nc = min(EN, N - nh * EN);
+            if ((N & 1) == 0) {  // rows 16-byte aligned
 #pragma unroll
-            for (int n = 0; n < EN; n++) {
-                const int gj = nh * EN + n;
-                if (gj < N) out[gj] = ldexp((double)hi[n] + (double)lo[n], ea[gi] + ex[gj] - 12);
+                for (int n = 0; n < EN; n += 2)
+                    if (n < nc) *reinterpret_cast<float4*>(out + n) = make_float4(hi[n], lo[n], hi[n + 1], lo[n + 1]);
+            } else {
+#pragma unroll
+                for (int n = 0; n < EN; n++)
+                    if (n < nc) out[n] = make_float2(hi[n], lo[n]);
             }
         }
     }
@@ -375,11 +382,30 @@ __global__ void __launch_bounds__(E_THREADS, 1)
     }
 }
 
-__global__ void k_emu_reduce(size_t n, int S, const double* __restrict__ W, double* __restrict__ Y) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        double v = 0.0;
-        for (int z = 0; z < S; z++) v += W[(size_t)z * n + i];
-        Y[i] = v;
+// v 2^e, exact (the exponent field, where the result is normal)
+__device__ __forceinline__ double scale2(double v, int e) {
+    const long long b = __double_as_longlong(v);
+    const int x = (int)((b >> 52) & 0x7ff);
+    return x != 0 && x != 0x7ff && x + e > 0 && x + e < 0x7ff ? __longlong_as_double(b + ((long long)e << 52))
+                                                             : ldexp(v, e);
+}
+
+// Y = the S partial products, summed in order in compensated FP32 (the pairs carry
+// 48 bits, the slices 41 at most), times the row's and the column's scale
+__global__ void __launch_bounds__(256) k_emu_reduce(int M, int N, int S, const float2* __restrict__ W,
+                                                    const int* __restrict__ ea, const int* __restrict__ ex,
+                                                    double* __restrict__ Y) {
+    const size_t n = (size_t)M * N;
+    for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
+        float hi = 0.f, lo = 0.f;
+#pragma unroll 4
+        for (int z = 0; z < S; z++) {
+            const float2 w = W[(size_t)z * n + i];
+            twosum(hi, lo, w.x);
+            lo += w.y;
+        }
+        const int r = (int)(i / N), c = (int)(i - (size_t)r * N);
+        Y[i] = scale2((double)hi + (double)lo, ea[r] + ex[c] - 12);
     }
 }
 
@@ -427,7 +453,7 @@ int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, doub
     S = (KT + kts - 1) / kts;
     const int NSL = A.nsl;
     const size_t x16 = sizeof(uint16_t) * (size_t)NH * KT * NSL * EN * EK;
-    const size_t part = S > 1 ? sizeof(double) * (size_t)S * A.M * N : 0;
+    const size_t part = (sizeof(float2) * (size_t)S * A.M * N + 15) / 16 * 16;
     const size_t need = x16 + part + sizeof(int) * 256;
     if (need > h->emuws_bytes) {
         if (h->d_emuws) {
@@ -440,7 +466,7 @@ int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, doub
         h->emuws_bytes = need;
     }
     if (N > 256) return fail(h, MOT_EINVAL, "emulated FP64 product: N > 256");
-    double* ws = reinterpret_cast<double*>(h->d_emuws);
+    float2* ws = reinterpret_cast<float2*>(h->d_emuws);
     __nv_bfloat16* d_x16 = reinterpret_cast<__nv_bfloat16*>(h->d_emuws + part);
     int* d_ex = reinterpret_cast<int*>(h->d_emuws + part + x16);
     {
@@ -466,20 +492,14 @@ int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, doub
     });
     dim3 grid(MT, NH, S);
     const auto* a16 = reinterpret_cast<const __nv_bfloat16*>(A.a16);
-    double* out = S > 1 ? ws : Y;
     if (NSL == 6) {
-        k_emu_gemm<6><<<grid, E_THREADS, EmuCfg<6>::SMEM, s>>>(A.M, N, K, kts, a16, A.ea, d_x16, d_ex, out,
-                                                               h->d_cg_iters + 2);
+        k_emu_gemm<6><<<grid, E_THREADS, EmuCfg<6>::SMEM, s>>>(A.M, N, K, kts, a16, d_x16, ws, h->d_cg_iters + 2);
     } else {
-        k_emu_gemm<4><<<grid, E_THREADS, EmuCfg<4>::SMEM, s>>>(A.M, N, K, kts, a16, A.ea, d_x16, d_ex, out,
-                                                               h->d_cg_iters + 2);
+        k_emu_gemm<4><<<grid, E_THREADS, EmuCfg<4>::SMEM, s>>>(A.M, N, K, kts, a16, d_x16, ws, h->d_cg_iters + 2);
     }
-    h->launches += 2;
-    if (S > 1) {
-        const size_t n = (size_t)A.M * N;
-        k_emu_reduce<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256, 0, s>>>(n, S, ws, Y);
-        h->launches++;
-    }
+    const size_t n = (size_t)A.M * N;
+    k_emu_reduce<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256, 0, s>>>(A.M, N, S, ws, A.ea, d_ex, Y);
+    h->launches += 3;
     return MOT_OK;
 }
 
