@@ -118,9 +118,10 @@ __device__ __forceinline__ void dots(const Part<G>& P, int L, const double* V, s
         double p[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
         for (int l = share * 32 + lane; l < L; l += parts * 32) {
-            const int ix = P.at(l);
-            if (ix < 0) continue;
-            const double x = SM ? ws[l] : w[ix];
+            // no branch, so that the unrolled loads go out together: past the
+            // vector's end x is 0
+            const int at = P.at(l), ix = at < 0 ? 0 : at;
+            const double x = SM ? ws[l] : at < 0 ? 0.0 : w[ix];
 #pragma unroll
             for (int i = 0; i < 4; i++)
                 if (v0 + i < ns) p[i] = fma(v0 + i < nv ? V[(size_t)(v0 + i) * vs + ix] : x, x, p[i]);

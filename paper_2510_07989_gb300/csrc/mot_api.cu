@@ -1340,6 +1340,11 @@ int build_tiles(mot_handle* h, const mot_operators* ops) {
     if ((st = make_list(th_lag0, rb_lag0, h->lag0)) != MOT_OK) return st;
     if (h->opt.precision == MOT_PREC_MIXED && (h->opt.mixed_flags & MOT_MIX_TC)) {
         if ((st = make_tc_list(h, th_hist, rb_hist, MOT_TC_CHUNK, 0.4)) != MOT_OK) return st;
+        // epilogue warps until tuned or set: four fold a large launch faster (924
+        // edges, B = 64, 190 637 tasks: 826 us against 885 with eight; 448 303 tasks:
+        // 1776 against 1916), eight fill and drain the short chunks of a small one
+        // faster (14 046 tasks, B = 8: 100 us against 114)
+        h->tc_epi = h->hist_tc_list.ntasks >= 1 << 17 ? 4 : 8;
         h->tc_tasks_host = std::move(th_hist);  // kept for re-chunking by the tuner
         h->tc_rbs_host = std::move(rb_hist);
     }

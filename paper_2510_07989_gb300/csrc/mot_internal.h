@@ -184,7 +184,7 @@ struct mot_handle {
     bool tc_bulk = false;          // tensor-core history in the bulk form (global column order, blocked ring)
     int tc_stages = 0;             // pipeline stages of the tensor-core history (0: the deepest that fits)
     int tc_cap = 0;                // tasks per chunk the tensor-core list was cut with
-    int tc_epi = 8;                // epilogue warps of the tensor-core history (4 or 8)
+    int tc_epi = 8;                // epilogue warps of the tensor-core history (4 or 8, by the launch's size)
     int tc_tps = 1;                // tasks per pipeline stage of the tensor-core history (1 or 2)
     // FP64 path with fp64_direct: dense inverses formed at load, in place of CG
     double* d_Ginv64 = nullptr;    // G^{-1}, npad x npad
