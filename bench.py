@@ -537,9 +537,9 @@ def run_ours(args):
                        "c_dt": ops.dt, "k_max": ops.kmax, "history_lags": K, "rhs_per_step": B,
                        "precision": ("mixed (history on tensor cores: FP32 tiles and coefficients as bf16 x 3, "
                                      "compensated FP32 sums; FP32 dense Q_0 and Q_0^-1, FP64 left factor, "
-                                     "FP64 refinement, FP64 CG projector)" if kern == 2 else
+                                     "FP64 refinement, FP64 refined projector)" if kern == 2 else
                                      "mixed (FP32 history tiles, dense FP32 Q_0 and left factors, FP64 sums, "
-                                     "FP64 CG projector)") if args.precision == "mixed" else "fp64 plain",
+                                     "FP64 refined projector)") if args.precision == "mixed" else "fp64 plain",
                        "history_prefill_steps": K + 1,
                        "tc_form": args.tc_form,
                        "tuner": {"chunk_cap": info1["tc_chunk_cap"], "lag_frac": info1["tc_lag_frac"],

@@ -64,7 +64,7 @@ typedef struct {
     double gmres_tol;      /* relative residual of the Q_0 solve, default 1e-13 (FP64), 1e-11 (mixed) */
     int32_t gmres_maxit;   /* default 200 */
     double cg_tol;         /* relative residual of Laplacian / Gram solves, default 1e-14 */
-    int32_t cg_maxit;      /* default 5000 */
+    int32_t cg_maxit;      /* sweeps (or CG iterations) of such a solve, default 5000 */
     int32_t timing;        /* 1: time every history-contraction launch with CUDA events
                               on its stream (reported by mot_get_info); default 0 */
     int32_t mixed_flags;   /* MOT_PREC_MIXED only; 0 = default (MOT_MIX_DEFAULT). Bits:
@@ -88,13 +88,16 @@ typedef struct {
                                  (relative error about 2^-40 of sum |A||x|) */
     int32_t refine_sweeps; /* MOT_MIX_REFINE: FP64 residual + correction sweeps per step
                               (stops early once |r| <= gmres_tol |b|); default 1 */
-    int32_t fp64_precond;  /* MOT_PREC_FP64 only. 0 (default): GMRES on Q_0 in product form,
-                              unpreconditioned. 1: right-preconditioned GMRES, Q_0 M z = b,
-                              x = M z, with M = Q_0^{-1} formed at load in FP64 (Q_0 from the
-                              product form on unit columns, LU with partial pivoting); every
-                              product stays FP64, so the result matches the unpreconditioned
-                              solve to the GMRES tolerance while the iteration count drops to
-                              a few. Costs (2 npad)^2 doubles of device memory. */
+    int32_t fp64_precond;  /* MOT_PREC_FP64 only. 0 (default): GMRES on Q_0, unpreconditioned;
+                              Q_0 is assembled densely at load from its product form on unit
+                              columns ((2 npad)^2 doubles of device memory) or, where that is
+                              not possible (no memory, a projector solve at its limit),
+                              applied in product form. 1: right-preconditioned GMRES,
+                              Q_0 M z = b, x = M z, with M = Q_0^{-1} formed at load in FP64
+                              (LU with partial pivoting); every product stays FP64, so the
+                              result matches the unpreconditioned solve to the GMRES tolerance
+                              while the iteration count drops to a few. Costs (2 npad)^2
+                              doubles of device memory more. */
     int32_t hist_stall_test; /* testing of the failure path only; 0 (default) = off. k > 0:
                               every tensor-core history launch withholds the copies of the
                               k-th pipeline stage of its first CTA (the k-th task with one
@@ -103,12 +106,13 @@ typedef struct {
                               and raises the error word, and mot_step returns MOT_ECUDA
                               with the GPU context intact. */
     int32_t fp64_direct;   /* MOT_PREC_FP64 only. 0 (default): the Gram solves (G^{-1} in the
-                              left factor) by CG on the normal equations and the projector
-                              solves by CG on the graph Laplacians, to cg_tol. 1: by dense
-                              FP64 inverses formed at load (LU with partial pivoting; the
-                              Laplacians as (L + 11^T/N)^{-1}, their pseudo-inverse on the
-                              mean-free right-hand sides), exact to rounding; costs
-                              npad^2 + nf^2 + nv^2 doubles of device memory. */
+                              left factor) and the projectors' graph-Laplacian solves by FP64
+                              refinement with FP32 dense inverses formed at load, to cg_tol
+                              (plain CG where the inverses do not serve, e.g. a surface of
+                              several components). 1: by dense FP64 inverses formed at load (LU
+                              with partial pivoting; the Laplacians as (L + 11^T/N)^{-1}, their
+                              pseudo-inverse on the mean-free right-hand sides), exact to
+                              rounding; costs npad^2 + nf^2 + nv^2 doubles of device memory. */
 } mot_options;
 
 enum { MOT_MIX_HIST32 = 1, MOT_MIX_LF32 = 2, MOT_MIX_Q032 = 4, MOT_MIX_REFINE = 8, MOT_MIX_PRECOND = 16,
@@ -182,7 +186,7 @@ typedef struct {
     double D, tmax, dt;
     int32_t last_gmres_iters;   /* max over the batch, last step */
     double last_gmres_resid;    /* max relative residual, last step */
-    int32_t last_cg_iters;      /* max CG iterations of any projector/Gram solve, last step */
+    int32_t last_cg_iters;      /* most sweeps or CG iterations of any projector/Gram solve, last step */
     int64_t device_bytes;       /* device memory held by the handle */
     int64_t gpu_launches;       /* kernels launched by this handle so far */
     double tile_fill;           /* nonzero fraction of the stored history tiles */
@@ -320,7 +324,9 @@ int mot_run_many(mot_handle* const* hs, int n, int n_steps, const mot_wave* cons
  * epilogue warps in {4, 8} -- is applied and its launch (one
  * for all n handles) timed
  * three times with CUDA events on `stream` after one warm-up; the fastest
- * (median) is kept by every handle and reported by mot_get_info. The trial
+ * (median) is kept by every handle and reported by mot_get_info. Tasks per chunk
+ * is an upper limit: a launch that would be fewer than four such chunks per SM is
+ * cut smaller. The trial
  * launches read the current march state and change nothing a later step
  * reads. Requires handles on the tensor-core history (mixed precision, B a
  * multiple of 8) of one kernel form on one device that have taken a step

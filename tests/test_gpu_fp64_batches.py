@@ -30,11 +30,12 @@ def torus():
     return ops, P.ProductSystem(ops)
 
 
-@pytest.mark.parametrize("kw", [{}, {"fp64_precond": 1}, {"fp64_direct": 1}], ids=["plain", "precond", "direct"])
-@pytest.mark.parametrize("B", [1, 2, 3, 5, 7, 8, 9, 15, 16, 17, 24, 33, 64])
-def test_fp64_march_over_batches(M, torus, B, kw):
-    if kw and B not in (3, 9, 33):
-        pytest.skip("the products' forms are those of the plain path")
+CASES = [({}, B) for B in (1, 2, 3, 5, 7, 8, 9, 15, 16, 17, 24, 33, 64)]
+CASES += [({k: 1}, B) for k in ("fp64_precond", "fp64_direct") for B in (3, 9, 33)]
+
+
+@pytest.mark.parametrize("kw,B", CASES, ids=lambda v: str(v) if isinstance(v, int) else "-".join(v) or "plain")
+def test_fp64_march_over_batches(M, torus, kw, B):
     ops, S = torus
     exc = MS.fibonacci_batch(B, ops.dt, w_steps=20, t0_steps=20, r_obj=1.3)
     n = 35
