@@ -87,3 +87,23 @@ def test_far_field_over_batches(M, torus, B, n_dir):
             X = cur.T @ FF.dft_weights(w, ops.dt, n)
             ref = FF.far_field(ops.rwg, X[:ops.ne], X[ops.ne:], w, 1.0, dirs) / FF.pulse_spectrum(exc, b, w)
             assert np.abs(E[b, f] - ref).max() <= 1e-9 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("kw,B,tol", [({}, 2, 1e-10), ({"fp64_precond": 1}, 5, 1e-10), ({"precision": 1}, 8, 1e-6)],
+                         ids=["plain", "precond", "mixed"])
+def test_two_separate_spheres(M, kw, B, tol):
+    """One mesh of two components: its graph Laplacians have a null space larger
+    than the constants, so the dense inverses behind the projector solves do not
+    serve and plain CG takes their place. Against the product-form oracle,
+    within the paths' usual bounds."""
+    a = MS.icosphere(1)
+    m = MS.build_edges(MS.Mesh(np.concatenate([a.verts * 0.5 - [0.8, 0, 0], a.verts * 0.5 + [0.8, 0, 0]]),
+                               np.concatenate([a.tris, a.tris + a.nv]).astype(np.int32), name="two spheres"))
+    ops = assemble(m, 2.0, 1.0, 0.3)
+    exc = MS.fibonacci_batch(B, ops.dt, w_steps=20, t0_steps=20, r_obj=1.4)
+    n = 40
+    s = M.Solver(ops, **kw)
+    W = s.run(exc, n)
+    assert s.noconv == 0
+    ref = P.ProductSystem(ops).march(exc, n, b=B - 1)
+    assert np.abs(W[:, B - 1].reshape(n, -1) - ref).max() < tol * np.abs(ref).max()
