@@ -562,6 +562,27 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Grows the chunk-sum buffer of h to the current tensor-core list.
+int fit_partial(mot_handle* h) {
+    const size_t need = sizeof(double) * (size_t)std::max(1, h->hist_tc_list.nchunks) * 2 * MOT_TILE * 2 * h->B;
+    if (need <= h->partial_bytes) return MOT_OK;
+    cudaFree(h->d_partial);
+    h->device_bytes -= (int64_t)h->partial_bytes;
+    h->partial_bytes = 0;
+    h->d_partial = (double*)dalloc(h, need);
+    if (!h->d_partial) return fail(h, MOT_EOOM, "device allocation (history chunk sums)");
+    h->partial_bytes = need;
+    return MOT_OK;
+}
+
+// What a launch of the tensor-core history needs of h, whatever became of the
+// re-cuts of its list before: the list, and room for one partial result per chunk.
+int tc_ready(mot_handle* h) {
+    if (!(h->hist_tc_list.packed && h->hist_tc_list.rb_ptr && h->hist_tc_list.rb_chunks))
+        return fail(h, MOT_ESTATE, "tensor-core history: no task list (a re-cut of the list failed)");
+    return fit_partial(h);
+}
+
 // One MOT step in three phases (a full step runs all of them on one stream):
 //   STEP_INPUTS   right-hand side, windowed sums of the K~ tail, reduced-precision panels
 //   STEP_HISTORY  the history contraction, subtracted from the right-hand side: W.y1, W.y2
@@ -595,8 +616,10 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
         }
     }
     if ((phases & STEP_HISTORY) && i >= 2) {
-        if (h->hist_tc && !(h->hist_tc_list.packed && h->hist_tc_list.rb_ptr && h->hist_tc_list.rb_chunks))
-            return fail(h, MOT_ESTATE, "tensor-core history: no task list (a re-cut of the list failed)");
+        if (h->hist_tc) {
+            const int st = tc_ready(h);
+            if (st != MOT_OK) return st;
+        }
         if (h->hist_tc)
             launch_history_tc(h, h->hist_tc_list, i, W.rho1, W.rho2, W.y1, W.y2, s);
         else if (h32)
@@ -1834,18 +1857,6 @@ class HostBarrier {
     long gen_ = 0;
 };
 
-// Grows the chunk-sum buffer of h to the current tensor-core list.
-int fit_partial(mot_handle* h) {
-    const size_t need = sizeof(double) * (size_t)std::max(1, h->hist_tc_list.nchunks) * 2 * MOT_TILE * 2 * h->B;
-    if (need <= h->partial_bytes) return MOT_OK;
-    cudaFree(h->d_partial);
-    h->device_bytes -= (int64_t)h->partial_bytes;
-    h->d_partial = (double*)dalloc(h, need);
-    if (!h->d_partial) return fail(h, MOT_EOOM, "device allocation (history chunk sums)");
-    h->partial_bytes = need;
-    return MOT_OK;
-}
-
 // Autotuner of the tensor-core history for handles marched together (one
 // launch serves all of them): every candidate (tasks per chunk, lags per L2
 // range, pipeline stages and tasks per stage, epilogue warps) is applied,
@@ -1952,9 +1963,10 @@ MOT_API int mot_set_tc_config(mot_handle* h, int cap, double lag_frac, int stage
     int st;
     if ((st = make_tc_list(h, h->tc_tasks_host, h->tc_rbs_host, cap, lag_frac)) != MOT_OK) return st;
     if (!h->hist_tc_list.packed) return fail(h, MOT_EINVAL, "tensor-core list not available");
+    // the handle keeps the new list even if the pipeline is refused: its chunks need their room first
+    if ((st = fit_partial(h)) != MOT_OK) return st;
     if (!history_tc_config_fits(h->npad, h->tc_bulk, h->hist_tc_list.cap, stages, tasks_per_stage))
         return fail(h, MOT_EINVAL, "mot_set_tc_config: stages x tasks per stage do not fit in shared memory");
-    if ((st = fit_partial(h)) != MOT_OK) return st;
     h->tc_stages = stages;
     h->tc_tps = tasks_per_stage;
     h->tc_epi = epilogue_warps;
@@ -2050,6 +2062,12 @@ MOT_API int mot_run_many(mot_handle* const* hs, int n, int n_steps, const mot_wa
                 const int t = tune_tc(hm.data(), (int)hm.size(), gs);
                 if (t != MOT_OK) group_status = t;
             }
+            for (mot_handle* h : hm) {
+                const int t = tc_ready(h);
+                if (t != MOT_OK && group_status == MOT_OK) group_status = t;
+            }
+        }
+        if (!hm.empty() && group_status == MOT_OK) {
             const bool timed = full && hm[0]->opt.timing;
             const float ms = launch_history_tc_many(hm.data(), (int)hm.size(), rho1.data(), rho2.data(), y1.data(),
                                                     y2.data(), gs, timed);
@@ -2092,6 +2110,10 @@ MOT_API int mot_run_many(mot_handle* const* hs, int n, int n_steps, const mot_wa
                 bar.wait();
                 if (g == 0) group_history();
                 bar.wait();
+                if (ok && group_status != MOT_OK) {  // no history sums: the step cannot go on
+                    st[i] = group_status;
+                    ok = false;
+                }
                 if (ok) {
                     cudaStreamWaitEvent(s, ev_hist, 0);
                     double* dst = out ? out + (size_t)k * B[i] * 2 * h->ne : nullptr;
