@@ -436,13 +436,6 @@ int emu_prepare(mot_handle* h, const double* A, int M, int K, EmuMat* out, int n
     return MOT_OK;
 }
 
-void emu_free(mot_handle* h, EmuMat* m) {
-    if (m->ea) cudaFree(m->ea);
-    if (m->a16) cudaFree(m->a16);
-    m->ea = nullptr;
-    m->a16 = nullptr;
-}
-
 int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, double* Y, cudaStream_t s) {
     const int K = A.K, KT = K / EK, NH = (N + EN - 1) / EN, MT = A.Mp / EM;
     int nsm = 148;
@@ -456,10 +449,7 @@ int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, doub
     const size_t part = (sizeof(float2) * (size_t)S * A.M * N + 15) / 16 * 16;
     const size_t need = x16 + part + sizeof(int) * 256;
     if (need > h->emuws_bytes) {
-        if (h->d_emuws) {
-            cudaFree(h->d_emuws);
-            h->device_bytes -= (int64_t)h->emuws_bytes;
-        }
+        dfree(h, h->d_emuws);
         h->emuws_bytes = 0;
         h->d_emuws = (unsigned char*)dalloc(h, need);
         if (!h->d_emuws) return fail(h, MOT_EOOM, "device allocation (emulated FP64 workspace)");

@@ -421,10 +421,7 @@ void launch_history32(mot_handle* h, const TaskList& tl, const float* tiles, con
 
 double* split_workspace(mot_handle* h, size_t bytes) {
     if (bytes > h->sgws_bytes) {
-        if (h->d_sgws) {
-            cudaFree(h->d_sgws);
-            h->device_bytes -= (int64_t)h->sgws_bytes;
-        }
+        dfree(h, h->d_sgws);
         h->sgws_bytes = 0;
         h->d_sgws = (double*)dalloc(h, bytes);
         if (h->d_sgws) h->sgws_bytes = bytes;

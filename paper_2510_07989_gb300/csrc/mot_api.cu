@@ -57,7 +57,16 @@ void* dalloc(mot_handle* h, size_t bytes) {
         return nullptr;
     }
     h->device_bytes += (int64_t)bytes;
+    h->blocks[p] = bytes;
     return p;
+}
+
+void dfree(mot_handle* h, void* p) {
+    const auto it = h->blocks.find(p);
+    if (it == h->blocks.end()) return;
+    cudaFree(p);
+    h->device_bytes -= (int64_t)it->second;
+    h->blocks.erase(it);
 }
 
 // mixed-precision kernels (k_mixed.cu)
@@ -509,12 +518,10 @@ void free_state(mot_handle* h) {
     void* ptrs[] = {h->d_waves, h->d_ring, h->d_win, h->d_ptfield, h->d_ptcur, h->d_cur, h->d_dft, h->d_work, h->d_partial, h->d_V, h->d_H,
                     h->d_g, h->d_cs, h->d_sn, h->d_Z, h->d_resid, h->d_gm_bnorm, h->d_wscale,
                     h->d_wprev1, h->d_wprev2};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    for (void* p : ptrs) dfree(h, p);
     h->d_wprev1 = h->d_wprev2 = nullptr;
     void* fptrs[] = {h->d_ring32, h->d_win32, h->d_xf, h->d_ring16, h->d_win16};
-    for (void* p : fptrs)
-        if (p) cudaFree(p);
+    for (void* p : fptrs) dfree(h, p);
     h->d_ring32 = h->d_win32 = h->d_xf = nullptr;
     h->d_ring16 = h->d_win16 = nullptr;
     h->hist_tc = false;
@@ -566,8 +573,7 @@ bool is_device_ptr(const void* p) {
 int fit_partial(mot_handle* h) {
     const size_t need = sizeof(double) * (size_t)std::max(1, h->hist_tc_list.nchunks) * 2 * MOT_TILE * 2 * h->B;
     if (need <= h->partial_bytes) return MOT_OK;
-    cudaFree(h->d_partial);
-    h->device_bytes -= (int64_t)h->partial_bytes;
+    dfree(h, h->d_partial);
     h->partial_bytes = 0;
     h->d_partial = (double*)dalloc(h, need);
     if (!h->d_partial) return fail(h, MOT_EOOM, "device allocation (history chunk sums)");
@@ -976,8 +982,7 @@ int make_tc_list(mot_handle* h, const std::vector<HistTask>& tasks, const std::v
     {  // a list made before (re-tuning) is replaced
         TaskList& old = h->hist_tc_list;
         void* ptrs[] = {old.packed, old.chunks, old.rb_ptr, old.rb_chunks};
-        for (void* p : ptrs)
-            if (p) cudaFree(p);
+        for (void* p : ptrs) dfree(h, p);
         old.packed = nullptr;
         old.chunks = nullptr;
         old.rb_ptr = old.rb_chunks = nullptr;
@@ -1420,9 +1425,9 @@ int precompute_mixed(mot_handle* h) {
         dense_pad_identity(h, (int)n2, h->ne, lu, s);
         const int bad = dense_lu(h, (int)n2, lu, piv, piv + n2, s);
         if (bad > 0) {
-            cudaFree(lu);
-            cudaFree(inv);
-            cudaFree(piv);
+            dfree(h, lu);
+            dfree(h, inv);
+            dfree(h, piv);
             return fail(h, MOT_EINVAL, "Q_0 is singular to working precision (LU pivot breakdown)");
         }
         dense_inverse_from_lu(h, (int)n2, lu, piv, inv, s);
@@ -1432,10 +1437,9 @@ int precompute_mixed(mot_handle* h) {
             if ((st = emu_prepare(h, inv, (int)n2, (int)n2, &h->emu_Minv, 4)) != MOT_OK) return st;
         }
         CK(cudaDeviceSynchronize());
-        cudaFree(lu);
-        cudaFree(inv);
-        cudaFree(piv);
-        h->device_bytes -= (int64_t)(2 * sizeof(double) * (size_t)n2 * n2 + sizeof(int) * (size_t)(n2 + 1));
+        dfree(h, lu);
+        dfree(h, inv);
+        dfree(h, piv);
     }
     CK(cudaGetLastError());
     CK(cudaDeviceSynchronize());
@@ -1453,10 +1457,8 @@ int precompute_mixed(mot_handle* h) {
         CK(cudaDeviceSynchronize());
     }
     if (h32) {  // the FP64 lag-0 tiles (the dense Q_0 assembly's input) are no longer read
-        cudaFree(h->d_tiles);
-        cudaFree(h->d_tmask);
-        h->device_bytes -= (int64_t)((sizeof(double) * MOT_TILE * MOT_TILE + sizeof(uint32_t) * MOT_TILE) *
-                                     (size_t)std::max<int64_t>(1, h->ntiles_fp64));
+        dfree(h, h->d_tiles);
+        dfree(h, h->d_tmask);
         h->d_tiles = nullptr;
         h->d_tmask = nullptr;
     }
@@ -1480,14 +1482,12 @@ int precompute_fp64(mot_handle* h) {
     cudaStream_t s = 0;
     const long long n2 = 2LL * h->npad;
     const size_t qbytes = sizeof(double) * (size_t)n2 * n2;
-    const int64_t held = h->device_bytes;  // without the assembly's temporary march state
     h->precomputing = true;
     int st = ensure_state(h, Bp);
     double* q0 = st == MOT_OK ? (double*)dalloc(h, qbytes) : nullptr;
     if (!q0) {
         free_state(h);
         h->precomputing = false;
-        h->device_bytes = held;
         if (need) return st != MOT_OK ? st : fail(h, MOT_EOOM, "device allocation (FP64 Q_0)");
         h->err.clear();
         return MOT_OK;
@@ -1505,20 +1505,18 @@ int precompute_fp64(mot_handle* h) {
     CK(cudaMemcpy(it, h->d_cg_iters, 2 * sizeof(int), cudaMemcpyDeviceToHost));
     free_state(h);
     h->precomputing = false;
-    h->device_bytes = held;
     if (it[1] > 0) {
-        cudaFree(q0);
+        dfree(h, q0);
         return need ? fail(h, MOT_ENOCONV, "a CG solve did not converge while assembling Q_0") : MOT_OK;
     }
     h->d_Q0 = q0;
-    h->device_bytes += (int64_t)qbytes;
     if (!need) return MOT_OK;
     double* lu = (double*)dalloc(h, qbytes);
     int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(n2 + 1));
     h->d_Minv64 = (double*)dalloc(h, qbytes);
     if (!lu || !piv || !h->d_Minv64) {
-        if (lu) cudaFree(lu);
-        if (piv) cudaFree(piv);
+        dfree(h, lu);
+        dfree(h, piv);
         return fail(h, MOT_EOOM, "device allocation (FP64 Q_0 factorisation)");
     }
     CK(cudaMemcpyAsync(lu, q0, qbytes, cudaMemcpyDeviceToDevice, s));
@@ -1527,9 +1525,8 @@ int precompute_fp64(mot_handle* h) {
     if (bad == 0) dense_inverse_from_lu(h, (int)n2, lu, piv, h->d_Minv64, s);
     CK(cudaGetLastError());
     CK(cudaDeviceSynchronize());
-    cudaFree(lu);
-    cudaFree(piv);
-    h->device_bytes -= (int64_t)(qbytes + sizeof(int) * (size_t)(n2 + 1));
+    dfree(h, lu);
+    dfree(h, piv);
     if (bad > 0) return fail(h, MOT_EINVAL, "Q_0 is singular to working precision (LU pivot breakdown)");
     return MOT_OK;
 }
@@ -1549,7 +1546,6 @@ int form_refine_inverse(mot_handle* h, int kind) {
     cudaStream_t s = 0;
     const int npd = ((kind == INV_GRAM ? h->npad : A.n) + 63) / 64 * 64;
     const size_t nn = (size_t)npd * npd;
-    const int64_t held = h->device_bytes;
     double* a = (double*)dalloc(h, sizeof(double) * nn);
     double* inv = (double*)dalloc(h, sizeof(double) * nn);
     int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(npd + 1));
@@ -1586,10 +1582,8 @@ int form_refine_inverse(mot_handle* h, int kind) {
     CK(cudaDeviceSynchronize());
     CK(cudaGetLastError());
     void* tmp[] = {a, inv, piv, trial, good ? nullptr : *out};
-    for (void* p : tmp)
-        if (p) cudaFree(p);
+    for (void* p : tmp) dfree(h, p);
     if (!good) *out = nullptr;
-    h->device_bytes = held + (good ? (int64_t)(sizeof(float) * nn) : 0);
     return MOT_OK;
 }
 
@@ -1619,10 +1613,9 @@ int prepare_fp64_direct(mot_handle* h, const std::vector<std::tuple<int, int, do
                                  cudaMemcpyDeviceToDevice, s));
         }
         CK(cudaDeviceSynchronize());
-        cudaFree(A);
-        cudaFree(inv);
-        cudaFree(piv);
-        h->device_bytes -= (int64_t)(2 * sizeof(double) * (size_t)gpd * gpd + sizeof(int) * (size_t)(gpd + 1));
+        dfree(h, A);
+        dfree(h, inv);
+        dfree(h, piv);
         if (bad != 0) return fail(h, MOT_EINVAL, "G is singular to working precision (LU pivot breakdown)");
     }
     auto lap = [&](const DCsr& L, int n, double** out, int* npd_out) -> int {
@@ -1635,9 +1628,8 @@ int prepare_fp64_direct(mot_handle* h, const std::vector<std::tuple<int, int, do
         const int bad = dense_lu(h, npd, A, piv, piv + npd, s);
         if (bad == 0) dense_inverse_from_lu(h, npd, A, piv, *out, s);
         CK(cudaDeviceSynchronize());
-        cudaFree(A);
-        cudaFree(piv);
-        h->device_bytes -= (int64_t)(sizeof(double) * (size_t)npd * npd + sizeof(int) * (size_t)(npd + 1));
+        dfree(h, A);
+        dfree(h, piv);
         if (bad != 0) return fail(h, MOT_EINVAL, "a graph Laplacian plus 11^T/N is singular (surface not connected?)");
         *npd_out = npd;
         return MOT_OK;
@@ -1758,7 +1750,7 @@ MOT_API int mot_set_frequencies(mot_handle* h, int n_freq, const double* omega) 
     if (h->step != 0 || h->B != 0) return fail(h, MOT_ESTATE, "set frequencies before the first step");
     if (n_freq < 0 || (n_freq > 0 && !omega)) return fail(h, MOT_EINVAL, "bad frequency list");
     CK(cudaSetDevice(h->dev));
-    if (h->d_omega) cudaFree(h->d_omega);
+    dfree(h, h->d_omega);
     h->d_omega = nullptr;
     h->nfreq = n_freq;
     h->omega.assign(omega, omega + n_freq);
@@ -2192,10 +2184,8 @@ MOT_API int mot_fields(mot_handle* h, const mot_wave* waves, int n_dir, const do
     launch_far_field(h, n_dir, dd, de, 0);
     CK(cudaDeviceSynchronize());
     CK(cudaMemcpy(E_out, de, sizeof(double) * (size_t)h->B * h->nfreq * n_dir * 6, cudaMemcpyDeviceToHost));
-    cudaFree(dd);
-    cudaFree(de);
-    h->device_bytes -= (int64_t)(sizeof(double) * 3 * std::max(1, n_dir) +
-                                 sizeof(double) * (size_t)h->B * h->nfreq * std::max(1, n_dir) * 6);
+    dfree(h, dd);
+    dfree(h, de);
     return MOT_OK;
 }
 
@@ -2350,23 +2340,7 @@ MOT_API void mot_destroy(mot_handle* h) {
     if (!h) return;
     cudaSetDevice(h->dev);
     cudaDeviceSynchronize();
-    free_state(h);
-    void* ptrs[] = {h->d_edge_faces, h->d_edge_verts, h->d_face_edges, h->d_face_sgn, h->d_iperm, h->d_cg_iters,
-                    h->vtx_edges.rowptr, h->vtx_edges.col, h->vtx_edges.val, h->Lf.rowptr, h->Lf.col, h->Lf.val,
-                    h->Lv.rowptr, h->Lv.col, h->Lv.val, h->G.rowptr, h->G.col, h->G.val, h->Gt.rowptr,
-                    h->Gt.col, h->Gt.val, h->d_T0s, h->d_T0h, h->d_rhs_wf, h->d_pts, h->d_ptidx,
-                    h->d_ptptr, h->d_ptent, h->d_tiles, h->d_tmask,
-                    h->hist.tasks, h->hist.chunks, h->hist.chunk_ptr, h->lag0.tasks, h->lag0.chunks,
-                    h->lag0.chunk_ptr, h->d_omega, h->d_colidx, h->d_tiles32, h->d_Q0, h->d_Q0f, h->d_LF,
-                    h->d_LFf, h->d_Minvf, h->d_Minv64, h->d_Lfinvf, h->d_Lvinvf, h->d_Ginvf, h->hist_tc_list.packed, h->hist_tc_list.chunks,
-                    h->hist_tc_list.rb_ptr, h->hist_tc_list.rb_chunks, h->d_tiles16, h->d_sgws, h->d_emuws,
-                    h->d_Ginv64, h->d_Lfinv64, h->d_Lvinv64, h->d_dir_r, h->d_dir_z, h->d_dir_sc};
-    emu_free(h, &h->emu_Q0);
-    emu_free(h, &h->emu_LF);
-    emu_free(h, &h->emu_Q0s);
-    emu_free(h, &h->emu_Minv);
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    for (const auto& b : h->blocks) cudaFree(b.first);
     if (h->h_cg_iters) cudaFreeHost(h->h_cg_iters);
     if (h->h_gmstat) cudaFreeHost(h->h_gmstat);
     if (h->ev0) cudaEventDestroy(h->ev0);

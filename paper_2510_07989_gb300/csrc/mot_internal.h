@@ -6,6 +6,7 @@
 #include <atomic>
 
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/mot.h"
@@ -168,7 +169,8 @@ struct mot_handle {
     double last_gmres_resid = 0;
     int last_cg_iters = 0;
     int64_t launches = 0;
-    int64_t device_bytes = 0;
+    int64_t device_bytes = 0;  // sum of blocks
+    std::unordered_map<void*, size_t> blocks;  // device memory held (dalloc, dfree)
     cudaStream_t stream = nullptr;
     // algorithmic work of a full-depth history contraction
     double hist_nnz_tasks = 0;   // sum over history tasks of the tile's nonzeros
@@ -252,6 +254,7 @@ inline void once_per_device(std::atomic<unsigned long long>& done, int dev, F&& 
 }
 int cuda_fail(mot_handle* h, cudaError_t e, const char* where);
 void* dalloc(mot_handle* h, size_t bytes);
+void dfree(mot_handle* h, void* p);  // p from dalloc of h, or null
 
 // workspace of the split-K products (grown on demand; null: no memory, take one split)
 double* split_workspace(mot_handle* h, size_t bytes);
@@ -288,7 +291,6 @@ float launch_history_tc_many(mot_handle* const* hs, int n, const double* const* 
 // emulated FP64 products on tensor cores (k_emu64.cu): Y (M x N) = A X with A
 // prepared once by emu_prepare from the device FP64 matrix A (M x K, ld K)
 int emu_prepare(mot_handle* h, const double* A, int M, int K, EmuMat* out, int nsl);
-void emu_free(mot_handle* h, EmuMat* m);
 int launch_emu_gemm(mot_handle* h, const EmuMat& A, const double* X, int N, double* Y, cudaStream_t s);
 
 // block-vector helpers (rows npad, C columns)
