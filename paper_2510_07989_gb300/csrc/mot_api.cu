@@ -427,8 +427,12 @@ int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double
         }
         add = true;
         if (converged || total >= maxit) break;
-        // restart from the true residual
-        apply_q0(h, W, x, W.r, s);
+        // restart from the true residual; of a refinement the FP64 one, as its first: with the
+        // reduced-precision Q_0 the later cycles would drive x to the solution of that matrix
+        if (kind == GM_REFINE)
+            apply_q0_dense64(h, x, W.r, s);
+        else
+            apply_q0(h, W, x, W.r, s);
         launch_axpby(h, (int)bv, 1.0, b, -1.0, W.r, W.r, s);
         launch_gm_begin(h, b, false, W.r, h->d_V, s);
     }
