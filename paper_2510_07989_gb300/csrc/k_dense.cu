@@ -202,7 +202,7 @@ __global__ void k_demean_cols(int N, int C, const double* __restrict__ f, double
         if (threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
         __syncthreads();
     }
-    const int e = red[0] > 0.0 ? ilogb(red[0]) : 0;
+    const int e = red[0] > 0.0 ? mot_scale_exponent(red[0]) : 0;
     const double sc = ldexp(1.0, -e);
     for (int row = threadIdx.x; row < N; row += blockDim.x)
         r[(size_t)row * C + c] = (f[(size_t)row * C + c] - mean) * sc;

@@ -138,7 +138,7 @@ __device__ __forceinline__ double col_reduce_max(double v, double* red, double* 
 
 // 2^-e with 2^e the power of two at or below m (1 for m = 0): multiplying by
 // it (and later by its inverse) is exact and brings a column to O(1)
-__device__ __forceinline__ double pow2_scale(double m) { return m > 0.0 ? ldexp(1.0, -ilogb(m)) : 1.0; }
+__device__ __forceinline__ double pow2_scale(double m) { return m > 0.0 ? ldexp(1.0, -mot_scale_exponent(m)) : 1.0; }
 
 template <int CW, bool NORMAL>
 __global__ void __launch_bounds__(1024) k_cg(int N, int C, CsrV A, CsrV A2, const double* __restrict__ f,
@@ -493,7 +493,7 @@ __global__ void k_wave_scale(int npad, int B, const double* __restrict__ x, doub
         if (threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) sc[b] = red[0] > 0.0 ? ldexp(1.0, -ilogb(red[0])) : 1.0;
+    if (threadIdx.x == 0) sc[b] = red[0] > 0.0 ? ldexp(1.0, -mot_scale_exponent(red[0])) : 1.0;
 }
 
 // x[:, b] and x[:, B + b] times sc[b] (inverse: divided by it; exact, powers of two)

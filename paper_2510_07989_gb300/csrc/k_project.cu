@@ -76,7 +76,7 @@ __device__ __forceinline__ float warp_sums(float (&v)[NV]) {
 }
 
 __device__ __forceinline__ double pow2_at(double m, int sign) {
-    return m > 0.0 && m < INFINITY ? ldexp(1.0, sign * ilogb(m)) : 1.0;
+    return m > 0.0 && m < INFINITY ? ldexp(1.0, sign * mot_scale_exponent(m)) : 1.0;
 }
 
 template <int CW, int MODE>
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(PT) k_refine_solve(Problem Q, const double* __
     __syncthreads();
     const double thr = thr_s[c];
     int it = 0;
-    bool open = true;
+    bool open = true, lost = false;  // lost: this thread saw a row that is no number
     while (open && it < maxit) {
         for (int i = t; i < N * CW; i += PT) rs[sidx(i / CW, i % CW)] = __ldcg(rg + i);
         __syncthreads();
@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(PT) k_refine_solve(Problem Q, const double* __
             r[ix] = rn;
             z[ix] += (double)__ldcg(d + ix);
             rg[ix] = (float)rn;
-            mine |= fabs(rn) > thr;
+            mine |= fabs(rn) > thr;  // a row or threshold that is no number ends its column's sweeps ..
+            lost |= !(fabs(rn) <= INFINITY) || !(thr <= INFINITY);
         }
         if (mine) open_s[it & 1] = 1;
         cl.sync();
@@ -233,6 +234,7 @@ __global__ void __launch_bounds__(PT) k_refine_solve(Problem Q, const double* __
         for (int k = 0; k < CL; k++) open |= cl.map_shared_rank(open_s, k)[it & 1] != 0;
         it++;
     }
+    if (lost) atomicAdd(noconv, 1);  // .. and counts as not converged
     const double us = pow2_at(top, 1);
     if (MODE == GRAM) {
         for (int row = r0 + tr; row < r1; row += RS)

@@ -24,6 +24,14 @@
 // Size (doubles) of the fixed device array used by mot_fields_noalloc.
 #define MOT_NOALLOC_FIELD_DOUBLES 262144
 
+#ifdef __CUDACC__
+// Exponent e of the power of two 2^e at or below m > 0 by which a vector of
+// largest magnitude m is scaled (by 2^-e, exact) and scaled back. At least
+// -1000: below 2^-1023 the scale 2^-e itself would overflow, and a subnormal
+// vector is brought to 1e-23 or more this way, far from any underflow.
+__device__ __forceinline__ int mot_scale_exponent(double m) { return max(ilogb(m), -1000); }
+#endif
+
 // One tile product of the history contraction:
 //   out[code.out] (TILE rows of row block rb, 2B columns)
 //     += tile (TILE x TILE) * panel(k, code.part, code.variant)[rows of column block cb]
