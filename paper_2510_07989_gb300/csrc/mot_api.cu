@@ -443,9 +443,7 @@ int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double
     return converged ? MOT_OK : fail(h, MOT_ENOCONV, "GMRES reached its iteration limit");
 }
 
-int ensure_state(mot_handle* h, int B) {
-    if (h->B == B && h->d_ring) return MOT_OK;
-    if (h->B != 0 && h->B != B) return fail(h, MOT_EINVAL, "batch size changed without mot_reset");
+int alloc_state(mot_handle* h, int B) {
     h->B = B;
     const size_t bv = (size_t)h->npad * 2 * B;
     h->gm_m = std::min(std::max(h->opt.gmres_maxit, 1), 100);
@@ -537,6 +535,16 @@ void free_state(mot_handle* h) {
     h->B = 0;
     h->step = 0;
     h->gmres_iters_total = 0;
+}
+
+// The march state for batches of B: all of it, or (no memory) none, so that a
+// later call finds no half of one.
+int ensure_state(mot_handle* h, int B) {
+    if (h->B == B && h->d_ring) return MOT_OK;
+    if (h->B != 0 && h->B != B) return fail(h, MOT_EINVAL, "batch size changed without mot_reset");
+    const int st = alloc_state(h, B);
+    if (st != MOT_OK) free_state(h);
+    return st;
 }
 
 int check_waves(mot_handle* h, const mot_wave* waves, int B) {

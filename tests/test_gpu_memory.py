@@ -40,3 +40,32 @@ def test_device_bytes_over_resets(M, ops, kw):
     # from the first reset on only buffers that outlive a march stay; none grows in the second pair
     assert seen[4:] == [seen[4], seen[3], seen[6], seen[3]]
     assert seen[4] > seen[6] > seen[3]
+
+
+def hold(free):
+    """Device memory taken so that about `free` bytes are left."""
+    import torch
+    torch.cuda.empty_cache()
+    return torch.empty(max(0, torch.cuda.mem_get_info()[0] - int(free)), dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("kw", [{}, {"precision": 1}], ids=["fp64", "mixed"])
+def test_march_after_a_refused_state(M, ops, kw):
+    """A step that finds no memory for its state (half of it is there) says so and
+    leaves a handle that marches once there is: the same steps as any other."""
+    exc = MS.fibonacci_batch(64, ops.dt, w_steps=20, t0_steps=20, r_obj=1.3)
+    s = M.Solver(ops, **kw)
+    loaded = s.info()["device_bytes"]
+    ref = s.run(exc, 3)
+    state = s.info()["device_bytes"] - loaded
+    M.mot_reset(s.h)
+    t = M.Solver(ops, **kw)
+    held = hold(state / 2)
+    for _ in range(2):
+        with pytest.raises(M.MotError) as e:
+            t.run(exc, 1)
+        assert e.value.code == M.MOT_EOOM
+    del held
+    import torch
+    torch.cuda.empty_cache()
+    assert np.array_equal(t.run(exc, 3), ref)
