@@ -44,6 +44,7 @@ int cuda_fail(mot_handle* h, cudaError_t e, const char* where) {
 void* dalloc(mot_handle* h, size_t bytes) {
     void* p = nullptr;
     if (bytes == 0) bytes = 16;
+    h->asked_bytes += bytes;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
@@ -366,8 +367,8 @@ enum { GM_MAIN = 0, GM_REFINE = 1 };
 
 // GMRES on Q_0 x = b to |residual| <= tol |b|. r0 null: from x = 0; else x holds
 // the initial guess and r0 = b - Q_0 x. prec: right preconditioned, Q_0 M z = b,
-// x = M z, with the vectors M V_j kept (MOT_GM_ZCAP of them) so that x is their
-// combination; a longer solve applies M once more to the combination of the V_j.
+// x = M z, with the vectors M V_j kept (MOT_GM_ZCAP of them, or none) so that x is
+// their combination; a longer solve applies M once more to the combination of the V_j.
 // GM_REFINE: the largest |r0| / |b| of the batch is left in last_gmres_resid, and
 // nothing more is done when it is within gmres_tol already.
 //
@@ -380,6 +381,7 @@ int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double
           cudaStream_t s) {
     const int B = h->B, m = h->gm_m, maxit = h->opt.gmres_maxit;
     const size_t bv = (size_t)h->npad * 2 * B;
+    const int zcap = h->d_Z ? MOT_GM_ZCAP : 0;
     const double* res = h->h_gmstat;
     const int* act = (const int*)(res + 2 * B);
     const int* jen = act + B;
@@ -400,7 +402,7 @@ int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double
     for (;;) {
         int jend = 0;
         for (int j = 0; j < m && total < maxit && !converged; j++) {
-            double* mv = !prec ? nullptr : j < MOT_GM_ZCAP ? h->d_Z + (size_t)j * bv : W.q1;
+            double* mv = !prec ? nullptr : j < zcap ? h->d_Z + (size_t)j * bv : W.q1;
             apply_q0(h, W, h->d_V + (size_t)j * bv, W.w, s, mv);
             launch_gm_iter(h, j, W.w, tol, kind == GM_REFINE ? 1e-6 : 0.0, s);
             jend = j + 1;
@@ -418,7 +420,7 @@ int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double
         int used = 1;
         for (int k = 0; k < B; k++) used = std::max(used, std::min(jen[k], jend));
         total -= jend - used;
-        if (prec && used > MOT_GM_ZCAP) {
+        if (prec && used > zcap) {
             launch_gm_finish(h, h->d_V, used, false, W.ygm, W.q1, s);
             apply_m(h, W.q1, W.t1, s);
             launch_axpby(h, (int)bv, 1.0, W.t1, add ? 1.0 : 0.0, add ? x : nullptr, x, s);
@@ -450,10 +452,7 @@ int alloc_state(mot_handle* h, int B) {
     h->d_waves = (double*)dalloc(h, sizeof(double) * 10 * B);
     h->d_ring = (double*)dalloc(h, sizeof(double) * (size_t)h->R * 6 * bv);
     h->d_ptfield = (double*)dalloc(h, sizeof(double) * 2 * (size_t)h->npts * B);
-    if (h->nfreq > 0) {
-        h->d_ptcur = (double*)dalloc(h, sizeof(double) * 12 * (size_t)h->npts * B);
-        if (!h->d_ptcur) return fail(h, MOT_EOOM, "device allocation of the march state");
-    }
+    if (h->nfreq > 0) h->d_ptcur = (double*)dalloc(h, sizeof(double) * 12 * (size_t)h->npts * B);
     h->d_cur = (double*)dalloc(h, sizeof(double) * 4 * (size_t)h->npad * B);
     if (h->opt.precision == MOT_PREC_MIXED && !h->precomputing) {
         int major = 0;
@@ -481,13 +480,9 @@ int alloc_state(mot_handle* h, int B) {
         h->d_xf = (float*)dalloc(h, sizeof(float) * 2 * bv);
         if (!h->d_xf) return fail(h, MOT_EOOM, "device allocation of the march state");
     }
-    if (!h->hist_tc) {
-        h->d_win = (double*)dalloc(h, sizeof(double) * (size_t)(h->max_tail_lag + 1) * bv);
-        if (!h->d_win) return fail(h, MOT_EOOM, "device allocation of the march state");
-    }
+    if (!h->hist_tc) h->d_win = (double*)dalloc(h, sizeof(double) * (size_t)(h->max_tail_lag + 1) * bv);
     h->d_wprev1 = (double*)dalloc(h, sizeof(double) * bv);
     h->d_wprev2 = (double*)dalloc(h, sizeof(double) * bv);
-    if (!h->d_wprev1 || !h->d_wprev2) return fail(h, MOT_EOOM, "device allocation of the march state");
     h->d_dft = (double*)dalloc(h, sizeof(double) * std::max(1, h->nfreq) * 4 * (size_t)h->npad * B * 2);
     h->work_bytes = sizeof(double) * work_doubles(h);
     h->d_work = (double*)dalloc(h, h->work_bytes);
@@ -499,19 +494,18 @@ int alloc_state(mot_handle* h, int B) {
     h->d_g = (double*)dalloc(h, sizeof(double) * (size_t)B * (h->gm_m + 1));
     h->d_cs = (double*)dalloc(h, sizeof(double) * (size_t)B * h->gm_m);
     h->d_sn = (double*)dalloc(h, sizeof(double) * (size_t)B * h->gm_m);
-    const bool prec = !h->precomputing && (h->d_Minvf || h->d_Minv64);
-    if (prec) {
-        h->d_Z = (double*)dalloc(h, sizeof(double) * MOT_GM_ZCAP * bv);
-        if (!h->d_Z) return fail(h, MOT_EOOM, "device allocation of the march state");
-    }
     h->d_resid = (double*)dalloc(h, sizeof(double) * 3 * B);
     h->d_gm_active = (int*)(h->d_resid + 2 * B);
     h->d_gm_jend = h->d_gm_active + B;
     h->d_gm_bnorm = (double*)dalloc(h, sizeof(double) * B);
     h->d_wscale = (double*)dalloc(h, sizeof(double) * B);
     if (!h->d_waves || !h->d_ring || !h->d_ptfield || !h->d_cur || !h->d_dft || !h->d_work || !h->d_partial ||
-        !h->d_V || !h->d_H || !h->d_g || !h->d_cs || !h->d_sn || !h->d_resid || !h->d_gm_bnorm || !h->d_wscale)
+        !h->d_V || !h->d_H || !h->d_g || !h->d_cs || !h->d_sn || !h->d_resid || !h->d_gm_bnorm || !h->d_wscale ||
+        !h->d_wprev1 || !h->d_wprev2 || (!h->hist_tc && !h->d_win) || (h->nfreq > 0 && !h->d_ptcur))
         return fail(h, MOT_EOOM, "device allocation of the march state");
+    // without memory for them M V_j is not kept: one more product with M at a solve's end
+    if (!h->precomputing && (h->d_Minvf || h->d_Minv64))
+        h->d_Z = (double*)dalloc(h, sizeof(double) * MOT_GM_ZCAP * bv);
     h->h_waves.assign(10 * B, NAN);
     return MOT_OK;
 }
@@ -537,13 +531,45 @@ void free_state(mot_handle* h) {
     h->gmres_iters_total = 0;
 }
 
+// FP64 path: operators that make its march faster and that it can do without
+// (dense Q_0: the product form; FP32 inverses: CG) are formed only where twice
+// their memory is free, and given back when the march state finds none.
+size_t free_memory() {
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return free;
+}
+bool spare_memory(size_t bytes) { return free_memory() / 2 >= bytes; }
+
+// gives them back if that makes room for `need` bytes
+bool release_spare(mot_handle* h, size_t need) {
+    if (h->opt.precision == MOT_PREC_MIXED) return false;
+    void* ptrs[] = {h->d_Q0, h->d_Lfinvf, h->d_Lvinvf, h->d_Ginvf};
+    size_t held = 0;
+    for (void* p : ptrs)
+        if (p) held += h->blocks[p];
+    if (held == 0 || free_memory() + held < need) return false;
+    for (void* p : ptrs) dfree(h, p);
+    h->d_Q0 = nullptr;
+    h->d_Lfinvf = h->d_Lvinvf = h->d_Ginvf = nullptr;
+    return true;
+}
+
 // The march state for batches of B: all of it, or (no memory) none, so that a
 // later call finds no half of one.
 int ensure_state(mot_handle* h, int B) {
     if (h->B == B && h->d_ring) return MOT_OK;
     if (h->B != 0 && h->B != B) return fail(h, MOT_EINVAL, "batch size changed without mot_reset");
-    const int st = alloc_state(h, B);
+    h->asked_bytes = 0;
+    int st = alloc_state(h, B);
     if (st != MOT_OK) free_state(h);
+    if (st == MOT_EOOM && !h->precomputing && release_spare(h, h->asked_bytes)) {
+        st = alloc_state(h, B);
+        if (st != MOT_OK) free_state(h);
+    }
     return st;
 }
 
@@ -1486,14 +1512,16 @@ int precompute_mixed(mot_handle* h) {
 // alone are as many multiplications as one product with the dense Q_0
 // (4 npad^2 B each), so the dense form is taken whenever it can be formed. It
 // cannot when the memory is not there or a CG solve runs into its limit while
-// assembling: the march then applies the product form (with fp64_precond the
-// load fails as it needs Q_0 itself).
+// assembling: the march then applies the product form. With fp64_precond the
+// load needs Q_0 itself and fails without it; short of memory it factorises Q_0
+// in place and the march applies the product form.
 int precompute_fp64(mot_handle* h) {
     const int Bp = 64;
     const bool need = h->opt.fp64_precond != 0;
     cudaStream_t s = 0;
     const long long n2 = 2LL * h->npad;
     const size_t qbytes = sizeof(double) * (size_t)n2 * n2;
+    if (!need && !spare_memory(qbytes)) return MOT_OK;
     h->precomputing = true;
     int st = ensure_state(h, Bp);
     double* q0 = st == MOT_OK ? (double*)dalloc(h, qbytes) : nullptr;
@@ -1523,15 +1551,19 @@ int precompute_fp64(mot_handle* h) {
     }
     h->d_Q0 = q0;
     if (!need) return MOT_OK;
-    double* lu = (double*)dalloc(h, qbytes);
     int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(n2 + 1));
     h->d_Minv64 = (double*)dalloc(h, qbytes);
-    if (!lu || !piv || !h->d_Minv64) {
-        dfree(h, lu);
+    if (!piv || !h->d_Minv64) {
         dfree(h, piv);
         return fail(h, MOT_EOOM, "device allocation (FP64 Q_0 factorisation)");
     }
-    CK(cudaMemcpyAsync(lu, q0, qbytes, cudaMemcpyDeviceToDevice, s));
+    double* lu = spare_memory(qbytes) ? (double*)dalloc(h, qbytes) : nullptr;
+    if (lu) {
+        CK(cudaMemcpyAsync(lu, q0, qbytes, cudaMemcpyDeviceToDevice, s));
+    } else {
+        lu = q0;
+        h->d_Q0 = nullptr;
+    }
     dense_pad_identity(h, (int)n2, h->ne, lu, s);
     const int bad = dense_lu(h, (int)n2, lu, piv, piv + n2, s);
     if (bad == 0) dense_inverse_from_lu(h, (int)n2, lu, piv, h->d_Minv64, s);
@@ -1558,6 +1590,7 @@ int form_refine_inverse(mot_handle* h, int kind) {
     cudaStream_t s = 0;
     const int npd = ((kind == INV_GRAM ? h->npad : A.n) + 63) / 64 * 64;
     const size_t nn = (size_t)npd * npd;
+    if (!spare_memory((2 * sizeof(double) + sizeof(float)) * nn)) return MOT_OK;
     double* a = (double*)dalloc(h, sizeof(double) * nn);
     double* inv = (double*)dalloc(h, sizeof(double) * nn);
     int* piv = (int*)dalloc(h, sizeof(int) * (size_t)(npd + 1));

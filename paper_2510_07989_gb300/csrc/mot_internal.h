@@ -179,6 +179,7 @@ struct mot_handle {
     int64_t launches = 0;
     int64_t device_bytes = 0;  // sum of blocks
     std::unordered_map<void*, size_t> blocks;  // device memory held (dalloc, dfree)
+    size_t asked_bytes = 0;  // asked of dalloc, refused or not, since last set to 0
     cudaStream_t stream = nullptr;
     // algorithmic work of a full-depth history contraction
     double hist_nnz_tasks = 0;   // sum over history tasks of the tile's nonzeros

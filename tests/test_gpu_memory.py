@@ -1,6 +1,8 @@
 """Device memory of a handle: what mot_get_info reports is what the handle
 holds -- the march state goes with mot_reset, and marching again after it
 takes the same memory as before, on every path."""
+from contextlib import contextmanager, nullcontext
+
 import numpy as np
 import pytest
 
@@ -42,11 +44,16 @@ def test_device_bytes_over_resets(M, ops, kw):
     assert seen[4] > seen[6] > seen[3]
 
 
-def hold(free):
-    """Device memory taken so that about `free` bytes are left."""
+@contextmanager
+def only(free):
+    """Device memory taken meanwhile so that about `free` bytes are left."""
     import torch
-    torch.cuda.empty_cache()
-    return torch.empty(max(0, torch.cuda.mem_get_info()[0] - int(free)), dtype=torch.uint8, device="cuda")
+    held = torch.empty(max(0, torch.cuda.mem_get_info()[0] - int(free)), dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del held
+        torch.cuda.empty_cache()
 
 
 @pytest.mark.parametrize("kw", [{}, {"precision": 1}], ids=["fp64", "mixed"])
@@ -60,12 +67,38 @@ def test_march_after_a_refused_state(M, ops, kw):
     state = s.info()["device_bytes"] - loaded
     M.mot_reset(s.h)
     t = M.Solver(ops, **kw)
-    held = hold(state / 2)
-    for _ in range(2):
-        with pytest.raises(M.MotError) as e:
-            t.run(exc, 1)
-        assert e.value.code == M.MOT_EOOM
-    del held
-    import torch
-    torch.cuda.empty_cache()
+    with only(state / 2):
+        for _ in range(2):
+            with pytest.raises(M.MotError) as e:
+                t.run(exc, 1)
+            assert e.value.code == M.MOT_EOOM
     assert np.array_equal(t.run(exc, 3), ref)
+
+
+@pytest.fixture(scope="module")
+def larger():
+    return assemble(MS.torus(1.0, 0.3, 36, 12), 4.0, 1.0, 0.3)  # 1296 edges: dense Q_0 of 55 MB
+
+
+@pytest.mark.parametrize("kw,when", [({}, "load"), ({}, "state"), ({"fp64_precond": 1}, "state")],
+                         ids=["plain-load", "plain-state", "precond-state"])
+def test_march_where_the_dense_operators_do_not_fit(M, larger, kw, when):
+    """A march that fits without the operators it can do without runs without
+    them: not formed at the load, or given back at its first step. Two ways to the
+    same solution, to the 1e-10 of the FP64 path."""
+    ops, B, n = larger, 16, 3
+    exc = MS.fibonacci_batch(B, ops.dt, w_steps=20, t0_steps=4, r_obj=1.3)
+    s = M.Solver(ops, **kw)
+    loaded = s.info()["device_bytes"]
+    ref = s.run(exc, n)
+    state = s.info()["device_bytes"] - loaded
+    M.mot_destroy(s.h)
+    q0 = 8 * (2 * ((ops.ne + 31) // 32 * 32)) ** 2
+    with only(loaded - 0.5 * q0) if when == "load" else nullcontext():
+        t = M.Solver(ops, **kw)
+    assert (t.info()["device_bytes"] < loaded - q0) == (when == "load")
+    with only(state - 0.3 * q0) if when == "state" else nullcontext():
+        W = t.run(exc, n)
+    assert t.info()["device_bytes"] < loaded + state - q0
+    assert t.noconv == 0
+    assert np.abs(W - ref).max() < 1e-10 * np.abs(ref).max()
