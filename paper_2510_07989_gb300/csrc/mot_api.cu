@@ -1795,16 +1795,18 @@ MOT_API int mot_set_frequencies(mot_handle* h, int n_freq, const double* omega) 
     if (h->step != 0 || h->B != 0) return fail(h, MOT_ESTATE, "set frequencies before the first step");
     if (n_freq < 0 || (n_freq > 0 && !omega)) return fail(h, MOT_EINVAL, "bad frequency list");
     CK(cudaSetDevice(h->dev));
+    for (int f = 0; f < n_freq; f++)
+        if (!std::isfinite(omega[f]) || omega[f] < 0)
+            return fail(h, MOT_EINVAL, "frequencies must be finite and >= 0");
     dfree(h, h->d_omega);
     h->d_omega = nullptr;
-    h->nfreq = n_freq;
+    h->nfreq = 0;
     h->omega.assign(omega, omega + n_freq);
-    for (double w : h->omega)
-        if (!std::isfinite(w) || w < 0) return fail(h, MOT_EINVAL, "frequencies must be finite and >= 0");
     if (n_freq > 0) {
         h->d_omega = (double*)dalloc(h, sizeof(double) * n_freq);
         if (!h->d_omega) return fail(h, MOT_EOOM, "device allocation (frequencies)");
         CK(cudaMemcpy(h->d_omega, omega, sizeof(double) * n_freq, cudaMemcpyHostToDevice));
+        h->nfreq = n_freq;
     }
     return MOT_OK;
 }
