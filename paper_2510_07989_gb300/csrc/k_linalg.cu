@@ -533,10 +533,10 @@ __global__ void k_pack_cur(int ne, int npad, int B, const int* __restrict__ iper
     }
 }
 
-// Point currents of one frequency: the Fourier sums of j and m (loop and star
-// parts summed here, after separate accumulation) times the quadrature's weight *
-// basis function, summed over the edges whose tables share the point.
-// cur[pt][12][b]: j_x re, im, j_y .., then m
+// Point currents of a frequency (blockIdx.y): the Fourier sums of j and m (loop
+// and star parts summed here, after separate accumulation) times the quadrature's
+// weight * basis function, summed over the edges whose tables share the point.
+// cur[f][pt][12][b]: j_x re, im, j_y .., then m
 __global__ void __launch_bounds__(128) k_point_currents(int npts, int npad, int B, int nq,
                                                         const int* __restrict__ ptr, const int* __restrict__ ent,
                                                         const double* __restrict__ wf, const double* __restrict__ D,
@@ -545,6 +545,8 @@ __global__ void __launch_bounds__(128) k_point_currents(int npts, int npad, int 
     if (i >= npts * B) return;
     const int pt = i / B, b = i - pt * B;
     const size_t nb = (size_t)npad * B;
+    D += (size_t)blockIdx.y * 4 * nb * 2;
+    cur += (size_t)blockIdx.y * npts * 12 * B;
     double a[12];
 #pragma unroll
     for (int k = 0; k < 12; k++) a[k] = 0.0;
@@ -566,80 +568,81 @@ __global__ void __launch_bounds__(128) k_point_currents(int npts, int npad, int 
     for (int k = 0; k < 12; k++) cur[((size_t)pt * 12 + k) * B + b] = a[k];
 }
 
-// Far field E_inf(r) = (j k / 4 pi) [eta r x (r x N) + r x L] / S(w) of one
-// frequency; N, L the sums of the point currents times e^{j k r.x}. Bound by
-// the FP64 units: 24 multiply-adds per point, direction and wave, and one
-// sine and cosine per point and direction, shared by the waves (and by the
-// three edges of a point's triangle; per edge and wave they were 24 times as
-// many: 2.62 ms at 480 edges, 8 waves, 3 frequencies, 181 directions). A cluster
-// of eight CTAs takes DT directions: its threads are (share of the points,
-// direction, wave), the shares are summed in shared memory and then over the
-// cluster, in order.
+// Far field E_inf(r) = (j k / 4 pi) [eta r x (r x N) + r x L] / S(w); N, L the
+// sums of the point currents times e^{j k r.x}. Bound by the FP64 units where
+// there is work for all of them: 24 multiply-adds per point, direction, wave and
+// frequency, and one sine and cosine per point, direction and frequency, shared
+// by the waves (and by the three edges of a point's triangle). A cluster of eight
+// CTAs takes DT directions and BT waves of one frequency (grid: direction tiles,
+// wave tiles, frequencies); its threads are (share of the points, direction,
+// wave), the shares are summed in shared memory and then over the cluster, in
+// order. BT and DT are chosen at the launch. A mot_fields call at 480 edges: 8
+// waves, 3 frequencies, 181 directions 697 us, one wave and direction at 100
+// frequencies 162 us; with a launch per frequency over all waves 984 and 7254 us;
+// with a CTA per output over its edges, no points or phases shared, 2750 and 157 us.
 constexpr int FT = 256, FCL = 8;
-__global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, int f, int ndir, int DT,
+__global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, int f0, int ndir, int DT, int BT,
                                                   const double* __restrict__ pts, const double* __restrict__ cur,
                                                   const double* __restrict__ omega, const double* __restrict__ dirs,
                                                   const double* __restrict__ waves, double c, double eta,
                                                   double* __restrict__ E) {
     __shared__ double2 phase[FT];
-    __shared__ double sums[FT * 12];  // shares, then this CTA's sums [12][DT * B]
+    __shared__ double sums[FT * 12];  // shares [12][nsub][DT * BT]; their sums in share 0
     cg::cluster_group cl = cg::this_cluster();
-    const int rk = (int)cl.block_rank(), t = threadIdx.x;
-    const int G = DT * B, nsub = FT / G, sub = t / G, l = t - sub * G, d = l / B, b = l - d * B;
+    const int rk = (int)cl.block_rank(), t = threadIdx.x, f = f0 + blockIdx.z;
+    const int G = DT * BT, nsub = FT / G, sub = t / G, l = t - sub * G, d = l / BT, q = l - d * BT;
     const bool on = sub < nsub;
-    const int dir = blockIdx.x / FCL * DT + d;
+    const int dir = blockIdx.x / FCL * DT + d, b = blockIdx.y * BT + q;
+    const bool wave = b < B;
     const double w = omega[f], k = w / c;
+    cur += (size_t)blockIdx.z * npts * 12 * B;
     double r[3] = {0, 0, 0};
     if (on && dir < ndir)
         for (int i = 0; i < 3; i++) r[i] = dirs[3 * dir + i];
     double acc[12];
 #pragma unroll
     for (int j = 0; j < 12; j++) acc[j] = 0.0;
-    // a share takes B consecutive points at a time: thread (d, b) the phase of point b
-    const int step = FCL * nsub * B;
+    // a share takes BT consecutive points at a time: thread (d, q) the phase of point q
+    const int step = FCL * nsub * BT;
     for (int p0 = 0; p0 < npts; p0 += step) {
-        const int first = p0 + (rk * nsub + sub) * B, n = on ? max(0, min(B, npts - first)) : 0;
-        if (b < n) {
-            const double* x = pts + 3 * (size_t)(first + b);
+        const int first = p0 + (rk * nsub + sub) * BT, n = on ? max(0, min(BT, npts - first)) : 0;
+        if (q < n) {
+            const double* x = pts + 3 * (size_t)(first + q);
             double sn, cs;
             sincos(k * (r[0] * x[0] + r[1] * x[1] + r[2] * x[2]), &sn, &cs);
             phase[t] = make_double2(cs, sn);
         }
         __syncthreads();
-        for (int i = 0; i < n; i++) {
-            const double2 e = phase[t - b + i];
-            const double* v = cur + (size_t)(first + i) * 12 * B + b;
+        if (wave)
+            for (int i = 0; i < n; i++) {
+                const double2 e = phase[t - q + i];
+                const double* v = cur + (size_t)(first + i) * 12 * B + b;
 #pragma unroll
-            for (int j = 0; j < 6; j++) {
-                const double re = v[(2 * j) * B], im = v[(2 * j + 1) * B];
-                acc[2 * j] = fma(re, e.x, fma(-im, e.y, acc[2 * j]));
-                acc[2 * j + 1] = fma(re, e.y, fma(im, e.x, acc[2 * j + 1]));
+                for (int j = 0; j < 6; j++) {
+                    const double re = v[(2 * j) * B], im = v[(2 * j + 1) * B];
+                    acc[2 * j] = fma(re, e.x, fma(-im, e.y, acc[2 * j]));
+                    acc[2 * j + 1] = fma(re, e.y, fma(im, e.x, acc[2 * j + 1]));
+                }
             }
-        }
         __syncthreads();
     }
 #pragma unroll
     for (int j = 0; j < 12; j++) sums[j * FT + t] = acc[j];
-    __syncthreads();
-    double own[12];
-    if (t < G)
+    for (int m = nsub; m > 1;) {  // the upper half of the shares onto the lower
+        const int half = (m + 1) / 2;
+        __syncthreads();
+        if (sub < m - half)
 #pragma unroll
-        for (int j = 0; j < 12; j++) {
-            double s = 0.0;
-            for (int u = 0; u < nsub; u++) s += sums[j * FT + u * G + t];
-            own[j] = s;
-        }
-    __syncthreads();
-    if (t < G)
-#pragma unroll
-        for (int j = 0; j < 12; j++) sums[j * FT + t] = own[j];
+            for (int j = 0; j < 12; j++) sums[j * FT + t] += sums[j * FT + t + half * G];
+        m = half;
+    }
     cl.sync();
-    if (t < G && t % FCL == rk && dir < ndir) {
+    if (t < G && t % FCL == rk && dir < ndir && wave) {
         double v[12];
 #pragma unroll
         for (int j = 0; j < 12; j++) {
             v[j] = 0.0;
-            for (int q = 0; q < FCL; q++) v[j] += cl.map_shared_rank(sums, q)[j * FT + t];
+            for (int u = 0; u < FCL; u++) v[j] += cl.map_shared_rank(sums, u)[j * FT + t];
         }
         double out[6];
         for (int part = 0; part < 2; part++) {  // real, imag
@@ -861,14 +864,26 @@ void launch_pack_cur(mot_handle* h, double* out, cudaStream_t s) {
 
 void launch_far_field(mot_handle* h, int n_dir, const double* dirs, double* E, cudaStream_t s) {
     if (h->B * h->nfreq * n_dir == 0) return;
-    const int DT = std::max(1, std::min(8, FT / h->B));
     const size_t nb = (size_t)h->npad * h->B;
-    for (int f = 0; f < h->nfreq; f++) {
-        k_point_currents<<<(h->npts * h->B + 127) / 128, 128, 0, s>>>(h->npts, h->npad, h->B, h->nq, h->d_ptptr,
-                                                                      h->d_ptent, h->d_rhs_wf,
-                                                                      h->d_dft + (size_t)f * 4 * nb * 2, h->d_ptcur);
+    int nsm = 148;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    for (int f0 = 0; f0 < h->nfreq; f0 += h->ptcur_freqs) {
+        const int nf = std::min(h->ptcur_freqs, h->nfreq - f0);
+        // A cluster takes all waves, for which its phases then serve, unless that leaves SMs idle
+        // (one direction and frequency, 64 waves at 480 edges: a call takes 590 us with all of them
+        // in eight CTAs, 125 us at eight waves a cluster); then directions, up to a warp of
+        // (direction, wave) pairs or eight, which cost no phases but share a cluster's reductions.
+        auto ctas = [&](int bt, int dt) {
+            return (long long)((h->B + bt - 1) / bt) * ((n_dir + dt - 1) / dt) * nf * FCL;
+        };
+        int BT = h->B, DT = 1;
+        while (BT > 8 && ctas(BT, 1) < 2 * nsm) BT = (BT + 1) / 2;
+        while (2 * DT <= std::min(8, n_dir) && DT * BT < 32 && ctas(BT, 2 * DT) >= 2 * nsm) DT *= 2;
+        k_point_currents<<<dim3((h->npts * h->B + 127) / 128, nf), 128, 0, s>>>(
+            h->npts, h->npad, h->B, h->nq, h->d_ptptr, h->d_ptent, h->d_rhs_wf, h->d_dft + (size_t)f0 * 4 * nb * 2,
+            h->d_ptcur);
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((n_dir + DT - 1) / DT * FCL);
+        cfg.gridDim = dim3((n_dir + DT - 1) / DT * FCL, (h->B + BT - 1) / BT, nf);
         cfg.blockDim = dim3(FT);
         cfg.stream = s;
         cudaLaunchAttribute at[1];
@@ -877,7 +892,7 @@ void launch_far_field(mot_handle* h, int n_dir, const double* dirs, double* E, c
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_far_field, h->npts, h->B, h->nfreq, f, n_dir, DT, (const double*)h->d_pts,
+        cudaLaunchKernelEx(&cfg, k_far_field, h->npts, h->B, h->nfreq, f0, n_dir, DT, BT, (const double*)h->d_pts,
                            (const double*)h->d_ptcur, (const double*)h->d_omega, dirs, (const double*)h->d_waves, h->c,
                            h->eta, E);
         h->launches += 2;

@@ -21,6 +21,10 @@
 #define MOT_TC_MAX_JOBS 32
 // Preconditioned Krylov vectors M V_j kept by a GMRES solve.
 #define MOT_GM_ZCAP 12
+// Bytes of point currents the far field keeps at most (at least one frequency's):
+// more frequencies than that go in turn. 64 MB is half of L2 and 31 frequencies of
+// 480 edges and 10 waves, whose clusters fill the chip for any number of directions.
+#define MOT_PTCUR_BYTES ((size_t)64 << 20)
 // Size (doubles) of the fixed device array used by mot_fields_noalloc.
 #define MOT_NOALLOC_FIELD_DOUBLES 262144
 
@@ -116,7 +120,8 @@ struct mot_handle {
     int* d_ptidx = nullptr;        // [npad][nq] point of every entry of the table
     int* d_ptptr = nullptr;        // [npts+1] entries (row * nq + q) of the table at each point ..
     int* d_ptent = nullptr;        // .. [ne * nq]
-    double* d_ptcur = nullptr;     // [npts][12][B] point currents of one frequency (far field)
+    double* d_ptcur = nullptr;     // [ptcur_freqs][npts][12][B] point currents (far field)
+    int ptcur_freqs = 1;           // frequencies it holds at a time
     double* d_ptfield = nullptr;   // [npts][2][B] incident field integrals of the step
 
     // block-sparse history
