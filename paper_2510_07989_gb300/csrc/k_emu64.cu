@@ -390,22 +390,25 @@ __device__ __forceinline__ double scale2(double v, int e) {
                                                              : ldexp(v, e);
 }
 
-// Y = the S partial products, summed in order in compensated FP32 (the pairs carry
-// 48 bits, the slices 41 at most), times the row's and the column's scale
+// Y = the S partial products, summed in order without loss in three FP32 terms (an
+// FP64 sum's additions and conversions run in a unit of two operations per clock
+// and SM), times the row's and the column's scale
 __global__ void __launch_bounds__(256) k_emu_reduce(int M, int N, int S, const float2* __restrict__ W,
                                                     const int* __restrict__ ea, const int* __restrict__ ex,
                                                     double* __restrict__ Y) {
     const size_t n = (size_t)M * N;
     for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
-        float hi = 0.f, lo = 0.f;
+        float hi = 0.f, lo = 0.f, tail = 0.f;
 #pragma unroll 4
         for (int z = 0; z < S; z++) {
             const float2 w = W[(size_t)z * n + i];
-            twosum(hi, lo, w.x);
-            lo += w.y;
+            float e = 0.f;
+            twosum(hi, e, w.x);
+            twosum(lo, tail, e);
+            twosum(lo, tail, w.y);
         }
         const int r = (int)(i / N), c = (int)(i - (size_t)r * N);
-        Y[i] = scale2((double)hi + (double)lo, ea[r] + ex[c] - 12);
+        Y[i] = scale2((double)hi + ((double)lo + (double)tail), ea[r] + ex[c] - 12);
     }
 }
 
