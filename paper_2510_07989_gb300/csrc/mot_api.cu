@@ -732,9 +732,9 @@ int do_step(mot_handle* h, cudaStream_t s, int phases = STEP_ALL) {
         for (int sweep = 0; sweep < max_sweeps; sweep++) {
             apply_q0_dense64(h, W.x, W.r, s);
             launch_axpby(h, n, 1.0, W.b, -1.0, W.r, W.r, s);
-            // the correction's solve goes on to two digits below what is asked of the step's, or
-            // six digits below its own right-hand side
-            const int st2 = gmres(h, W, W.b, W.x, W.r, prec, 1e-2 * h->opt.gmres_tol, GM_REFINE, s);
+            // the correction's solve goes on to six digits below its own right-hand side, in every
+            // wave (gmres: kind GM_REFINE), however good the wave's first solve was
+            const int st2 = gmres(h, W, W.b, W.x, W.r, prec, 0.0, GM_REFINE, s);
             if (st2 != MOT_OK && st2 != MOT_ENOCONV) return st2;
             if (h->last_gmres_resid <= h->opt.gmres_tol) break;
             h->refine_sweeps++;

@@ -61,3 +61,22 @@ def test_fp64_solve_through_a_restart(M, torus, B):
     ops, exc, ref = torus
     s = M.Solver(ops, gmres_maxit=800)
     assert err(first_step(M, s, ops, exc, B), ref[:B]) < COND * 2e-13
+
+
+def test_correction_gains_six_digits_whatever_the_tolerance(M):
+    """gmres_tol says when a step's residual needs no (further) correction; a
+    correction that is made goes six digits below its residual. Without the
+    preconditioner the first solve ends between 1e-7 and 1e-6, so the step is within
+    4e-12 (the correction, and the emulated products of the two right-hand sides)
+    times the condition number of Q_0, here 250."""
+    ops = assemble(MS.torus(1.0, 0.3, 9, 5), 4.0, 1.0, 0.3)
+    exc = MS.fibonacci_batch(8, ops.dt, w_steps=20, t0_steps=4, r_obj=1.3)
+    S = P.ProductSystem(ops)
+    Q = np.array([S.q0(c) for c in np.eye(2 * ops.ne)]).T
+    ref = np.array([np.linalg.solve(Q, S.left(*O.rhs_parts(ops, exc, b, 1))) for b in range(8)])
+    flags = M.MOT_MIX_DEFAULT & ~M.MOT_MIX_PRECOND
+    s = M.Solver(ops, precision=M.MOT_PREC_MIXED, mixed_flags=flags, gmres_tol=1e-7)
+    out = np.zeros((8, 2, ops.ne))
+    assert M.mot_step(s.h, M.mot_waves(exc), 8, out) == M.MOT_OK
+    assert s.info()["last_gmres_resid"] > 1e-7
+    assert err(out.reshape(8, -1), ref) < 250 * 4e-12
