@@ -1498,6 +1498,10 @@ int precompute_mixed(mot_handle* h) {
             return st;
         CK(cudaDeviceSynchronize());
     }
+    // the left factor's two inverses: a step applies the dense [M1 | M2]
+    dfree(h, h->d_Ginvf);
+    dfree(h, h->d_Lvinvf);
+    h->d_Ginvf = h->d_Lvinvf = nullptr;
     if (h32) {  // the FP64 lag-0 tiles (the dense Q_0 assembly's input) are no longer read
         dfree(h, h->d_tiles);
         dfree(h, h->d_tmask);

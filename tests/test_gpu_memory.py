@@ -102,3 +102,20 @@ def test_march_where_the_dense_operators_do_not_fit(M, larger, kw, when):
     assert t.info()["device_bytes"] < loaded + state - q0
     assert t.noconv == 0
     assert np.abs(W - ref).max() < 1e-10 * np.abs(ref).max()
+
+
+def test_mixed_handle_holds_what_its_march_reads(M, larger):
+    """The FP32 history without tensor cores or preconditioner: dense Q_0 and
+    [M1 | M2] in both precisions, T_0, tiles, column orders and the face inverse, and
+    beside them the split workspace (64 x 32 tiles of doubles, four CTAs per SM), 32
+    bytes a tile for the task lists and a megabyte of tables: no Gram inverse (7.2 MB),
+    which only the load needs."""
+    import torch
+    ops = larger
+    s = M.Solver(ops, precision=M.MOT_PREC_MIXED, mixed_flags=M.MOT_MIX_HIST32 | M.MOT_MIX_Q032)
+    q = s.info()
+    n, f = (ops.ne + 31) // 32 * 32, (ops.mesh.nf + 63) // 64 * 64
+    dense = 12 * (2 * n) ** 2 + 12 * n * 2 * n + 2 * 8 * n ** 2 + 4 * f ** 2
+    tiles = (4 * 1024 + 32) * q["tile_count"] + 4 * n * (n // 32)
+    split = 4 * torch.cuda.get_device_properties(0).multi_processor_count * 64 * 32 * 8
+    assert dense < q["device_bytes"] < dense + tiles + split + (1 << 20)
