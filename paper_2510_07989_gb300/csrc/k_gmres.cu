@@ -1,6 +1,6 @@
 // Batched GMRES of the Q_0 solve (paper Eq. (MOT)): one launch starts a cycle,
-// one launch orthogonalises a new Krylov vector and updates the least-squares
-// problem, one solves it, one combines the basis.
+// one launch (in long solves eight) orthogonalises a new Krylov vector and updates
+// the least-squares problem, one solves it, one combines the basis.
 //
 // System b of the batch uses columns b and B + b of a block vector
 // [npad][2B]. A thread-block cluster owns G systems (4, so that a row's
@@ -154,6 +154,42 @@ __device__ __forceinline__ double combine(const double* V, size_t vs, int nv, in
 // Below this squared norm a vector of an O(1) system is a breakdown: its system is done.
 constexpr double TINY2 = 1e-300;
 
+// End of iteration j for system sys: the new column h(0 .. j), |w| (n2 its square, inv
+// its inverse or 0) of the Hessenberg matrix rotated, the residual, and whether the
+// system is done. cs(i), sn(i): the earlier rotations; gj, ibn, floor_r: g_j, 1 / |b|
+// and the residual at which it is done.
+template <class H, class C, class D>
+__device__ __forceinline__ void new_column(const GmState& S, int sys, int j, H h, C cs, D sn, double n2, double inv,
+                                           double gj, double ibn, double floor_r) {
+    double* Hb = S.H + (size_t)sys * (S.m + 1) * S.m;
+    double a = h(0);
+    for (int i = 0; i < j; i++) {
+        const double x = h(i + 1), cc = cs(i), ss = sn(i);
+        Hb[(size_t)i * S.m + j] = cc * a + ss * x;
+        a = -ss * a + cc * x;
+    }
+    n2 = fmax(n2, 0.0);
+    const double nrm = n2 > TINY2 ? n2 * inv : sqrt(n2);
+    const double d2 = fma(a, a, n2);  // all O(1) or less: b is scaled to O(1)
+    double d = 0.0, cc = 1.0, ss = 0.0;
+    if (d2 > 0.0) {
+        const double id = rsqrt(d2);
+        d = d2 * id;
+        cc = a * id;
+        ss = nrm * id;
+    }
+    S.cs[(size_t)sys * S.m + j] = cc;
+    S.sn[(size_t)sys * S.m + j] = ss;
+    Hb[(size_t)j * S.m + j] = d;
+    double* gb = S.g + (size_t)sys * (S.m + 1);
+    gb[j + 1] = -ss * gj;
+    gb[j] = cc * gj;
+    const double rr = fabs(ss * gj) * ibn;
+    S.resid[sys] = rr;
+    S.jend[sys] = j + 1;
+    if (rr <= floor_r || !(nrm > 0.0)) S.active[sys] = 0;
+}
+
 // Start of a cycle: beta = |r| per system, V_0 = r / beta. On the first cycle
 // also the reference norm |b| (b == r: one vector).
 template <int G>
@@ -300,36 +336,118 @@ __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const do
         const double x = (SM ? ws[l] : w[ix]) - combine<G>(V, vs, nv, ix, h2, l % G);
         Vnext[ix] = iv != 0.0 ? x * iv : 0.0;
     }
-    if (rk == 0 && live) {
-        double* Hb = S.H + (size_t)sys * (S.m + 1) * S.m;
-        double a = h1[t] + h2[t];
-        for (int i = 0; i < j; i++) {
-            const double x = h1[(i + 1) * G + t] + h2[(i + 1) * G + t];
-            const double cc = rot[i * G + t], ss = rot[(j + i) * G + t];
-            Hb[(size_t)i * S.m + j] = cc * a + ss * x;
-            a = -ss * a + cc * x;
-        }
-        const double n2 = fmax(n2_s[t], 0.0), nrm = n2 > TINY2 ? n2 * inv_s[t] : sqrt(n2);
-        const double d2 = fma(a, a, n2);  // all O(1) or less: b is scaled to O(1)
-        double d = 0.0, cc = 1.0, ss = 0.0;
-        if (d2 > 0.0) {
-            const double id = rsqrt(d2);
-            d = d2 * id;
-            cc = a * id;
-            ss = nrm * id;
-        }
-        S.cs[(size_t)sys * S.m + j] = cc;
-        S.sn[(size_t)sys * S.m + j] = ss;
-        Hb[(size_t)j * S.m + j] = d;
-        double* gb = S.g + (size_t)sys * (S.m + 1);
-        gb[j + 1] = -ss * gj;
-        gb[j] = cc * gj;
-        const double rr = fabs(ss * gj) * ibn;
-        S.resid[sys] = rr;
-        S.jend[sys] = j + 1;
-        if (rr <= floor_r || !(nrm > 0.0)) S.active[sys] = 0;
-    }
+    if (rk == 0 && live)
+        new_column(S, sys, j, [&](int i) { return h1[i * G + t] + h2[i * G + t]; },
+                   [&](int i) { return rot[i * G + t]; }, [&](int i) { return rot[(j + i) * G + t]; }, n2_s[t],
+                   inv_s[t], gj, ibn, floor_r);
     c.barrier_wait();  // ... and they of this one's
+}
+
+// The same iteration in launches over the whole chip, for long ones (launch_gm_iter).
+// partial[chunk][v * B + b] = the chunk of rows' part of <V_v, w>_b, v < nv: four
+// vectors a CTA, its threads (row of a stride, system).
+constexpr int DT = 256;
+__global__ void __launch_bounds__(DT) k_gm_dots(int npad, int B, int rows, const double* __restrict__ V, size_t vs,
+                                                int nv, const double* __restrict__ w, double* __restrict__ partial) {
+    __shared__ double red[4][DT];
+    const int t = threadIdx.x, RS = DT / B, rs = t / B, b = t - rs * B, v0 = blockIdx.y * 4, nl = min(4, nv - v0);
+    const int r1 = min(npad, (int)(blockIdx.x + 1) * rows);
+    double p[4] = {0.0, 0.0, 0.0, 0.0};
+    if (rs < RS)
+#pragma unroll 4
+        for (int r = blockIdx.x * rows + rs; r < r1; r += RS) {
+            const size_t ix = (size_t)r * 2 * B + b;
+            const double x = w[ix], y = w[ix + B];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {  // past the last vector its values again, not used
+                const double* v = V + (size_t)(v0 + min(i, nl - 1)) * vs + ix;
+                p[i] = fma(v[B], y, fma(v[0], x, p[i]));
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < 4; i++) red[i][t] = p[i];
+    for (int m = RS; m > 1;) {  // the upper half of the row strides onto the lower
+        const int half = (m + 1) / 2;
+        __syncthreads();
+        if (rs < m - half)
+#pragma unroll
+            for (int i = 0; i < 4; i++) red[i][t] += red[i][t + half * B];
+        m = half;
+    }
+    __syncthreads();
+    for (int i = t; i < nl * B; i += DT)
+        partial[(size_t)blockIdx.x * nv * B + v0 * B + i] = red[i / B][i % B];
+}
+
+// h[i] = the chunks' partials of sum i, in order
+__global__ void __launch_bounds__(128) k_gm_dots_sum(int n, int chunks, const double* __restrict__ partial,
+                                                     double* __restrict__ h) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < chunks; c++) s += partial[(size_t)c * n + i];
+    h[i] = s;
+}
+
+// w -= sum_v V_v h[v][b]
+__global__ void __launch_bounds__(128) k_gm_update(int n, int B, const double* __restrict__ V, size_t vs, int nv,
+                                                   const double* __restrict__ h, double* __restrict__ w) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const int b = i % B;
+    double s0 = 0.0, s1 = 0.0;
+    int v = 0;
+#pragma unroll 4
+    for (; v + 2 <= nv; v += 2) {
+        s0 = fma(V[(size_t)v * vs + i], h[v * B + b], s0);
+        s1 = fma(V[(size_t)(v + 1) * vs + i], h[(v + 1) * B + b], s1);
+    }
+    if (v < nv) s0 = fma(V[(size_t)v * vs + i], h[v * B + b], s0);
+    w[i] -= s0 + s1;
+}
+
+// |w| of system blockIdx.x, its new column (coefficients h1 + h2) and the factor
+// that makes V_{j+1} of w: 0 for a system that is done
+__global__ void __launch_bounds__(DT) k_gm_column(int npad, int B, int j, const double* __restrict__ w,
+                                                  const double* __restrict__ h1, const double* __restrict__ h2,
+                                                  double tol, double gain, GmState S, double* __restrict__ inv) {
+    extern __shared__ double sm[];
+    double *h = sm, *cs = h + j + 1, *sn = cs + j;  // j + 1, j, j
+    __shared__ double red[DT / 32];
+    const int b = blockIdx.x, t = threadIdx.x;
+    for (int i = t; i <= j; i += DT) h[i] = h1[i * B + b] + h2[i * B + b];
+    for (int i = t; i < j; i += DT) {
+        cs[i] = S.cs[(size_t)b * S.m + i];
+        sn[i] = S.sn[(size_t)b * S.m + i];
+    }
+    double s = 0.0;
+#pragma unroll 8
+    for (int r = t; r < 2 * npad; r += DT) {
+        const double x = w[(size_t)r * B + b];
+        s = fma(x, x, s);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if ((t & 31) == 0) red[t >> 5] = s;
+    __syncthreads();
+    if (t > 0) return;
+    double n2 = 0.0;
+    for (int i = 0; i < DT / 32; i++) n2 += red[i];
+    const bool live = S.active[b] != 0;
+    const double iv = live && n2 > TINY2 ? rsqrt(n2) : 0.0;
+    inv[b] = iv;
+    if (live)
+        new_column(S, b, j, [&](int i) { return h[i]; }, [&](int i) { return cs[i]; }, [&](int i) { return sn[i]; }, n2,
+                   iv, S.g[(size_t)b * (S.m + 1) + j], 1.0 / S.bnorm[b], fmax(tol, gain * S.resid0[b]));
+}
+
+__global__ void __launch_bounds__(128) k_gm_scale(int n, int B, const double* __restrict__ w,
+                                                  const double* __restrict__ inv, double* __restrict__ Vnext) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const double iv = inv[i % B];
+    Vnext[i] = iv != 0.0 ? w[i] * iv : 0.0;
 }
 
 // y = H^{-1} g (upper triangular, size jend[b]) into y[i][b], i < nv (0 past
@@ -422,6 +540,41 @@ Shape shape_of(const mot_handle* h, int per) {
 
 namespace mot {
 
+// An iteration is one cluster launch below LONG elements times vectors a CTA, and
+// the eight launches of long_iter from there on: a cluster's groups of four systems
+// run on eight SMs each (16 SMs for 8 waves), whose FP64 units and load latency
+// grow with elements times vectors (1296 edges, 8 waves: 124 us at 30 vectors),
+// where eight launches over the whole chip stay near their 30 us. A step with 38
+// to 40 iterations without preconditioner (mixed, 2 / 8 / 64 waves): 1296 edges
+// 9.3 / 8.3 / 11.5 ms, in cluster launches only 12.6 / 11.7 / 15.0; 2160 edges 16.5 /
+// 12.4 / 17.5 and 24.9 / 20.4 / 25.9. At 8192 the solves of 120 and 270 edges
+// (22 to 50 iterations) took 3 to 11 % longer, at 16384 they take as long.
+constexpr long long LONG = 16384;
+
+static void long_iter(mot_handle* h, int j, double* w, double tol, double gain, double* work, size_t work_size,
+                      cudaStream_t s) {
+    const int B = h->B, nv = j + 1, n = nv * B, el = h->npad * 2 * B, groups = (nv + 3) / 4;
+    const size_t vs = (size_t)el;
+    int nsm = 148;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    // chunks of whole row strides, about four CTAs an SM in all, at most 64 to be summed
+    const int RS = DT / B, strides = (h->npad + RS - 1) / RS;
+    const size_t room = work_size - 2 * (size_t)n - B;
+    int chunks = std::max(1, std::min({4 * nsm / groups, 64, strides, (int)(room / n)}));
+    const int rows = (strides + chunks - 1) / chunks * RS;
+    chunks = (h->npad + rows - 1) / rows;
+    double *h1 = work, *h2 = h1 + n, *inv = h2 + n, *partial = inv + B;
+    for (double* hh : {h1, h2}) {
+        k_gm_dots<<<dim3(chunks, groups), DT, 0, s>>>(h->npad, B, rows, h->d_V, vs, nv, w, partial);
+        k_gm_dots_sum<<<(n + 127) / 128, 128, 0, s>>>(n, chunks, partial, hh);
+        k_gm_update<<<(el + 127) / 128, 128, 0, s>>>(el, B, h->d_V, vs, nv, hh, w);
+    }
+    k_gm_column<<<B, DT, sizeof(double) * (3 * (size_t)j + 1), s>>>(h->npad, B, j, w, h1, h2, tol, gain, state_of(h),
+                                                                    inv);
+    k_gm_scale<<<(el + 127) / 128, 128, 0, s>>>(el, B, w, inv, h->d_V + (size_t)(j + 1) * vs);
+    h->launches += 8;
+}
+
 void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r, double* V0, cudaStream_t s) {
     const Shape p = shape_of(h, 2048);
     launch_cluster(p.G == 1 ? k_gm_begin<1> : k_gm_begin<4>, p.groups, p.cl, 0, s, h->npad, h->B, b, first ? 1 : 0, r,
@@ -429,9 +582,14 @@ void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r
     h->launches++;
 }
 
-void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, cudaStream_t s) {
+void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, double* work, size_t work_size,
+                    cudaStream_t s) {
     set_attributes(h);
     const Shape p = shape_of(h, 512);
+    if (p.per_cta * (j + 1) >= LONG) {
+        long_iter(h, j, w, tol, gain, work, work_size, s);
+        return;
+    }
     const size_t vs = (size_t)h->npad * 2 * h->B;
     const int n = (j + 1) * p.G;
     const bool sm = p.per_cta <= SLICE;

@@ -177,7 +177,8 @@ struct Work {
     double *Y4, *GY4, *X4, *PX4;  // 4B-column block vectors
     double *q1, *q2, *t1, *t2, *dd, *pd;
     double *fvec, *zvec;      // faces / vertices x 4B
-    double *cgw;              // CG scratch 4 x maxN x 4B
+    double *cgw;              // scratch 4 x maxN x 4B of the projector and Gram solves and of a long
+    size_t ncgw;              // GMRES iteration, and its size
     double *ygm;
 };
 
@@ -219,7 +220,8 @@ Work work_of(mot_handle* h) {
     W.pd = take(bv);
     W.fvec = take((size_t)std::max(h->nf, h->nv) * 4 * h->B);
     W.zvec = take((size_t)std::max(h->nf, h->nv) * 4 * h->B);
-    W.cgw = take((size_t)4 * maxN * 4 * h->B);
+    W.ncgw = (size_t)4 * maxN * 4 * h->B;
+    W.cgw = take(W.ncgw);
     const size_t gm = (size_t)(h->gm_m + 1) * h->B;
     W.ygm = take(gm);
     return W;
@@ -404,7 +406,7 @@ int gmres(mot_handle* h, const Work& W, const double* b, double* x, const double
         for (int j = 0; j < m && total < maxit && !converged; j++) {
             double* mv = !prec ? nullptr : j < zcap ? h->d_Z + (size_t)j * bv : W.q1;
             apply_q0(h, W, h->d_V + (size_t)j * bv, W.w, s, mv);
-            launch_gm_iter(h, j, W.w, tol, kind == GM_REFINE ? 1e-6 : 0.0, s);
+            launch_gm_iter(h, j, W.w, tol, kind == GM_REFINE ? 1e-6 : 0.0, W.cgw, W.ncgw, s);
             jend = j + 1;
             total++;
             if (total >= h->gm_pred[kind] || jend == m || total == maxit) {

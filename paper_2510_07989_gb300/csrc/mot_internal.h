@@ -336,8 +336,9 @@ void launch_pack_w(mot_handle* h, const double* x, double* out, cudaStream_t s);
 // start of a cycle: V0 = r / |r| per system; first: also the reference norms |b|
 void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r, double* V0, cudaStream_t s);
 // iteration j: w = Q_0 V_j orthogonalised, V_{j+1}, rotated Hessenberg column, residual against
-// tol |b| and gain |r0|
-void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, cudaStream_t s);
+// tol |b| and gain |r0|; work: scratch of work_size doubles, at least 4 (j + 2) B
+void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, double* work, size_t work_size,
+                    cudaStream_t s);
 // x = (add ? x : 0) + sum_{v < nv} Z_v y_v, y the least-squares solution
 void launch_gm_finish(mot_handle* h, const double* Z, int nv, bool add, double* y, double* x, cudaStream_t s);
 // power-of-two scale of every wave's system (sc[b] = 2^-e) and its application

@@ -80,3 +80,17 @@ def test_correction_gains_six_digits_whatever_the_tolerance(M):
     assert M.mot_step(s.h, M.mot_waves(exc), 8, out) == M.MOT_OK
     assert s.info()["last_gmres_resid"] > 1e-7
     assert err(out.reshape(8, -1), ref) < 250 * 4e-12
+
+
+@pytest.mark.parametrize("B", [3, 7, 33, 64])
+def test_long_iterations_over_batches(M, B):
+    """Solves of 100 vectors and more, whose iterations change from one launch to
+    several on the way (here at 32 vectors): batches that fill the threads of a row
+    stride or leave some over."""
+    ops = assemble(MS.torus(1.0, 0.3, 10, 5), 2.0, 100.0, 1.0)
+    exc = MS.fibonacci_batch(B, ops.dt, w_steps=20, t0_steps=4, r_obj=1.3)
+    S = P.ProductSystem(ops)
+    Q = np.array([S.q0(c) for c in np.eye(2 * ops.ne)]).T
+    ref = np.linalg.solve(Q, np.array([S.left(*O.rhs_parts(ops, exc, b, 1)) for b in range(B)]).T).T
+    s = M.Solver(ops, gmres_maxit=800)
+    assert err(first_step(M, s, ops, exc, B), ref) < COND * 2e-13
