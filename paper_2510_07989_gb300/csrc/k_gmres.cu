@@ -24,7 +24,6 @@ namespace cg = cooperative_groups;
 
 constexpr int GT = 256;      // threads per CTA
 constexpr int NW = GT / 32;
-constexpr int SLICE = 12288; // elements of the new vector a CTA keeps in shared memory
 constexpr int MAXCL = 8;     // CTAs per cluster (the portable limit)
 
 struct GmState {
@@ -108,9 +107,9 @@ __device__ __forceinline__ int shares(int groups) { return groups >= NW ? 1 : NW
 // of the elements: sixteen loads in flight a lane. (All warps over the same
 // vectors, eight at a time: 46 us an iteration at 1920 edges, B = 1, 17 vectors
 // on average.)
-template <int G, bool SM>
+template <int G>
 __device__ __forceinline__ void dots(const Part<G>& P, int L, const double* V, size_t vs, int nv, bool norm,
-                                     const double* w, const double* ws, double* red) {
+                                     const double* ws, double* red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ns = nv + (norm ? 1 : 0), n = ns * G, ng = (ns + 3) / 4, parts = shares(ng);
     for (int gi = warp; gi < ng * parts; gi += NW) {
@@ -120,8 +119,8 @@ __device__ __forceinline__ void dots(const Part<G>& P, int L, const double* V, s
         for (int l = share * 32 + lane; l < L; l += parts * 32) {
             // no branch, so that the unrolled loads go out together: past the
             // vector's end x is 0
-            const int at = P.at(l), ix = at < 0 ? 0 : at;
-            const double x = SM ? ws[l] : at < 0 ? 0.0 : w[ix];
+            const int ix = max(P.at(l), 0);
+            const double x = ws[l];
 #pragma unroll
             for (int i = 0; i < 4; i++)
                 if (v0 + i < ns) p[i] = fma(v0 + i < nv ? V[(size_t)(v0 + i) * vs + ix] : x, x, p[i]);
@@ -250,9 +249,9 @@ __global__ void __launch_bounds__(GT) k_gm_begin(int npad, int B, const double* 
 // of tol |b|, or of gain times its residual at the start. A system that is done
 // writes V_{j+1} = 0 from its next iteration on and keeps its state, so
 // iterations past its end change nothing.
-template <int G, bool SM>
+template <int G>
 __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const double* __restrict__ V, size_t vs,
-                                                double* __restrict__ w, double* __restrict__ Vnext, double tol,
+                                                const double* __restrict__ w, double* __restrict__ Vnext, double tol,
                                                 double gain, GmState S) {
     extern __shared__ double sm[];
     __shared__ double inv_s[G], n2_s[G];
@@ -267,7 +266,7 @@ __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const do
     double* h2 = h1 + n;             // n + G: coefficients, |w|^2
     double* sq = h2 + n + G;         // G
     double* rot = sq + G;            // 2 x j x G: cosines, sines of the earlier rotations
-    double* ws = rot + 2 * j * G;    // L (SM)
+    double* ws = rot + 2 * j * G;    // L: this CTA's part of the new vector
     const int sys = P.g0 + t;        // of threads t < G
     const bool mine = t < G && sys < B;
     // read before the first barrier, written after the last by rank 0
@@ -285,23 +284,20 @@ __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const do
             floor_r = fmax(tol, gain * S.resid0[sys]);
         }
     }
-    if (SM)
-        for (int l = t; l < L; l += GT) {
-            const int ix = P.at(l);
-            ws[l] = ix >= 0 ? w[ix] : 0.0;
-        }
+    for (int l = t; l < L; l += GT) {
+        const int ix = P.at(l);
+        ws[l] = ix >= 0 ? w[ix] : 0.0;
+    }
     __syncthreads();
-    dots<G, SM>(P, L, V, vs, nv, false, w, ws, red);
+    dots<G>(P, L, V, vs, nv, false, ws, red);
     cluster_sums(n, shares((nv + 3) / 4), red, part, h1, cl);
     for (int l = t; l < L; l += GT) {
         const int ix = P.at(l);
         if (ix < 0) continue;
-        const double s = combine<G>(V, vs, nv, ix, h1, l % G);
-        if (SM) ws[l] -= s;
-        else w[ix] -= s;
+        ws[l] -= combine<G>(V, vs, nv, ix, h1, l % G);
     }
     __syncthreads();
-    dots<G, SM>(P, L, V, vs, nv, true, w, ws, red);
+    dots<G>(P, L, V, vs, nv, true, ws, red);
     cluster_sums(n + G, shares((nv + 4) / 4), red, part + n, h2, cl);
     if (t < G) {
         double s = h2[n + t], m = s;
@@ -318,7 +314,7 @@ __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const do
         for (int l = t; l < L; l += GT) {
             const int ix = P.at(l);
             if (ix < 0) continue;
-            const double x = (SM ? ws[l] : w[ix]) - combine<G>(V, vs, nv, ix, h2, l % G);
+            const double x = ws[l] - combine<G>(V, vs, nv, ix, h2, l % G);
             p[0] = fma(x, x, p[0]);
         }
         const double s = warp_sum4<G>(p);
@@ -333,7 +329,7 @@ __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const do
         const int ix = P.at(l);
         if (ix < 0) continue;
         const double iv = inv_s[l % G];
-        const double x = (SM ? ws[l] : w[ix]) - combine<G>(V, vs, nv, ix, h2, l % G);
+        const double x = ws[l] - combine<G>(V, vs, nv, ix, h2, l % G);
         Vnext[ix] = iv != 0.0 ? x * iv : 0.0;
     }
     if (rk == 0 && live)
@@ -512,10 +508,8 @@ void set_attributes(mot_handle* h) {
     static std::atomic<unsigned long long> attr{0};
     mot::once_per_device(attr, h->dev, [] {
         const int mx = 200 * 1024;
-        cudaFuncSetAttribute(k_gm_iter<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_gm_iter<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_gm_iter<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_gm_iter<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_gm_iter<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_gm_iter<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         cudaFuncSetAttribute(k_gm_back, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     });
 }
@@ -592,12 +586,9 @@ void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, do
     }
     const size_t vs = (size_t)h->npad * 2 * h->B;
     const int n = (j + 1) * p.G;
-    const bool sm = p.per_cta <= SLICE;
     const size_t smem = sizeof(double) * ((size_t)NW * (n + p.G) + 4 * n + 4 * p.G + 2 * (size_t)j * p.G +
-                                          (sm ? (size_t)p.per_cta : 0));
-    auto* k = p.G == 1 ? (sm ? k_gm_iter<1, true> : k_gm_iter<1, false>)
-                       : (sm ? k_gm_iter<4, true> : k_gm_iter<4, false>);
-    launch_cluster(k, p.groups, p.cl, smem, s, h->npad, h->B, j, (const double*)h->d_V, vs, w,
+                                          (size_t)p.per_cta);  // LONG elements at most: 128 KB, 27 KB of the rest
+    launch_cluster(p.G == 1 ? k_gm_iter<1> : k_gm_iter<4>, p.groups, p.cl, smem, s, h->npad, h->B, j, (const double*)h->d_V, vs, (const double*)w,
                    h->d_V + (size_t)(j + 1) * vs, tol, gain, state_of(h));
     h->launches++;
 }
