@@ -176,7 +176,10 @@ __global__ void __launch_bounds__(PT) k_refine_solve(Problem Q, const double* __
     __syncthreads();
     const double thr = thr_s[c];
     int it = 0;
-    bool open = true, lost = false;  // lost: this thread saw a row that is no number
+    // lost: this thread saw a value that is no number (looked at as an integer: the FP64
+    // unit's comparisons cost what its multiply-adds do)
+    auto no_number = [](double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; };
+    bool open = true, lost = no_number(thr);
     while (open && it < maxit) {
         for (int i = t; i < N * CW; i += PT) rs[sidx(i / CW, i % CW)] = __ldcg(rg + i);
         __syncthreads();
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(PT) k_refine_solve(Problem Q, const double* __
             z[ix] += (double)__ldcg(d + ix);
             rg[ix] = (float)rn;
             mine |= fabs(rn) > thr;  // a row or threshold that is no number ends its column's sweeps ..
-            lost |= !(fabs(rn) <= INFINITY) || !(thr <= INFINITY);
+            lost |= no_number(rn);
         }
         if (mine) open_s[it & 1] = 1;
         cl.sync();
