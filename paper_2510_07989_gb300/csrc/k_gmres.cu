@@ -153,22 +153,12 @@ __device__ __forceinline__ double combine(const double* V, size_t vs, int nv, in
 // Below this squared norm a vector of an O(1) system is a breakdown: its system is done.
 constexpr double TINY2 = 1e-300;
 
-// End of iteration j for system sys: the new column h(0 .. j), |w| (n2 its square, inv
-// its inverse or 0) of the Hessenberg matrix rotated, the residual, and whether the
-// system is done. cs(i), sn(i): the earlier rotations; gj, ibn, floor_r: g_j, 1 / |b|
-// and the residual at which it is done.
-template <class H, class C, class D>
-__device__ __forceinline__ void new_column(const GmState& S, int sys, int j, H h, C cs, D sn, double n2, double inv,
-                                           double gj, double ibn, double floor_r) {
-    double* Hb = S.H + (size_t)sys * (S.m + 1) * S.m;
-    double a = h(0);
-    for (int i = 0; i < j; i++) {
-        const double x = h(i + 1), cc = cs(i), ss = sn(i);
-        Hb[(size_t)i * S.m + j] = cc * a + ss * x;
-        a = -ss * a + cc * x;
-    }
-    n2 = fmax(n2, 0.0);
-    const double nrm = n2 > TINY2 ? n2 * inv : sqrt(n2);
+// End of iteration j for system sys, whose new column the earlier rotations have
+// left at a (and above it in H), with |w| = nrm below: the new rotation, the
+// residual, and whether the system is done. gj, ibn, floor_r: g_j, 1 / |b| and the
+// residual at which it is done.
+__device__ __forceinline__ void new_column(const GmState& S, int sys, int j, double a, double n2, double nrm, double gj,
+                                           double ibn, double floor_r) {
     const double d2 = fma(a, a, n2);  // all O(1) or less: b is scaled to O(1)
     double d = 0.0, cc = 1.0, ss = 0.0;
     if (d2 > 0.0) {
@@ -179,7 +169,7 @@ __device__ __forceinline__ void new_column(const GmState& S, int sys, int j, H h
     }
     S.cs[(size_t)sys * S.m + j] = cc;
     S.sn[(size_t)sys * S.m + j] = ss;
-    Hb[(size_t)j * S.m + j] = d;
+    S.H[((size_t)sys * (S.m + 1) + j) * S.m + j] = d;
     double* gb = S.g + (size_t)sys * (S.m + 1);
     gb[j + 1] = -ss * gj;
     gb[j] = cc * gj;
@@ -332,10 +322,18 @@ __global__ void __launch_bounds__(GT) k_gm_iter(int npad, int B, int j, const do
         const double x = ws[l] - combine<G>(V, vs, nv, ix, h2, l % G);
         Vnext[ix] = iv != 0.0 ? x * iv : 0.0;
     }
-    if (rk == 0 && live)
-        new_column(S, sys, j, [&](int i) { return h1[i * G + t] + h2[i * G + t]; },
-                   [&](int i) { return rot[i * G + t]; }, [&](int i) { return rot[(j + i) * G + t]; }, n2_s[t],
-                   inv_s[t], gj, ibn, floor_r);
+    if (rk == 0 && live) {
+        double* Hb = S.H + (size_t)sys * (S.m + 1) * S.m;
+        double a = h1[t] + h2[t];
+        for (int i = 0; i < j; i++) {
+            const double x = h1[(i + 1) * G + t] + h2[(i + 1) * G + t];
+            const double cc = rot[i * G + t], ss = rot[(j + i) * G + t];
+            Hb[(size_t)i * S.m + j] = cc * a + ss * x;
+            a = -ss * a + cc * x;
+        }
+        const double n2 = fmax(n2_s[t], 0.0);
+        new_column(S, sys, j, a, n2, n2 > TINY2 ? n2 * inv_s[t] : sqrt(n2), gj, ibn, floor_r);
+    }
     c.barrier_wait();  // ... and they of this one's
 }
 
@@ -433,9 +431,16 @@ __global__ void __launch_bounds__(DT) k_gm_column(int npad, int B, int j, const 
     const bool live = S.active[b] != 0;
     const double iv = live && n2 > TINY2 ? rsqrt(n2) : 0.0;
     inv[b] = iv;
-    if (live)
-        new_column(S, b, j, [&](int i) { return h[i]; }, [&](int i) { return cs[i]; }, [&](int i) { return sn[i]; }, n2,
-                   iv, S.g[(size_t)b * (S.m + 1) + j], 1.0 / S.bnorm[b], fmax(tol, gain * S.resid0[b]));
+    if (!live) return;
+    double* Hb = S.H + (size_t)b * (S.m + 1) * S.m;
+    double a = h[0];
+    for (int i = 0; i < j; i++) {
+        const double x = h[i + 1], cc = cs[i], ss = sn[i];
+        Hb[(size_t)i * S.m + j] = cc * a + ss * x;
+        a = -ss * a + cc * x;
+    }
+    new_column(S, b, j, a, n2, n2 > TINY2 ? n2 * iv : sqrt(n2), S.g[(size_t)b * (S.m + 1) + j], 1.0 / S.bnorm[b],
+               fmax(tol, gain * S.resid0[b]));
 }
 
 __global__ void __launch_bounds__(128) k_gm_scale(int n, int B, const double* __restrict__ w,
