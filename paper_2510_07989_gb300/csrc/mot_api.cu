@@ -456,7 +456,8 @@ int alloc_state(mot_handle* h, int B) {
     h->d_ptfield = (double*)dalloc(h, sizeof(double) * 2 * (size_t)h->npts * B);
     if (h->nfreq > 0) {  // as many frequencies at a time as MOT_PTCUR_BYTES and the memory hold
         const size_t one = sizeof(double) * 12 * (size_t)std::max(1, h->npts) * B;
-        h->ptcur_freqs = (int)std::min<size_t>(h->nfreq, std::max<size_t>(1, MOT_PTCUR_BYTES / one));
+        const size_t most = std::min<size_t>(MOT_PTCUR_BYTES / one, 65535);  // a grid dimension of the far field
+        h->ptcur_freqs = (int)std::min<size_t>(h->nfreq, std::max<size_t>(1, most));
         while (!(h->d_ptcur = (double*)dalloc(h, one * h->ptcur_freqs)) && h->ptcur_freqs > 1) h->ptcur_freqs /= 2;
     }
     h->d_cur = (double*)dalloc(h, sizeof(double) * 4 * (size_t)h->npad * B);
