@@ -9,8 +9,8 @@
 // the cluster through distributed shared memory, in rank order (every CTA
 // gets the same sums). What bounds an iteration is latency: basis vectors from
 // L2, two cluster barriers, and chains of FP64 operations of a unit that does
-// two multiply-adds per clock and SM (a double-precision square root or
-// division costs a microsecond, so one thread per system does them).
+// two multiply-adds per clock and SM (square roots and divisions by one thread
+// per system, for the whole cluster).
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -523,8 +523,12 @@ struct Shape {
     int G, groups, cl;
     long long per_cta;  // elements
 };
-// Cluster size: about `per` elements per CTA, at most the portable eight CTAs.
-Shape shape_of(const mot_handle* h, int per) {
+// Cluster size: at most the portable eight CTAs, about 512 elements each, two a
+// thread: a cluster barrier costs less than a longer pass over the elements (at
+// 2048 an iteration of the first two takes 19.2 us for 14.0 at 216 edges, 8 waves,
+// 24.3 for 19.6 at 924 edges, 64 waves; the start of a cycle 5.4 for 4.7).
+Shape shape_of(const mot_handle* h) {
+    constexpr int per = 512;
     Shape p;
     p.G = h->B == 1 ? 1 : 4;
     p.groups = (h->B + p.G - 1) / p.G;
@@ -575,7 +579,7 @@ static void long_iter(mot_handle* h, int j, double* w, double tol, double gain, 
 }
 
 void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r, double* V0, cudaStream_t s) {
-    const Shape p = shape_of(h, 2048);
+    const Shape p = shape_of(h);
     launch_cluster(p.G == 1 ? k_gm_begin<1> : k_gm_begin<4>, p.groups, p.cl, 0, s, h->npad, h->B, b, first ? 1 : 0, r,
                    V0, state_of(h));
     h->launches++;
@@ -584,7 +588,7 @@ void launch_gm_begin(mot_handle* h, const double* b, bool first, const double* r
 void launch_gm_iter(mot_handle* h, int j, double* w, double tol, double gain, double* work, size_t work_size,
                     cudaStream_t s) {
     set_attributes(h);
-    const Shape p = shape_of(h, 512);
+    const Shape p = shape_of(h);
     if (p.per_cta * (j + 1) >= LONG) {
         long_iter(h, j, w, tol, gain, work, work_size, s);
         return;

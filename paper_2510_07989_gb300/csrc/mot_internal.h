@@ -19,7 +19,9 @@
 #define MOT_TC_CHUNK 1024
 // Scatterers one launch of the tensor-core history kernel serves at most.
 #define MOT_TC_MAX_JOBS 32
-// Preconditioned Krylov vectors M V_j kept by a GMRES solve.
+// Preconditioned Krylov vectors M V_j kept by a GMRES solve. The preconditioned solves
+// take one to three iterations and their corrections as many; twelve block vectors are
+// an eighth of what the basis V takes, and a longer solve costs one more product with M.
 #define MOT_GM_ZCAP 12
 // Bytes of point currents the far field keeps at most (at least one frequency's):
 // more frequencies than that go in turn. 64 MB is half of L2 and 31 frequencies of
