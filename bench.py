@@ -510,7 +510,7 @@ def run_ours(args):
         peak_rel = np.linalg.norm(wm - wf, axis=(1, 2)) / np.maximum(A["peak"], 1e-300)
         fp64 = {"value": throughput(world, B, n64, f_ms), "unit": "RHS·steps/s", "steps": n64,
                 "ms_per_step": f_ms / n64, "dtype": "f64",
-                "solver": "right-preconditioned GMRES, Q_0 in FP64 product form, M = FP64 dense Q_0^-1",
+                "solver": "right-preconditioned GMRES, dense FP64 Q_0, M = FP64 dense Q_0^-1",
                 "gmres_iters_per_step": (fi1["gmres_iters_total"] - fi0["gmres_iters_total"]) / n64,
                 "e2e": {"value": throughput(world, B, n64, f_e2e), "unit": "RHS·steps/s",
                         "h2d_bytes_per_step": 80 * B, "d2h_bytes_per_step": 8 * 2 * ops.ne * B},

@@ -90,9 +90,10 @@ typedef struct {
                               (stops early once |r| <= gmres_tol |b|); default 1 */
     int32_t fp64_precond;  /* MOT_PREC_FP64 only. 0 (default): GMRES on Q_0, unpreconditioned;
                               Q_0 is assembled densely at load from its product form on unit
-                              columns ((2 npad)^2 doubles of device memory) or, where that is
-                              not possible (no memory, a projector solve at its limit),
-                              applied in product form. 1: right-preconditioned GMRES,
+                              columns ((2 npad)^2 doubles of device memory) where twice that
+                              is free, else (or where a projector solve runs into its limit)
+                              applied in product form; it is given back if the march state
+                              finds no memory beside it. 1: right-preconditioned GMRES,
                               Q_0 M z = b, x = M z, with M = Q_0^{-1} formed at load in FP64
                               (LU with partial pivoting); every product stays FP64, so the
                               result matches the unpreconditioned solve to the GMRES tolerance
@@ -109,7 +110,7 @@ typedef struct {
                               left factor) and the projectors' graph-Laplacian solves by FP64
                               refinement with FP32 dense inverses formed at load, to cg_tol
                               (plain CG where the inverses do not serve, e.g. a surface of
-                              several components). 1: by dense FP64 inverses formed at load (LU
+                              several components, or have no memory). 1: by dense FP64 inverses formed at load (LU
                               with partial pivoting; the Laplacians as (L + 11^T/N)^{-1}, their
                               pseudo-inverse on the mean-free right-hand sides), exact to
                               rounding; costs npad^2 + nf^2 + nv^2 doubles of device memory. */
@@ -215,7 +216,8 @@ typedef struct {
     /* GMRES iterations of the Q_0 solves summed over every step since the
        march (re)started (the refinement's correction solves excluded) */
     int64_t gmres_iters_total;
-    /* tensor-core history: the configuration in use -- tasks per chunk, the
+    /* tensor-core history: the configuration in use -- tasks per chunk (the
+       limit: launches of few tasks are cut smaller, see mot_tune), the
        fraction of the L2 one lag range of the task list may fill, pipeline
        stages (0: the deepest that fits) -- whether mot_tune (or mot_run_many)
        chose it, and its launch time in that tuning (ms) */
