@@ -572,15 +572,16 @@ __global__ void __launch_bounds__(128) k_point_currents(int npts, int npad, int 
 // sums of the point currents times e^{j k r.x}. Bound by the FP64 units where
 // there is work for all of them: 24 multiply-adds per point, direction, wave and
 // frequency, and one sine and cosine per point, direction and frequency, shared
-// by the waves (and by the three edges of a point's triangle). A cluster of eight
-// CTAs takes DT directions and BT waves of one frequency (grid: direction tiles,
+// by the waves (and by the three edges of a point's triangle). A cluster of up to
+// eight CTAs takes DT directions and BT waves of one frequency (grid: direction tiles,
 // wave tiles, frequencies); its threads are (share of the points, direction,
 // wave), the shares are summed in shared memory and then over the cluster, in
-// order. BT and DT are chosen at the launch. A mot_fields call at 480 edges: 8
-// waves, 3 frequencies, 181 directions 697 us, one wave and direction at 100
-// frequencies 162 us; with a launch per frequency over all waves 984 and 7254 us;
+// order. BT, DT and the cluster are chosen at the launch. A mot_fields call at 480
+// edges: 8 waves, 3 frequencies, 181 directions 697 us, one wave and direction at
+// 100 frequencies 135 us; with a launch per frequency over all waves 984 and 7254 us;
 // with a CTA per output over its edges, no points or phases shared, 2750 and 157 us.
-constexpr int FT = 256, FCL = 8;
+constexpr int FT = 256, FCL = 8;  // threads a CTA, most CTAs a cluster
+template <int CL>
 __global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, int f0, int ndir, int DT, int BT,
                                                   const double* __restrict__ pts, const double* __restrict__ cur,
                                                   const double* __restrict__ omega, const double* __restrict__ dirs,
@@ -592,7 +593,7 @@ __global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, in
     const int rk = (int)cl.block_rank(), t = threadIdx.x, f = f0 + blockIdx.z;
     const int G = DT * BT, nsub = FT / G, sub = t / G, l = t - sub * G, d = l / BT, q = l - d * BT;
     const bool on = sub < nsub;
-    const int dir = blockIdx.x / FCL * DT + d, b = blockIdx.y * BT + q;
+    const int dir = blockIdx.x / CL * DT + d, b = blockIdx.y * BT + q;
     const bool wave = b < B;
     const double w = omega[f], k = w / c;
     cur += (size_t)blockIdx.z * npts * 12 * B;
@@ -603,7 +604,7 @@ __global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, in
 #pragma unroll
     for (int j = 0; j < 12; j++) acc[j] = 0.0;
     // a share takes BT consecutive points at a time: thread (d, q) the phase of point q
-    const int step = FCL * nsub * BT;
+    const int step = CL * nsub * BT;
     for (int p0 = 0; p0 < npts; p0 += step) {
         const int first = p0 + (rk * nsub + sub) * BT, n = on ? max(0, min(BT, npts - first)) : 0;
         if (q < n) {
@@ -637,12 +638,12 @@ __global__ void __launch_bounds__(FT) k_far_field(int npts, int B, int nfreq, in
         m = half;
     }
     cl.sync();
-    if (t < G && t % FCL == rk && dir < ndir && wave) {
+    if (t < G && t % CL == rk && dir < ndir && wave) {
         double v[12];
 #pragma unroll
         for (int j = 0; j < 12; j++) {
             v[j] = 0.0;
-            for (int u = 0; u < FCL; u++) v[j] += cl.map_shared_rank(sums, u)[j * FT + t];
+            for (int u = 0; u < CL; u++) v[j] += cl.map_shared_rank(sums, u)[j * FT + t];
         }
         double out[6];
         for (int part = 0; part < 2; part++) {  // real, imag
@@ -879,22 +880,26 @@ void launch_far_field(mot_handle* h, int n_dir, const double* dirs, double* E, c
         int BT = h->B, DT = 1;
         while (BT > 8 && ctas(BT, 1) < 2 * nsm) BT = (BT + 1) / 2;
         while (2 * DT <= std::min(8, n_dir) && DT * BT < 32 && ctas(BT, 2 * DT) >= 2 * nsm) DT *= 2;
+        // Shares of a few points are mostly reduction: fewer CTAs a cluster, if the chip stays
+        // covered (one wave and direction, 100 frequencies, 480 edges: a call 135 us, with eight 162)
+        int CL = FCL;
+        while (CL > 2 && h->npts < 4 * CL * (FT / (DT * BT)) && ctas(BT, DT) / FCL * (CL / 2) >= 2 * nsm) CL /= 2;
         k_point_currents<<<dim3((h->npts * h->B + 127) / 128, nf), 128, 0, s>>>(
             h->npts, h->npad, h->B, h->nq, h->d_ptptr, h->d_ptent, h->d_rhs_wf, h->d_dft + (size_t)f0 * 4 * nb * 2,
             h->d_ptcur);
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((n_dir + DT - 1) / DT * FCL, (h->B + BT - 1) / BT, nf);
+        cfg.gridDim = dim3((n_dir + DT - 1) / DT * CL, (h->B + BT - 1) / BT, nf);
         cfg.blockDim = dim3(FT);
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = FCL;
+        at[0].val.clusterDim.x = CL;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_far_field, h->npts, h->B, h->nfreq, f0, n_dir, DT, BT, (const double*)h->d_pts,
-                           (const double*)h->d_ptcur, (const double*)h->d_omega, dirs, (const double*)h->d_waves, h->c,
-                           h->eta, E);
+        cudaLaunchKernelEx(&cfg, CL == 8 ? k_far_field<8> : CL == 4 ? k_far_field<4> : k_far_field<2>, h->npts, h->B,
+                           h->nfreq, f0, n_dir, DT, BT, (const double*)h->d_pts, (const double*)h->d_ptcur,
+                           (const double*)h->d_omega, dirs, (const double*)h->d_waves, h->c, h->eta, E);
         h->launches += 2;
     }
 }

@@ -38,7 +38,7 @@ def test_refused_list(M, ops, bad):
     assert np.array_equal(*E) and np.abs(E[0]).max() > 0
 
 
-@pytest.mark.parametrize("B,n_dir,F", [(1, 1, 40), (64, 1, 20), (64, 1, 1), (10, 2, 3), (5, 33, 1), (64, 9, 17)])
+@pytest.mark.parametrize("B,n_dir,F", [(1, 1, 40), (1, 1, 90), (1, 1, 160), (3, 2, 80), (64, 1, 20), (64, 1, 1), (10, 2, 3), (5, 33, 1), (64, 9, 17)])
 def test_far_field_of_many_frequencies(M, ops, B, n_dir, F):
     """Shapes that the far field cuts differently: more frequencies than its point
     currents hold (17 at this size and 64 waves), waves over several clusters, ragged
